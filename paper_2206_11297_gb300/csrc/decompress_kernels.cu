@@ -232,77 +232,6 @@ __global__ void __launch_bounds__(256) k_dec_parse(DevParams p, Scratch s, DecAr
   }
 }
 
-// decode: one thread per chunk (block = 64 chunks of one frame).
-constexpr int kDecThreads = 64;
-// Other blocks of the frame may mark it corrupt while this one starts, so the
-// go/no-go decision is read once and shared before any barrier.
-__global__ void __launch_bounds__(kDecThreads) k_dec_decode(DevParams p, Scratch s, DecArgs a) {
-  __shared__ uint32_t tab[kDecCanonWords];
-  __shared__ int go;
-  const uint32_t f = blockIdx.y;
-  if (threadIdx.x == 0) go = s.status[f] == ROIBIN_OK;
-  __syncthreads();
-  if (!go) return;
-  for (uint32_t i = threadIdx.x; i < kDecCanonWords; i += kDecThreads)
-    tab[i] = s.dec_table[(size_t)f * kDecTableWords + i];
-  __syncthreads();
-  const uint32_t k = blockIdx.x * kDecThreads + threadIdx.x;
-  if (k >= p.n_chunks) return;
-  const DecInfo di = s.dec_info[f];
-  const uint8_t* base = a.in + di.base;
-  const uint32_t* cidx = reinterpret_cast<const uint32_t*>(base + di.pl.off_cidx);
-  const uint32_t* words = reinterpret_cast<const uint32_t*>(base + di.pl.off_bits);
-  const uint32_t w0 = cidx[k];
-  const uint32_t w1 = k + 1 < p.n_chunks ? cidx[k + 1] : di.pl.n_words;
-  if (w0 > w1 || w1 > di.pl.n_words) {
-    mark_corrupt(s, f);
-    return;
-  }
-  const uint64_t bit_end = (uint64_t)(w1 - w0) * 32;
-  uint64_t bit = 0;
-  const uint32_t s0 = k * kChunk, s1 = min(p.M, s0 + kChunk);
-  int32_t* dq = s.dq + (size_t)f * p.M;
-  uint32_t zeros = 0;
-  // bit reader: `cur` holds the next up-to-32 bits, MSB first
-  uint32_t wi = w0;
-  uint64_t buf = 0;
-  int nbuf = 0;
-  for (uint32_t i = s0; i < s1; ++i) {
-    if (nbuf < 32) {
-      const uint32_t w = wi < w1 ? words[wi] : 0u;
-      ++wi;
-      buf |= (uint64_t)w << (32 - nbuf);
-      nbuf += 32;
-    }
-    // canonical decode: extend the code one bit at a time
-    uint32_t code = 0;
-    int sym = -1;
-    for (uint32_t L = 1; L <= 32; ++L) {
-      code = (code << 1) | (uint32_t)(buf >> (63 - (L - 1)) & 1u);
-      const uint32_t n = tab[L];
-      if (n && code - tab[34 + L] < n && code >= tab[34 + L]) {
-        sym = (int)tab[102 + tab[68 + L] + (code - tab[34 + L])];
-        buf <<= L;
-        nbuf -= (int)L;
-        bit += L;
-        break;
-      }
-    }
-    if (sym < 0 || bit > bit_end) {
-      mark_corrupt(s, f);
-      return;
-    }
-    if (sym == 0) {
-      dq[i] = kSentinel;
-      ++zeros;
-    } else {
-      dq[i] = sym - di.R;
-    }
-  }
-  if ((bit + 31) / 32 != (uint64_t)(w1 - w0)) mark_corrupt(s, f);
-  if (zeros) atomicAdd(s.dec_zero + f, zeros);
-}
-
 // lorenzo: scatter the Lorenzo-outlier deltas (must land on code-0 bins, in
 // strictly ascending order).
 __global__ void k_dec_lorenzo(DevParams p, Scratch s, DecArgs a) {
@@ -490,72 +419,64 @@ __global__ void k_dec_roi(DevParams p, Scratch s, DecArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// The panel path.
+// The decoders of both paths: several lanes per 4,096-symbol chunk.
 //
-// The panel path's decoders: one thread per chunk, up to kDecMaxThreads chunks
-// of one frame per block, like k_dec_decode, with two shortcuts.
+// A Huffman code resynchronises: a decoder started inside a codeword meets the
+// true codeword boundaries again after a few codewords.  So the chunk's bits
+// are cut into equal ranges, one per lane.  Every lane decodes its range from
+// the range's first bit, counting codewords, and says where the first codeword
+// past its range starts.  A lane whose left neighbour says another start than
+// the one it used decodes again from there, until no start changes (lane 0's is
+// right from the outset, so at most 31 times; once on detector frames).  Then
+// the starts are the serial decoder's own, an exclusive scan of the counts gives
+// every lane the index of its first symbol, and a last pass decodes and stores.
+// Bits of the zero padding may decode as symbols past the chunk's last one; they
+// are not stored.
+//
+// A thread per chunk (4,096 dependent lookups) kept too few lanes busy: a
+// 60-frame epix10k batch has 7,920 chunks.  What bounds these is the chain of
+// window, lookup and advance per lane, three times over.  us, a thread per
+// chunk -> now: 60 epix10k frames (2.9 bits a symbol, dense) 1,460 -> 187; one
+// CSPAD-like frame (1.02 bits, sparse) 54 -> 9.5, 400 of them 90 -> 62; 40 of
+// them as residuals for the multi-pass path 943 -> 66.
+//
+// Two shortcuts, as the code allows:
 //   - When a code of length 1 exists it is the all-zero code, so a run of z zero
 //     bits is z copies of its symbol, taken in one step (count of leading zeros).
-//   - Other codes: the next 12 bits index the prefix table (codes of up to 12
-//     bits resolve in one lookup; longer ones continue bit by bit from length 13).
-// A frame the parse step marked sparse (a length-1 code, and each chunk's bit
-// count leaves room for at most kDecSparseMax other symbols) takes
-// k_dec_decode_sparse, which lists only each chunk's other symbols (dec_list):
-// the panel kernel fills the rest with the length-1 code's symbol, so the
-// frame's symbols never go through device memory.  Other frames take
-// k_dec_decode_dense, which writes every symbol to the [n][n_chunks * kChunk]
-// u16 symbol array: it stages kDecRound symbols per thread in shared memory and
-// has the warp store its 32 slots together, instead of each thread storing into
-// its own cache lines.  Corrupt-stream checks are those of k_dec_decode.
-constexpr uint32_t kDecRound = 32;                     // symbols per thread and round (dense)
-constexpr uint32_t kDecSlotWords = kDecRound / 2 + 4;  // 64 bytes + 16 bytes of bank skew
-constexpr uint32_t kDecMaxThreads = 256;
+//   - Other codes: the next 12 bits index a table (several codewords at once in
+//     the dense decoder; codes of more than 12 bits are found by their length).
+//
+// What is stored:
+//   k_dec_dense<true> (the multi-pass path): every symbol's residual, as int32, at
+//   its bin;
+//   k_dec_sparse: a frame the parse step marked sparse (a length-1 code, and each chunk's
+//   bit count leaves room for at most kDecSparseMax other symbols) stores only
+//   each chunk's other symbols (dec_list): the panel kernel fills the rest, so the
+//   frame's symbols never go through device memory;
+//   k_dec_dense<false>: every symbol of the other frames, in the
+//   [n][n_chunks * kChunk] u16 symbol array.
+// Dense symbols are collected in shared memory (the lanes' runs start 128
+// symbols apart, so a word of padding per 32 keeps them off one bank) and leave
+// in whole lines.
+constexpr uint32_t kDecWarps = 8;              // warps per block
+constexpr uint32_t kDecStageWords = 704;       // a chunk's words in shared memory (longer chunks: through L1)
+constexpr uint32_t kDecSymWords = kChunk / 2 + kChunk / 64;  // its symbols, padded
+constexpr uint32_t kDecWarpWords = kDecStageWords + 8 + kDecSymWords;
+constexpr uint32_t kDecLutSize = 1u << kDecLutBits;
+// the canonical tables, the pair table, the count table, the warps' words and symbols: 2 blocks per SM
+constexpr uint32_t kDecPairAt = kDecCanonWords, kDecCountAt = kDecPairAt + kDecLutSize,
+                   kDecLongAt = kDecCountAt + kDecLutSize / 4, kDecWarpAt = kDecLongAt + 40;
+constexpr uint32_t kDecSmem = (kDecWarpAt + kDecWarps * kDecWarpWords) * 4;
+static_assert(2 * (kDecSmem + 1024) <= 228 * 1024, "two dense decoder blocks share an SM");
+static_assert(kDecWarps * kDecWarpWords >= kDecLutWords, "the prefix table is read from the warps' area");
 
-// Reads a chunk's words [w0, w1) in aligned 16-byte groups, one group ahead of
-// the one being consumed; words at or past w1 read as 0.  The bitstream section
-// starts 16-byte aligned and is padded to 16 bytes, so every group read lies
-// inside it.
-struct WordReader {
-  const uint4* g4;
-  uint32_t gi, ci, w1;
-  uint4 cur, nxt;
-  __device__ __forceinline__ uint4 group(uint32_t g) const {
-    return 4 * g < w1 ? g4[g] : make_uint4(0u, 0u, 0u, 0u);
-  }
-  __device__ __forceinline__ void init(const uint32_t* words, uint32_t w0, uint32_t w1_) {
-    g4 = reinterpret_cast<const uint4*>(words);
-    w1 = w1_;
-    gi = w0 >> 2;
-    ci = w0 & 3u;
-    cur = group(gi);
-    nxt = group(gi + 1);
-  }
-  __device__ __forceinline__ uint32_t next() {
-    uint32_t w = ci == 0 ? cur.x : ci == 1 ? cur.y : ci == 2 ? cur.z : cur.w;
-    if (4 * gi + ci >= w1) w = 0;
-    if (++ci == 4) {
-      ci = 0;
-      ++gi;
-      cur = nxt;
-      nxt = group(gi + 1);
-    }
-    return w;
-  }
-};
-
-// One code from the top of `buf` (at least 32 valid bits): its length, 0 when
-// no code of up to 32 bits matches; the symbol in `sym`.
-__device__ __forceinline__ uint32_t decode_one(const uint32_t* tab, const uint16_t* lut, uint64_t buf,
-                                               uint32_t& sym) {
-  const uint32_t ent = lut[(uint32_t)(buf >> (64 - kDecLutBits))];
-  sym = ent & 1023u;
-  if (ent >> 10) return ent >> 10;
-  uint32_t code = (uint32_t)(buf >> (64 - kDecLutBits));
+// A code of more than kDecLutBits bits from the top of `win` (the next 32 bits):
+// its length, 0 when no code matches; the symbol in `sym`.
+__device__ __noinline__ uint32_t decode_long(const uint32_t* tab, uint32_t win, uint32_t& sym) {
   for (uint32_t L = kDecLutBits + 1; L <= 32; ++L) {
-    code = (code << 1) | (uint32_t)(buf >> (63 - (L - 1)) & 1u);
-    const uint32_t n = tab[L];
-    if (n && code >= tab[34 + L] && code - tab[34 + L] < n) {
-      sym = tab[102 + tab[68 + L] + (code - tab[34 + L])];
+    const uint32_t n = tab[L], d = (win >> (32 - L)) - tab[34 + L];
+    if (d < n) {  // a code below the first of its length wraps far above n
+      sym = tab[102 + tab[68 + L] + d];
       return L;
     }
   }
@@ -575,220 +496,337 @@ __device__ __forceinline__ uint32_t* dec_list_count(const Scratch& s, const DevP
 }
 static_assert(kDecSparseMax * 4 <= kChunk * 2, "a chunk's list fits its slot of the symbol array");
 
-// The frame's decoding tables into shared memory; false when the frame is not
-// this kernel's (or not OK).  Read once by thread 0 and shared, since other
-// blocks of the frame may mark it corrupt meanwhile.
-__device__ __forceinline__ bool dec_load_tables(const Scratch& s, uint32_t f, bool want_sparse, uint32_t* tab,
-                                                int* go) {
-  if (threadIdx.x == 0) *go = s.status[f] == ROIBIN_OK && (s.dec_info[f].sparse != 0) == want_sparse;
+// Decodes the codewords of a chunk that start in bits [at, limit), at most
+// `room` of them; `word(i)` is the chunk's word i (0 past its end).  `other(i,
+// sym)` is called for the i-th codeword of the range unless it belongs to a run
+// of the length-1 code; sym is 0xFFFFFFFF where no code matches (one bit is
+// skipped then).  Returns the codewords decoded; `at` becomes the bit after them.
+// The window is fetched anew for every codeword (two words, one funnel shift):
+// fewer instructions than a bit buffer with its refills.
+template <class Word, class Other>
+__device__ __forceinline__ uint32_t decode_range(const uint32_t* tab, const uint16_t* lut, uint32_t& at, uint32_t limit,
+                                                 uint32_t room, Word word, Other other) {
+  uint32_t pos = at, n = 0;
+  while (pos < limit && n < room) {
+    const uint32_t win = __funnelshift_l(word((pos >> 5) + 1), word(pos >> 5), pos & 31u);
+    if ((int32_t)win >= 0) {  // a run of the length-1 code
+      const uint32_t z = min((uint32_t)__clz(win), min(limit - pos, room - n));
+      n += z;
+      pos += z;
+    } else {
+      const uint32_t ent = lut[win >> (32 - kDecLutBits)];
+      uint32_t sym = ent & 1023u, L = ent >> 10;
+      if (L == 0) L = decode_long(tab, win, sym);
+      if (L == 0) {
+        L = 1;
+        sym = 0xFFFFFFFFu;
+      }
+      other(n, sym);
+      ++n;
+      pos += L;
+    }
+  }
+  at = pos;
+  return n;
+}
+
+// The lanes' starts and counts of one chunk of nw words, decoded by a group of G
+// lanes (lane g of it covers the g-th of G equal ranges of bits).  Every lane of
+// the warp calls it.  `n`: codewords of the lane's range; `listed`: those not in
+// runs; `start`: the bit its first codeword starts at.
+template <class Decode>
+__device__ __forceinline__ void sync_ranges(uint32_t G, uint32_t g, uint32_t first_bit, uint32_t limit, uint32_t& start,
+                                            uint32_t& n, uint32_t& listed, Decode decode) {
+  start = first_bit;
+  uint32_t end = start;
+  listed = 0;
+  n = decode(end, limit, 0xFFFFFFFFu, [&](uint32_t, uint32_t) { ++listed; });
+  for (uint32_t round = 0; round < 32; ++round) {
+    const uint32_t left = __shfl_up_sync(0xffffffffu, end, 1, G);
+    const bool again = g > 0 && left != start;
+    if (!__any_sync(0xffffffffu, again)) break;
+    if (again) {
+      start = end = left;
+      listed = 0;
+      n = decode(end, limit, 0xFFFFFFFFu, [&](uint32_t, uint32_t) { ++listed; });
+    }
+  }
+}
+
+// Loads the frame's decoding tables; false when the frame is not sparse (or not OK).  Other blocks of the frame may mark it corrupt meanwhile, so the
+// decision is read once and shared.
+__device__ __forceinline__ bool dec_load_tables(const Scratch& s, uint32_t f, uint32_t* tab, int* go) {
+  if (threadIdx.x == 0) *go = s.status[f] == ROIBIN_OK && s.dec_info[f].sparse != 0;
   __syncthreads();
   if (!*go) return false;
   const uint4* src = reinterpret_cast<const uint4*>(s.dec_table + (size_t)f * kDecTableWords);
-  uint4* dst = reinterpret_cast<uint4*>(tab);
   static_assert(kDecTableWords % 4 == 0, "table copied in 16-byte pieces");
-  for (uint32_t i = threadIdx.x; i < kDecTableWords / 4; i += blockDim.x) dst[i] = src[i];
+  for (uint32_t i = threadIdx.x; i < kDecTableWords / 4; i += blockDim.x) reinterpret_cast<uint4*>(tab)[i] = src[i];
   __syncthreads();
   return true;
 }
 
-__global__ void __launch_bounds__(kDecMaxThreads) k_dec_decode_sparse(DevParams p, Scratch s, DecArgs a) {
+// Sparse frames: G = 2^lg lanes per chunk, words read through L1.
+__global__ void __launch_bounds__(kDecWarps * 32) k_dec_sparse(DevParams p, Scratch s, DecArgs a, uint32_t lg) {
   __shared__ __align__(16) uint32_t tab[kDecTableWords];
   __shared__ int go;
-  const uint32_t f = blockIdx.y;
-  if (!dec_load_tables(s, f, true, tab, &go)) return;
+  const uint32_t f = blockIdx.y, G = 1u << lg;
+  if (!dec_load_tables(s, f, tab, &go)) return;
   const uint16_t* lut = reinterpret_cast<const uint16_t*>(tab + kDecCanonWords);
-  // the length-1 code is code 0: its symbol comes first in the (length, symbol) order
-  const uint32_t zsym = tab[102];
-  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= p.n_chunks) return;
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, k = t >> lg, g = t & (G - 1);
+  if (((t & ~31u) >> lg) >= p.n_chunks) return;  // the whole warp
   const DecInfo& di = s.dec_info[f];
   const uint8_t* base = a.in + di.base;
   const uint32_t n_words = di.pl.n_words;
   const uint32_t* cidx = reinterpret_cast<const uint32_t*>(base + di.pl.off_cidx);
-  const uint32_t* words = reinterpret_cast<const uint32_t*>(base + di.pl.off_bits);
-  const uint32_t w0 = cidx[k];
-  const uint32_t w1 = k + 1 < p.n_chunks ? cidx[k + 1] : n_words;
-  uint32_t* count = dec_list_count(s, p, f) + k;
-  if (w0 > w1 || w1 > n_words) {
-    *count = 0;
-    mark_corrupt(s, f);
-    return;
-  }
-  const uint64_t bit_end = (uint64_t)(w1 - w0) * 32;
-  const uint32_t n_sym = min(p.M, k * kChunk + kChunk) - k * kChunk;
-  uint32_t* list = dec_list(s, p, f, k);
-  WordReader rd;
-  rd.init(words, w0, w1);
-  uint64_t buf = 0;  // next bits, MSB first; nbuf of them are valid
-  uint32_t nbuf = 0, pos = 0, zeros = 0, n_list = 0;
-  uint64_t bit = 0;
-  bool bad = false;
-  while (pos < n_sym) {
-    if (nbuf < 32) {
-      buf |= (uint64_t)rd.next() << (32 - nbuf);
-      nbuf += 32;
-    }
-    if ((buf >> 63) == 0) {
-      const uint32_t z = min(min((uint32_t)__clzll(buf), nbuf), n_sym - pos);
-      pos += z;
-      buf <<= z;
-      nbuf -= z;
-      bit += z;
-      if (zsym == 0) zeros += z;
-    } else {
-      uint32_t sym;
-      const uint32_t L = decode_one(tab, lut, buf, sym);
-      if (L == 0 || n_list == kDecSparseMax) {
-        bad = true;
-        break;
-      }
-      list[n_list++] = (pos << 16) | sym;
-      ++pos;
-      buf <<= L;
-      nbuf -= L;
-      bit += L;
-      zeros += sym == 0;
-    }
-    if (bit > bit_end) {
-      bad = true;
-      break;
-    }
-  }
-  *count = bad ? 0u : n_list;
-  if (bad || (bit + 31) / 32 != (uint64_t)(w1 - w0)) mark_corrupt(s, f);
-  if (zeros) atomicAdd(s.dec_zero + f, zeros);
-}
-
-struct SymbolWriter {  // eight u16 symbols per 16-byte shared-memory store
-  uint16_t* slot;      // this thread's slot (16-byte aligned)
-  uint32_t pos = 0;    // symbols emitted in the chunk
-  uint64_t lo = 0, hi = 0;
-  __device__ __forceinline__ void flush() {
-    *reinterpret_cast<uint4*>(slot + ((pos - 8) & (kDecRound - 1))) =
-        make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
-    lo = hi = 0;
-  }
-  __device__ __forceinline__ void put(uint32_t sym) {
-    const uint32_t k = pos & 7u;
-    if (k < 4) lo |= (uint64_t)sym << (16 * k);
-    else hi |= (uint64_t)sym << (16 * (k - 4));
-    ++pos;
-    if ((pos & 7u) == 0) flush();
-  }
-  __device__ __forceinline__ void run(uint32_t sym, uint32_t z) {
-    while (z && (pos & 7u)) {
-      put(sym);
-      --z;
-    }
-    const uint64_t rep = (uint64_t)sym * 0x0001000100010001ull;
-    for (; z >= 8; z -= 8) {
-      pos += 8;
-      lo = hi = rep;
-      flush();
-    }
-    while (z) {
-      put(sym);
-      --z;
-    }
-  }
-  __device__ __forceinline__ void finish() {  // the chunk's last partial group
-    const uint32_t k = pos & 7u, b = (pos - k) & (kDecRound - 1);
-#pragma unroll
-    for (uint32_t h = 0; h < 7; ++h)
-      if (h < k) slot[b + h] = (uint16_t)((h < 4 ? lo >> (16 * h) : hi >> (16 * (h - 4))) & 0xFFFFu);
-  }
-};
-
-__global__ void __launch_bounds__(kDecMaxThreads) k_dec_decode_dense(DevParams p, Scratch s, DecArgs a) {
-  __shared__ __align__(16) uint32_t tab[kDecTableWords];
-  __shared__ __align__(16) uint32_t slots[kDecMaxThreads * kDecSlotWords];
-  __shared__ int go;
-  const uint32_t f = blockIdx.y;
-  if (!dec_load_tables(s, f, false, tab, &go)) return;
-  const uint16_t* lut = reinterpret_cast<const uint16_t*>(tab + kDecCanonWords);
-  const uint32_t lane = lane_id();
-  const uint32_t warp0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u);  // chunk of lane 0
-  if (warp0 >= p.n_chunks) return;  // whole warp past the last chunk
-  const uint32_t k = warp0 + lane;
   const bool live = k < p.n_chunks;
-  const DecInfo& di = s.dec_info[f];
-  const uint8_t* base = a.in + di.base;
-  const uint32_t n_words = di.pl.n_words;
-  const uint32_t* cidx = reinterpret_cast<const uint32_t*>(base + di.pl.off_cidx);
-  const uint32_t* words = reinterpret_cast<const uint32_t*>(base + di.pl.off_bits);
-  uint32_t w0 = 0, w1 = 0, n_sym = 0;
+  uint32_t w0 = 0, nw = 0, n_sym = 0;
   bool bad = false;
   if (live) {
     w0 = cidx[k];
-    w1 = k + 1 < p.n_chunks ? cidx[k + 1] : n_words;
+    const uint32_t w1 = k + 1 < p.n_chunks ? cidx[k + 1] : n_words;
     n_sym = min(p.M, k * kChunk + kChunk) - k * kChunk;
-    if (w0 > w1 || w1 > n_words) bad = true;
+    // a chunk of n symbols takes at most n words
+    bad = w0 > w1 || w1 > n_words || w1 - w0 > kChunk;
+    nw = bad ? 0u : w1 - w0;
   }
-  const uint64_t bit_end = (uint64_t)(w1 - w0) * 32;
-  // the length-1 code, when there is one, is code 0: its symbol comes first
-  // in the (length, symbol) order
-  const bool zrun = tab[1] != 0;
-  const uint32_t zsym = tab[102];
-  uint32_t* warp_slots = slots + (threadIdx.x & ~31u) * kDecSlotWords;
-  SymbolWriter wr;
-  wr.slot = reinterpret_cast<uint16_t*>(warp_slots + lane * kDecSlotWords);
-  uint16_t* out = s.codes + (size_t)f * p.n_chunks * kChunk;
-  const uint32_t n_warp = min(32u, p.n_chunks - warp0);  // live lanes
-  WordReader rd;  // a lane with a bad chunk index reads nothing
-  rd.init(words, w0, live && !bad ? w1 : 0u);
-  uint64_t bit = 0;
-  uint32_t zeros = 0;
-  uint64_t buf = 0;  // next bits, MSB first; nbuf of them are valid
-  uint32_t nbuf = 0;
-  for (uint32_t r0 = 0; r0 < kChunk; r0 += kDecRound) {
-    const uint32_t target = min(n_sym, r0 + kDecRound);
-    while (!bad && wr.pos < target) {
-      if (nbuf < 32) {
-        buf |= (uint64_t)rd.next() << (32 - nbuf);
-        nbuf += 32;
-      }
-      if (zrun && (buf >> 63) == 0) {
-        const uint32_t z = min(min((uint32_t)__clzll(buf), nbuf), target - wr.pos);
-        wr.run(zsym, z);
-        buf <<= z;
-        nbuf -= z;
-        bit += z;
-        if (zsym == 0) zeros += z;
-      } else {
-        uint32_t sym;
-        const uint32_t L = decode_one(tab, lut, buf, sym);
-        if (L == 0) {
-          bad = true;
-          break;
-        }
-        wr.put(sym);
-        buf <<= L;
-        nbuf -= L;
-        bit += L;
-        zeros += sym == 0;
-      }
-      if (bit > bit_end) bad = true;
+  const uint32_t* words = reinterpret_cast<const uint32_t*>(base + di.pl.off_bits) + w0;
+  const uint32_t zsym = tab[102];  // the length-1 code is code 0: first in the (length, symbol) order
+  auto decode = [&](uint32_t& at, uint32_t limit, uint32_t room, auto other) {
+    return decode_range(tab, lut, at, limit, room, [&](uint32_t i) { return i < nw ? __ldg(words + i) : 0u; }, other);
+  };
+  const uint32_t share = nw << (5 - lg), limit = (g + 1) * share;
+  uint32_t start, n, listed;
+  sync_ranges(G, g, g * share, limit, start, n, listed, decode);
+  uint32_t first = n, at_list = listed;  // exclusive scans in the group
+  for (uint32_t d = 1; d < G; d <<= 1) {
+    const uint32_t x = __shfl_up_sync(0xffffffffu, first, d, G), y = __shfl_up_sync(0xffffffffu, at_list, d, G);
+    if (g >= d) {
+      first += x;
+      at_list += y;
     }
-    if (!bad && wr.pos == n_sym && (n_sym & 7u)) wr.finish();
-    __syncwarp();
-    // the warp writes the round out: lanes 0-15 one slot, lanes 16-31 the next
-    for (uint32_t b0 = 0; b0 < n_warp; b0 += 2) {
-      const uint32_t b = b0 + (lane >> 4), w = lane & 15u;
-      if (b < n_warp) {
-        const uint32_t kb = warp0 + b;
-        const uint32_t cnt = min(p.M, kb * kChunk + kChunk) - kb * kChunk;  // symbols of chunk kb
-        const uint32_t i = r0 + 2 * w;                                       // first symbol of the word
-        const uint32_t v = warp_slots[b * kDecSlotWords + w];
-        uint16_t* dst = out + (size_t)kb * kChunk + i;
-        if (i + 1 < cnt) *reinterpret_cast<uint32_t*>(dst) = v;
-        else if (i < cnt) *dst = (uint16_t)v;
-      }
-    }
-    __syncwarp();
   }
-  if (live) {
-    if (bad || (bit + 31) / 32 != (uint64_t)(w1 - w0)) mark_corrupt(s, f);
+  if (g == G - 1 && first < n_sym) bad = true;  // the chunk's bits end too early
+  first -= n;
+  at_list -= listed;
+  uint32_t zeros = 0, wrote = 0;
+  if (live && !bad && first < n_sym && n > 0) {
+    uint32_t* list = dec_list(s, p, f, k);
+    const uint32_t room = min(n, n_sym - first);
+    uint32_t bit = start;
+    decode(bit, limit, room, [&](uint32_t i, uint32_t sym) {
+      if (sym > 0xFFFFu || at_list + wrote >= kDecSparseMax) bad = true;
+      else list[at_list + wrote] = ((first + i) << 16) | sym;
+      ++wrote;
+      zeros += sym == 0;
+    });
+    if (zsym == 0) zeros += room - wrote;
+    // the chunk's last symbol: its words must end with it
+    if (first + room == n_sym && (bit + 31) / 32 != nw) bad = true;
+  }
+  uint32_t any_bad = bad;
+  for (uint32_t d = 1; d < G; d <<= 1) {
+    zeros += __shfl_xor_sync(0xffffffffu, zeros, d);
+    wrote += __shfl_xor_sync(0xffffffffu, wrote, d);
+    any_bad |= __shfl_xor_sync(0xffffffffu, any_bad, d);
+  }
+  if (live && g == 0) {
+    dec_list_count(s, p, f)[k] = any_bad ? 0u : wrote;
+    if (any_bad) mark_corrupt(s, f);
     if (zeros) atomicAdd(s.dec_zero + f, zeros);
+  }
+}
+
+// The dense decoder's tables in shared memory, from the frame's prefix table:
+//   pair[x], x the next 12 bits: bits 0-9 the first symbol, 20-23 its length (0:
+//     longer than 12 bits); bits 10-19 the second, 24-27 the length of both (0:
+//     the second does not end inside the 12 bits);
+//   count[x]: bits 0-3 the codewords that end inside the 12 bits, 4-7 their length.
+// The counting passes then take about four codewords of an epix10k frame per
+// lookup and the storing pass two.
+__device__ __forceinline__ void build_dense_tables(const uint32_t* frame_tab, uint32_t* sm) {
+  uint16_t* lut = reinterpret_cast<uint16_t*>(sm + kDecWarpAt);
+  for (uint32_t i = threadIdx.x; i < kDecCanonWords; i += blockDim.x) sm[i] = frame_tab[i];
+  for (uint32_t i = threadIdx.x; i < kDecLutWords; i += blockDim.x) sm[kDecWarpAt + i] = frame_tab[kDecCanonWords + i];
+  __syncthreads();
+  uint8_t* count = reinterpret_cast<uint8_t*>(sm + kDecCountAt);
+  const uint32_t most = sm[1] ? 2u : kDecLutBits;  // with a length-1 code the runs are taken by counting zeros
+  for (uint32_t x = threadIdx.x; x < kDecLutSize; x += blockDim.x) {
+    uint32_t pair = 0, at = 0, n = 0;
+    for (;;) {
+      const uint32_t ent = lut[(x << at) & (kDecLutSize - 1)], L = ent >> 10;
+      if (L == 0 || at + L > kDecLutBits) break;
+      at += L;
+      if (n == 0) pair = (ent & 1023u) | (L << 20);
+      if (n == 1) pair |= ((ent & 1023u) << 10) | (at << 24);
+      if (++n == most) break;
+    }
+    sm[kDecPairAt + x] = pair;
+    count[x] = (uint8_t)(n | (at << 4));
+  }
+  // codes of 13 .. 32 bits: the last 32-bit window that starts with a code of at
+  // most L bits (canonical codes grow with their length), then where the symbols
+  // of length L start, less its first code
+  if (threadIdx.x < 20) {
+    const uint32_t L = kDecLutBits + 1 + threadIdx.x;
+    uint32_t m = L;
+    while (m > 1 && sm[m] == 0) --m;
+    sm[kDecLongAt + threadIdx.x] = (uint32_t)(((uint64_t)sm[34 + m] + sm[m]) << (32 - m)) - 1u;
+    sm[kDecLongAt + 20 + threadIdx.x] = 102 + sm[68 + L] - sm[34 + L];
+  }
+  __syncthreads();
+}
+
+// A code of more than kDecLutBits bits from the top of `win`, by those tables:
+// the lengths 13 .. 20 are compared at once.
+__device__ __forceinline__ uint32_t decode_long_fast(const uint32_t* sm, uint32_t win, uint32_t& sym) {
+  const uint4* last = reinterpret_cast<const uint4*>(sm + kDecLongAt);
+  const uint4 a = last[0], b = last[1];
+  uint32_t i = (win > a.x) + (win > a.y) + (win > a.z) + (win > a.w) + (win > b.x) + (win > b.y) + (win > b.z) + (win > b.w);
+  if (i == 8) {
+    while (i < 20 && win > sm[kDecLongAt + i]) ++i;
+    if (i == 20) return 0;
+  }
+  const uint32_t L = kDecLutBits + 1 + i;
+  sym = sm[sm[kDecLongAt + 20 + i] + (win >> (32 - L))];
+  return L;
+}
+
+// Every symbol: a warp per chunk.  kDeltas: every frame, its residuals at their
+// bins; else the frames that are not sparse, their symbols.
+template <bool kDeltas>
+__global__ void __launch_bounds__(kDecWarps * 32, 2) k_dec_dense(DevParams p, Scratch s, DecArgs a) {
+  extern __shared__ __align__(16) uint32_t dec_sm[];
+  __shared__ int go;
+  const uint32_t f = blockIdx.y, lane = lane_id(), warp = threadIdx.x >> 5;
+  // other blocks of the frame may mark it corrupt meanwhile: read once and shared
+  if (threadIdx.x == 0) go = s.status[f] == ROIBIN_OK && (kDeltas || s.dec_info[f].sparse == 0);
+  __syncthreads();
+  if (!go) return;
+  build_dense_tables(s.dec_table + (size_t)f * kDecTableWords, dec_sm);
+  const uint32_t* tab = dec_sm;
+  const uint32_t* pair = dec_sm + kDecPairAt;
+  const uint8_t* counts = reinterpret_cast<const uint8_t*>(dec_sm + kDecCountAt);
+  uint32_t* stage = dec_sm + kDecWarpAt + warp * kDecWarpWords;
+  uint32_t* symw = stage + kDecStageWords + 8;
+  uint16_t* syms = reinterpret_cast<uint16_t*>(symw);
+  auto slot = [](uint32_t i) { return i + 2 * (i >> 6); };  // u16 index of symbol i in syms
+  const DecInfo& di = s.dec_info[f];
+  const uint8_t* base = a.in + di.base;
+  const uint32_t n_words = di.pl.n_words;
+  const uint32_t* cidx = reinterpret_cast<const uint32_t*>(base + di.pl.off_cidx);
+  const bool zrun = tab[1] != 0;  // the length-1 code is code 0: its symbol comes first in the (length, symbol) order
+  const uint32_t zsym = tab[102];
+  for (uint32_t k = blockIdx.x * kDecWarps + warp; k < p.n_chunks; k += gridDim.x * kDecWarps) {
+    const uint32_t w0 = cidx[k], w1 = k + 1 < p.n_chunks ? cidx[k + 1] : n_words;
+    const uint32_t nw = w1 - w0, n_sym = min(p.M, k * kChunk + kChunk) - k * kChunk;
+    if (w0 > w1 || w1 > n_words || nw > kChunk) {  // a chunk of n symbols takes at most n words
+      if (lane == 0) mark_corrupt(s, f);
+      continue;
+    }
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(base + di.pl.off_bits) + w0;
+    const bool staged = nw <= kDecStageWords;
+    if (staged) {
+      for (uint32_t i = lane; i < nw; i += 32) stage[i] = words[i];
+      if (lane < 8) stage[nw + lane] = 0;  // read past the end: a window starts below bit 32 nw
+    }
+    if (zrun)
+      for (uint32_t i = lane; i < kDecSymWords; i += 32) symw[i] = zsym * 0x10001u;
+    __syncwarp();
+    auto window = [&](uint32_t pos) {  // the 32 bits from bit pos < 32 nw
+      const uint32_t i = pos >> 5;
+      const uint32_t hi = staged ? stage[i] : __ldg(words + i);
+      const uint32_t lo = staged ? stage[i + 1] : (i + 1 < nw ? __ldg(words + i + 1) : 0u);
+      return __funnelshift_l(lo, hi, pos & 31u);
+    };
+    // counting pass over the codewords that start in [at, limit)
+    auto count_range = [&](uint32_t& at, uint32_t limit, uint32_t, auto) {
+      uint32_t pos = at, n = 0;
+      while (pos < limit) {
+        const uint32_t win = window(pos);
+        if (zrun && (int32_t)win >= 0) {
+          const uint32_t z = min((uint32_t)__clz(win), limit - pos);
+          n += z;
+          pos += z;
+          continue;
+        }
+        const uint32_t c = counts[win >> (32 - kDecLutBits)];
+        if (c != 0 && pos + kDecLutBits <= limit) {
+          n += c & 15u;
+          pos += c >> 4;
+          continue;
+        }
+        uint32_t L = (pair[win >> (32 - kDecLutBits)] >> 20) & 15u, sym;
+        if (L == 0) L = max(1u, decode_long_fast(dec_sm, win, sym));
+        ++n;
+        pos += L;
+      }
+      at = pos;
+      return n;
+    };
+    const uint32_t limit = (lane + 1) * nw;  // lane l covers bits [l nw, (l + 1) nw)
+    uint32_t start, n, listed;
+    sync_ranges(32, lane, lane * nw, limit, start, n, listed, count_range);
+    const uint32_t first = warp_incl_scan(n) - n;
+    // the storing pass: this lane's codewords are symbols first .. first + n - 1
+    uint32_t zeros = 0;
+    bool bad = false;
+    if (first < n_sym && n > 0) {
+      const uint32_t room = min(n, n_sym - first);
+      uint32_t pos = start, i = 0;
+      while (i < room) {
+        const uint32_t win = window(pos);
+        if (zrun && (int32_t)win >= 0) {  // prefilled
+          const uint32_t z = min((uint32_t)__clz(win), room - i);
+          if (zsym == 0) zeros += z;
+          i += z;
+          pos += z;
+          continue;
+        }
+        const uint32_t e = pair[win >> (32 - kDecLutBits)];
+        uint32_t L = (e >> 20) & 15u, sym = e & 1023u;
+        if (L == 0) {
+          L = decode_long_fast(dec_sm, win, sym);
+          if (L == 0) {
+            bad = true;
+            break;
+          }
+        }
+        syms[slot(first + i)] = (uint16_t)sym;
+        zeros += sym == 0;
+        ++i;
+        if ((e >> 24) != 0 && i < room) {
+          const uint32_t sym2 = (e >> 10) & 1023u;
+          syms[slot(first + i)] = (uint16_t)sym2;
+          zeros += sym2 == 0;
+          ++i;
+          L = e >> 24;
+        }
+        pos += L;
+      }
+      // the chunk's last symbol: its words must end with it
+      if (first + room == n_sym && (pos + 31) / 32 != nw) bad = true;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, first + n, 31);
+    bad = __any_sync(0xffffffffu, bad) || total < n_sym;
+    for (int d = 16; d > 0; d >>= 1) zeros += __shfl_xor_sync(0xffffffffu, zeros, d);
+    if (lane == 0) {
+      if (bad) mark_corrupt(s, f);
+      if (zeros) atomicAdd(s.dec_zero + f, zeros);
+    }
+    if (bad) continue;
+    __syncwarp();
+    if constexpr (kDeltas) {
+      int32_t* dq = s.dq + (size_t)f * p.M + (size_t)k * kChunk;
+      for (uint32_t i = lane; i < n_sym; i += 32) {
+        const uint32_t u = syms[slot(i)];
+        dq[i] = u ? (int32_t)u - di.R : kSentinel;
+      }
+    } else {
+      uint32_t* out = reinterpret_cast<uint32_t*>(s.codes + ((size_t)f * p.n_chunks + k) * kChunk);
+      for (uint32_t i = lane; 2 * i < n_sym; i += 32) out[i] = symw[i + (i >> 5)];  // a slot holds the whole last word
+    }
+    __syncwarp();  // the warp's area is free for its next chunk
   }
 }
 
@@ -814,7 +852,7 @@ __device__ __forceinline__ uint32_t place_strip_outliers(const uint2* v, uint32_
   }
 }
 
-// panel: one block per (panel, frame).  Strip by strip (sb binned rows):
+// The panel path: k_dec_sparse and k_dec_dense, then one block per (panel, frame).  Strip by strip (sb binned rows):
 //   symbols -> deltas in shared memory (code 0: sentinel), Lorenzo outliers in;
 //   column prefix sums carried from the strip above (thread per column);
 //   row prefix sums (thread per row segment: a sequential scan of its segment,
@@ -1080,9 +1118,27 @@ cudaError_t launch_dec_parse(const DevParams& p, const Scratch& s, const DecArgs
   k_dec_parse<<<a.n_frames, 256, 0, st>>>(p, s, a);
   return cudaGetLastError();
 }
-cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  dim3 grid(ceil_div(p.n_chunks, kDecThreads), a.n_frames);
-  k_dec_decode<<<grid, kDecThreads, 0, st>>>(p, s, a);
+cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArgs& a, bool deltas, cudaStream_t st) {
+  // dense blocks: one round of chunks each while that is at most two waves of 304
+  // resident blocks, else as many rounds as bring it there (each block builds its
+  // tables once, and the blocks of sparse frames end at once)
+  const uint32_t rounds = std::max<uint32_t>(1, (uint32_t)((uint64_t)ceil_div(p.n_chunks, kDecWarps) * a.n_frames / 608));
+  const dim3 grid(ceil_div(ceil_div(p.n_chunks, kDecWarps), rounds), a.n_frames);
+  const void* kern = deltas ? (const void*)k_dec_dense<true> : (const void*)k_dec_dense<false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmem);
+  if (e != cudaSuccess) return e;
+  if (deltas) {
+    k_dec_dense<true><<<grid, kDecWarps * 32, kDecSmem, st>>>(p, s, a);
+    return cudaGetLastError();
+  }
+  // lanes per chunk of a sparse frame: a whole warp while the lanes of all chunks
+  // fit the GPU at once (311,296 threads), else 16.  CSPAD-like frames, 32 / 16 / 8
+  // / 1 lanes: 1 frame 9.5 / 14 / 22 / 54 us, 64 frames 16.5 / 16.4 / 25 / 91 us,
+  // 400 frames 66 / 58 / 64 / 142 us, 1,000 frames 152 / 127 / 128 / 167 us.
+  const uint32_t lg = (uint64_t)p.n_chunks * a.n_frames <= 9728 ? 5 : 4;
+  k_dec_sparse<<<dim3(ceil_div(p.n_chunks << lg, kDecWarps * 32), a.n_frames), kDecWarps * 32, 0, st>>>(p, s, a, lg);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_dec_dense<false><<<grid, kDecWarps * 32, kDecSmem, st>>>(p, s, a);
   return cudaGetLastError();
 }
 cudaError_t launch_dec_lorenzo(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
@@ -1138,15 +1194,6 @@ uint32_t dec_panel_rows(const DevParams& p) {
   while (most < 32 && most < p.Hb && panel_smem_bytes(p.Wb, most + 1) <= 24576) ++most;
   const uint32_t strips = ceil_div(p.Hb, most);
   return ceil_div(p.Hb, strips);
-}
-cudaError_t launch_dec_decoders(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  // a thread per chunk, in whole warps; a frame's chunks in as few blocks as fit
-  const uint32_t threads = std::min<uint32_t>(kDecMaxThreads, ceil_div(p.n_chunks, 32) * 32);
-  dim3 grid(ceil_div(p.n_chunks, threads), a.n_frames);
-  k_dec_decode_sparse<<<grid, threads, 0, st>>>(p, s, a);
-  if (cudaGetLastError() != cudaSuccess) return cudaGetLastError();
-  k_dec_decode_dense<<<grid, threads, 0, st>>>(p, s, a);
-  return cudaGetLastError();
 }
 cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   const uint32_t sb = dec_panel_rows(p);

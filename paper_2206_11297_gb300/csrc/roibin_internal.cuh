@@ -1142,7 +1142,9 @@ struct DecArgs {
   int32_t* frame_status;
 };
 cudaError_t launch_dec_parse(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
-cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
+// decodes every chunk: residuals for the multi-pass path (deltas), else symbols
+// (or a sparse frame's lists of them) for the panel path
+cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArgs& a, bool deltas, cudaStream_t st);
 cudaError_t launch_dec_lorenzo(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_dec_rows(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_dec_cols(const DevParams& p, const Scratch& s, const DecArgs& a, bool dequant, cudaStream_t st);
@@ -1157,8 +1159,6 @@ cudaError_t launch_dec_finish(const Scratch& s, const DecArgs& a, cudaStream_t s
 // the panel path: decode through the prefix table into symbols, then one block
 // per (frame, panel) rebuilds the panel strip by strip
 uint32_t dec_panel_rows(const DevParams& p);  // binned rows per strip; 0: panel path unavailable
-// the decoders of the panel path: k_dec_decode_sparse, then k_dec_decode_dense
-cudaError_t launch_dec_decoders(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_roi_mask(const DevParams& p, const uint16_t* peaks, const uint32_t* npeaks,
                             uint32_t n, uint8_t* mask, cudaStream_t st);
