@@ -390,7 +390,40 @@ __global__ void k_dec_upsample(DevParams p, Scratch s, DecArgs a, int vec4) {
   }
 }
 
-// roi: restore every in-panel ROI pixel from the stream (one warp per peak).
+// One warp writes the in-panel pixels of the roi_h x roi_w window `src`, centred
+// on (r, c), into `panel`.  Ten loads a lane are in flight before the stores, so a
+// 17 x 17 window costs one round trip; (row, column) of the lane's elements are
+// stepped, not divided.
+__device__ __forceinline__ void warp_restore_roi(const float* __restrict__ src, int roi_h, int roi_w, float* panel, int H,
+                                                 int W, int r, int c) {
+  constexpr int U = 10;
+  const int win = roi_h * roi_w, lane = (int)lane_id(), r0 = r - roi_h / 2, c0 = c - roi_w / 2;
+  const int step_r = 32 / roi_w, step_c = 32 - step_r * roi_w;
+  int qr = lane / roi_w, qc = lane - qr * roi_w;
+  for (int e0 = lane; e0 < win + lane; e0 += 32 * U) {
+    float v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = e0 + 32 * u < win ? __ldg(src + e0 + 32 * u) : 0.0f;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int rr = r0 + qr, cc = c0 + qc;
+      if (e0 + 32 * u < win && rr >= 0 && rr < H && cc >= 0 && cc < W) panel[(size_t)rr * W + cc] = v[u];
+      qr += step_r;
+      qc += step_c;
+      if (qc >= roi_w) {
+        qc -= roi_w;
+        ++qr;
+      }
+    }
+  }
+}
+
+// roi: restore every in-panel ROI pixel from the stream (one warp per peak), on
+// both paths; a ROI section after the bitstream is restored by k_dec_roi_coded.
+// Inside the panel kernel the windows were one block's work per panel, each warp
+// looking at every peak of the frame in turn: 60 epix10k frames of 3,000 windows,
+// most of them on three panels, took 1,190 us there (108 us without windows), and
+// 87 us here.
 __global__ void k_dec_roi(DevParams p, Scratch s, DecArgs a) {
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
@@ -408,13 +441,8 @@ __global__ void k_dec_roi(DevParams p, Scratch s, DecArgs a) {
       continue;
     }
     float* panel = a.out + (size_t)f * p.frame_px + (size_t)pn * p.H * p.W;
-    const int r0 = (int)r - di.roi_h / 2, c0 = (int)c - di.roi_w / 2;
     if (!RB_CHECK(s, di.pl.off_roi + (uint64_t)(k + 1) * win * 4 <= di.pl.total, ROIBIN_CHECK_STREAM_READ)) continue;
-    for (uint32_t e = lane_id(); e < win; e += 32) {
-      const int rr = r0 + (int)(e / di.roi_w), cc = c0 + (int)(e % di.roi_w);
-      if (rr >= 0 && rr < (int)p.H && cc >= 0 && cc < (int)p.W)
-        panel[(size_t)rr * p.W + cc] = roi[(size_t)k * win + e];
-    }
+    warp_restore_roi(roi + (size_t)k * win, di.roi_h, di.roi_w, panel, (int)p.H, (int)p.W, (int)r, (int)c);
   }
 }
 
@@ -855,11 +883,13 @@ __device__ __forceinline__ uint32_t place_strip_outliers(const uint2* v, uint32_
 // The panel path: k_dec_sparse and k_dec_dense, then one block per (panel, frame).  Strip by strip (sb binned rows):
 //   symbols -> deltas in shared memory (code 0: sentinel), Lorenzo outliers in;
 //   column prefix sums carried from the strip above (thread per column);
-//   row prefix sums (thread per row segment: a sequential scan of its segment,
-//   then the segment totals scanned across the lanes of the row);
-//   b^ = fl(q * 2eb), prequantisation outliers in;
-//   the strip's output rows (every pixel takes its bin's value).
-// After the last strip, the panel's ROI windows overwrite their in-panel pixels.
+//   row prefix sums, b^ = fl(q * 2eb) and the row's pixels by a warp per row from
+//   registers (bin width 2).  Strips with prequantisation outliers and other bin
+//   widths take them apart: a thread per row segment, b^ back to the tile, the
+//   outliers in, then the output rows.  The one pass instead of three took the
+//   kernel from 185 to 108 us on 60 epix10k frames and from 650 to 617 us on 400
+//   CSPAD-like frames (5.96 TB/s of pixels written, 0.88 of the copy rate).
+// k_dec_roi then overwrites the pixels of the ROI windows.
 // The 2-D prefix sum wraps modulo 2^32 in any order, so column-then-row equals
 // the row-then-column definition.
 // The symbols of the next strip arrive by a 1-D TMA bulk copy (a 16-byte
@@ -946,6 +976,8 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
   const uint32_t dr = vec4 ? blockDim.x / W4 : 0, dc = vec4 ? blockDim.x - dr * W4 : 0;
   bool bad = false;
   for (uint32_t j = threadIdx.x; j < Wb; j += blockDim.x) carry[j] = 0;
+  const uint32_t lane = lane_id();
+  __syncthreads();
   for (uint32_t r0 = 0; r0 < Hb; r0 += sb) {
     const uint32_t nr = min(sb, Hb - r0), nb = nr * Wb;
     const uint32_t sb0 = pb + r0 * Wb, sb1 = sb0 + nb;
@@ -982,7 +1014,8 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
       // the buffer is free: the next strip's symbols come in behind this one
       if (threadIdx.x == 0 && r0 + sb < Hb) fetch(r0 + sb);
     }
-    lo_cur = place_strip_outliers(lo, lo_cur, lo_end, sb1, [&](uint32_t x, uint32_t y) {
+    if (lo_cur != lo_end)
+      lo_cur = place_strip_outliers(lo, lo_cur, lo_end, sb1, [&](uint32_t x, uint32_t y) {
       if (x < sb0 || tile[x - sb0] != (uint32_t)kSentinel) return false;
       tile[x - sb0] = y;
       return true;
@@ -998,56 +1031,82 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
       carry[j] = q;
     }
     __syncthreads();
-    // row prefix sums and b^ = fl(q * 2eb)
-    {
-      const bool mine = seg_row < nr;
-      uint32_t* row = tile + seg_row * Wb;
-      uint32_t run = 0;
-      if (mine)
-        for (uint32_t j = sj0; j < sj1; ++j) {
-          run += row[j];
-          row[j] = run;
-        }
-      // exclusive scan of the segment totals across the G lanes of the row
-      uint32_t incl = run;
-      for (uint32_t d = 1; d < G; d <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, d, G);
-        if (seg >= d) incl += v;
-      }
-      const uint32_t excl = incl - run;
-      if (mine)
-        for (uint32_t j = sj0; j < sj1; ++j)
-          tilef[seg_row * Wb + j] = __fmul_rn((float)(int32_t)(row[j] + excl), two_eb);
-    }
-    __syncthreads();
-    pq_cur = place_strip_outliers(pq, pq_cur, pq_end, sb1, [&](uint32_t x, uint32_t y) {
-      if (x < sb0) return false;
-      tilef[x - sb0] = __uint_as_float(y);
-      return true;
-    }, bad);
-    // output rows of the strip: bin row i covers pixel rows (r0 + i) * bh ...
-    // (streaming stores: the kernel never reads these pixels back)
-    if (vec4) {  // bin width 2, W % 4 == 0: one float4 = 2 bins, stored on each of its rows
-      const uint32_t n2 = nr * W4;
-      uint32_t i = threadIdx.x / W4, c4 = threadIdx.x - i * W4;
-      for (uint32_t e = threadIdx.x; e < n2; e += blockDim.x) {
-        const float2 v = *reinterpret_cast<const float2*>(tilef + i * Wb + 2 * c4);
-        const float4 o = make_float4(v.x, v.x, v.y, v.y);
+    // prequantisation outliers in this strip (the same answer in every thread)
+    const bool any_pq = pq_cur != pq_end && pq[pq_cur].x < sb1;
+    if (vec4 && !any_pq) {
+      // a warp per row: row prefix sums by shuffles, two bins a lane, and from the
+      // registers b^ = fl(q * 2eb) straight to the row's pixels (one float4 on each
+      // of its pixel rows; streaming stores: the kernel never reads them back)
+      for (uint32_t i = threadIdx.x >> 5; i < nr; i += kPanelThreads / 32) {
+        const uint2* row = reinterpret_cast<const uint2*>(tile + i * Wb);
         const uint32_t pr0 = (r0 + i) * bh, pr1 = min(H, pr0 + bh);
-        for (uint32_t pr = pr0; pr < pr1; ++pr) __stcs(reinterpret_cast<float4*>(panel + (size_t)pr * W) + c4, o);
-        i += dr;
-        c4 += dc;
-        if (c4 >= W4) {
-          c4 -= W4;
-          ++i;
+        float4* px = reinterpret_cast<float4*>(panel + (size_t)pr0 * W);
+        uint32_t run = 0;  // sum of the row before this round's bins
+        for (uint32_t c0 = 0; c0 < W4; c0 += 32) {
+          const uint32_t c4 = c0 + lane;
+          const uint2 v = c4 < W4 ? row[c4] : make_uint2(0u, 0u);
+          const uint32_t sum = v.x + v.y, incl = warp_incl_scan(sum);
+          const uint32_t q0 = run + incl - v.y, q1 = run + incl;
+          run += __shfl_sync(0xffffffffu, incl, 31);
+          if (c4 < W4) {
+            const float b0 = __fmul_rn((float)(int32_t)q0, two_eb), b1 = __fmul_rn((float)(int32_t)q1, two_eb);
+            const float4 o = make_float4(b0, b0, b1, b1);
+            for (uint32_t pr = pr0; pr < pr1; ++pr) __stcs(px + (size_t)(pr - pr0) * W4 + c4, o);
+          }
         }
       }
     } else {
-      const uint32_t ro0 = r0 * bh, ro1 = min(H, (r0 + nr) * bh);
-      const uint32_t n1 = (ro1 - ro0) * W;
-      for (uint32_t e = threadIdx.x; e < n1; e += blockDim.x) {
-        const uint32_t rr = e / W, c = e - rr * W;
-        __stcs(panel + (size_t)ro0 * W + e, tilef[((ro0 + rr) / bh - r0) * Wb + c / p.bw]);
+      // row prefix sums and b^ = fl(q * 2eb)
+      {
+        const bool mine = seg_row < nr;
+        uint32_t* row = tile + seg_row * Wb;
+        uint32_t run = 0;
+        if (mine)
+          for (uint32_t j = sj0; j < sj1; ++j) {
+            run += row[j];
+            row[j] = run;
+          }
+        // exclusive scan of the segment totals across the G lanes of the row
+        uint32_t incl = run;
+        for (uint32_t d = 1; d < G; d <<= 1) {
+          const uint32_t v = __shfl_up_sync(0xffffffffu, incl, d, G);
+          if (seg >= d) incl += v;
+        }
+        const uint32_t excl = incl - run;
+        if (mine)
+          for (uint32_t j = sj0; j < sj1; ++j)
+            tilef[seg_row * Wb + j] = __fmul_rn((float)(int32_t)(row[j] + excl), two_eb);
+      }
+      __syncthreads();
+      pq_cur = place_strip_outliers(pq, pq_cur, pq_end, sb1, [&](uint32_t x, uint32_t y) {
+        if (x < sb0) return false;
+        tilef[x - sb0] = __uint_as_float(y);
+        return true;
+      }, bad);
+      // output rows of the strip: bin row i covers pixel rows (r0 + i) * bh ...
+      // (streaming stores: the kernel never reads these pixels back)
+      if (vec4) {  // bin width 2, W % 4 == 0: one float4 = 2 bins, stored on each of its rows
+        const uint32_t n2 = nr * W4;
+        uint32_t i = threadIdx.x / W4, c4 = threadIdx.x - i * W4;
+        for (uint32_t e = threadIdx.x; e < n2; e += blockDim.x) {
+          const float2 v = *reinterpret_cast<const float2*>(tilef + i * Wb + 2 * c4);
+          const float4 o = make_float4(v.x, v.x, v.y, v.y);
+          const uint32_t pr0 = (r0 + i) * bh, pr1 = min(H, pr0 + bh);
+          for (uint32_t pr = pr0; pr < pr1; ++pr) __stcs(reinterpret_cast<float4*>(panel + (size_t)pr * W) + c4, o);
+          i += dr;
+          c4 += dc;
+          if (c4 >= W4) {
+            c4 -= W4;
+            ++i;
+          }
+        }
+      } else {
+        const uint32_t ro0 = r0 * bh, ro1 = min(H, (r0 + nr) * bh);
+        const uint32_t n1 = (ro1 - ro0) * W;
+        for (uint32_t e = threadIdx.x; e < n1; e += blockDim.x) {
+          const uint32_t rr = e / W, c = e - rr * W;
+          __stcs(panel + (size_t)ro0 * W + e, tilef[((ro0 + rr) / bh - r0) * Wb + c / p.bw]);
+        }
       }
     }
     __syncthreads();
@@ -1056,25 +1115,6 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
   if (timed_out) {
     if (threadIdx.x == 0) s.status[f] = ROIBIN_ERR_TIMEOUT;
     return;
-  }
-  // ROI windows of this panel's peaks (every block checks every peak's place);
-  // a ROI section after the bitstream is restored by k_dec_roi_coded instead
-  const uint16_t* pk = reinterpret_cast<const uint16_t*>(base + di.pl.off_peaks);
-  const float* roi = reinterpret_cast<const float*>(base + di.pl.off_roi);
-  const uint32_t win = (uint32_t)(di.roi_h * di.roi_w);
-  const uint32_t n_in_place = di.roi_coding == 0 ? di.pl.n_peaks : 0u;
-  for (uint32_t k = threadIdx.x >> 5; k < n_in_place; k += blockDim.x >> 5) {
-    const uint32_t kp = pk[3 * k], r = pk[3 * k + 1], c = pk[3 * k + 2];
-    if (kp >= p.P || r >= H || c >= W) {
-      bad = true;
-      continue;
-    }
-    if (kp != pn) continue;
-    const int r0 = (int)r - di.roi_h / 2, c0 = (int)c - di.roi_w / 2;
-    for (uint32_t e = lane_id(); e < win; e += 32) {
-      const int rr = r0 + (int)(e / di.roi_w), cc = c0 + (int)(e % di.roi_w);
-      if (rr >= 0 && rr < (int)H && cc >= 0 && cc < (int)W) panel[(size_t)rr * W + cc] = roi[(size_t)k * win + e];
-    }
   }
   if (bad) mark_corrupt(s, f);
 }
@@ -1178,7 +1218,8 @@ cudaError_t launch_dec_upsample(const DevParams& p, const Scratch& s, const DecA
   return cudaGetLastError();
 }
 cudaError_t launch_dec_roi(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  dim3 grid(64, a.n_frames);
+  // about 4,096 blocks of eight windows a round, at least 8 and at most 64 a frame
+  dim3 grid(std::max<uint32_t>(8, std::min<uint32_t>(64, 4096 / a.n_frames)), a.n_frames);
   k_dec_roi<<<grid, 256, 0, st>>>(p, s, a);
   return cudaGetLastError();
 }
