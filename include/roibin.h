@@ -318,10 +318,12 @@ int roibin_ctx_set_wait_limit(roibin_ctx* ctx, int64_t polls);
  * start, 4 plan done (head written); summed over the frame's chunk items:
  * 5 size items, 6 write items, 7 size waits, 8 write waits, 9 size chunk
  * loops, 10 write chunk loops, 11 write ROI copies (12..15 unused).  After
- * the n_frames * 16 words, every streaming item u of a traced frame f (items
- * are groups of consecutive panels, fewer than P per frame) writes 4 stamps
- * at index n_frames * 16 + (f * P + u) * 4: start, streaming done, peaks done
- * (3 unused; slots of items that do not exist stay zero).  The caller zeroes d_trace before the call and owns
+ * the n_frames * 16 words, every streaming item u < P of a traced frame f (items
+ * are groups of consecutive panels, in small batches row bands of them; those
+ * past the first P are not traced) writes 4 stamps at index
+ * n_frames * 16 + (f * P + u) * 4: start, streaming done, peaks done (3 unused;
+ * slots of items that do not exist stay zero).  The caller zeroes d_trace before
+ * the call and owns
  * it (device u64[n_frames * (16 + 4 P)]); n_frames = 0 switches tracing off.
  */
 int roibin_ctx_set_trace(roibin_ctx* ctx, uint64_t* d_trace, uint32_t n_frames);

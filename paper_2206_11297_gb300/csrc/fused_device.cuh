@@ -24,8 +24,9 @@ constexpr uint32_t kProducerWarp = 7;   // the warp whose lane 0 issues the row 
 constexpr uint32_t kThrLocalCap = 256;
 constexpr uint32_t kBlockKey = 1u << 31;  // a listed 2x4 block (else a listed candidate pixel)
 constexpr uint32_t kPqList = 128;  // prequantisation outliers an item lists before rescanning
-constexpr uint32_t kLagSize = 65535, kLagWrite = 64;  // see launch_fused
-constexpr uint32_t kPanelTimedOut = 0xFFFFFFFFu;  // peak count of an item whose rows never arrived
+constexpr uint32_t kHuffArea = 29 * 1024;  // bytes of the Huffman scratch and of what shares its place
+static_assert(sizeof(HuffSmem) <= kHuffArea, "the Huffman scratch fits its area");
+constexpr uint32_t kLagWrite = 64;  // see launch_fused
 
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
@@ -144,7 +145,6 @@ struct StreamView {
   uint32_t* thr;   // [kThrLocalCap] listed candidates (item-local pixel) or 2x4 blocks (kBlockKey set)
   float* thrv;     // [kThrLocalCap] value of each listed candidate
   float* nb;       // [kPW][side^2] peak-test neighbourhoods (aliases the ring)
-  uint32_t* acc;   // [sort_n2] accepted peaks of the item (aliases the ring)
   uint32_t* cand;  // [kThrLocalCap] listed candidates left after pruning (aliases the ring)
   uint32_t* ctl;
   unsigned char* ring;  // [stages][stage_bytes] raw rows in flight
@@ -155,16 +155,13 @@ struct FinView {
   uint32_t* total;  // [kMaxSymbols]
   uint8_t* cb_len;  // [kMaxSymbols]
   uint32_t* cb_code;
-  uint32_t* keys;  // [peak_cap]
   uint32_t* cw;    // [n_chunks] chunk words -> word offsets; then lo, pq
   uint32_t* clo;
   uint32_t* cpq;
-  uint32_t* offs;  // [U] offset of each item's peaks in the frame list
   uint32_t* ctl;
 };
 enum {
   CTL_THR = 0,
-  CTL_ACC,
   CTL_ITEM,
   CTL_LAST,
   CTL_BAD,
@@ -190,7 +187,6 @@ __device__ __forceinline__ StreamView stream_view(unsigned char* sm, const Fused
   v.thr = reinterpret_cast<uint32_t*>(sm + sh.off_thr);
   v.thrv = reinterpret_cast<float*>(sm + sh.off_thr + kThrLocalCap * 4);
   v.nb = reinterpret_cast<float*>(sm + sh.off_nb);
-  v.acc = reinterpret_cast<uint32_t*>(sm + sh.off_acc);
   v.cand = reinterpret_cast<uint32_t*>(sm + sh.off_cand);
   v.ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
   v.ring = sm + sh.off_ring;
@@ -203,41 +199,86 @@ __device__ __forceinline__ FinView fin_view(unsigned char* sm, const FusedShape&
   v.total = reinterpret_cast<uint32_t*>(sm + sh.off_total);
   v.cb_len = sm + sh.off_cblen;
   v.cb_code = reinterpret_cast<uint32_t*>(sm + sh.off_cbcode);
-  v.keys = reinterpret_cast<uint32_t*>(sm + sh.off_keys);
   v.cw = reinterpret_cast<uint32_t*>(sm + sh.off_cw);
   v.clo = v.cw + sh.n_chunks;
   v.cpq = v.clo + sh.n_chunks;
-  v.offs = reinterpret_cast<uint32_t*>(sm + sh.off_offs);
   v.ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
   return v;
 }
 
+// Per-frame words, zeroed before each launch:
+//   panel_done, size_done   streaming / size items finished;
+//   stage                   bit 0: the codebook is published, bit 1: the plan is;
+//   fin                     the plan and the write items finished (the one that
+//                           finishes last settles the frame's status); bit 31 is
+//                           set by any item that gave up waiting (sticky: no later
+//                           write of the frame's status can clear it);
+//   chunk_done              (per chunk of frames) frames whose peaks are known;
+//   peak_n, pq_n            peaks accepted, prequantisation outliers.
+struct SyncWords {
+  uint32_t *panel_done, *size_done, *stage, *fin, *chunk_done, *peak_n, *pq_n, *ticket;
+};
+constexpr uint32_t kStageCodebook = 1u, kStagePlan = 2u, kGaveUp = 1u << 31;
+__device__ __forceinline__ SyncWords sync_words(const Scratch& s, uint32_t n) {
+  SyncWords w;
+  w.panel_done = s.frame_done;
+  w.size_done = s.frame_done + n;
+  w.stage = s.frame_done + 2 * n;
+  w.fin = s.frame_done + 3 * n;
+  w.chunk_done = s.frame_done + 4 * n;
+  w.peak_n = s.frame_done + 5 * n;
+  w.pq_n = s.frame_done + 6 * n;
+  w.ticket = s.frame_done + kSyncWordsPerFrame * n;
+  return w;
+}
+// A peak accepted by a streaming item: to the frame's list, in any order (the
+// codebook stage sorts it); past max_peaks it is only counted.
+__device__ __forceinline__ void add_peak(const DevParams& p, const PlainArgs& a, uint32_t* peak_n, uint32_t f, uint32_t px) {
+  const uint32_t slot = atomicAdd(peak_n + f, 1u);
+  if (slot < p.max_peaks) a.peaks_key_out[(size_t)f * p.max_peaks + slot] = px;
+}
+
 // ---------------------------------------------------------------------------
-// a1 + a2 for an item with more candidates than its list holds (hot pixels),
-// one lane per candidate, every pixel read from shared memory.  The item's
-// panels are taken in bands of rows: a band of B rows plus `reach` rows above
-// and below (the whole neighbourhood of every candidate in it) is staged in
-// the ring's memory by one bulk copy.  The band's pixels >=
-// amax_thr are ranked in a block-wide scan (each thread counts its own run of
-// the band, then the runs' counts are scanned), and rank q goes to thread
-// q mod 256 in rounds, so every thread holds a candidate whatever their number.
-// Each thread runs the local-maximum rule and the evaluation in the sequential
-// order of is_local_max_at / evaluate_peak_at.  Accepted pixels (item-local
-// index) are collected in the item's slot of s.peak_part; the caller sorts them.
-__device__ __noinline__ void dense_band_peaks(const DevParams& p, const Scratch& s, const FusedShape& sh,
-                                              const StreamView& v, const float* item_px, uint32_t kp, size_t fu) {
+// a1 + a2 for an item with many candidates (hot pixels), one lane per candidate,
+// every pixel read from shared memory.  The item's panels are taken in bands of
+// rows: a band of B rows plus `reach` rows above and below (the whole
+// neighbourhood of every candidate in it) is staged in the ring's memory by one
+// bulk copy.  Each thread marks the pixels >= amax_thr of its float4s in a bit
+// mask, a block-wide scan ranks them, and up to kBandList of them at a time are
+// listed: those 6 or more pixels inside the panel from the front (peak_test_inner,
+// a lane each), the others from the back (warp_peak_test_small, a warp each; a
+// lane's test with its checks per pixel took 13 thousand cycles, and one such
+// candidate held up its whole band).  Other windows and rings run the general
+// test.  Accepted pixels go to the frame's list (add_peak).
+// The test is bound by its chain of ordered sums and by shared-memory reads of
+// scattered pixels: an SM holds about 12 warps of candidates (what fits its shared
+// memory with the halos), each issuing one instruction in 8 cycles.  100 epix10k
+// hot-pixel frames, per item of 2,700 candidates: 590 -> 430 us; 30 such frames on
+// the plain variant, a warp per candidate before: 3,530 -> 690 us in all.
+constexpr uint32_t kBandList = 2 * kThrLocalCap;  // candidates listed at once (the words of thr and thrv)
+
+__device__ __noinline__ void dense_band_peaks(const DevParams& p, const PlainArgs& a, const FusedShape& sh,
+                                              uint32_t* peak_n, uint32_t f, uint32_t pn0, uint32_t kp, uint32_t row0,
+                                              uint32_t row1, uint32_t band_rows) {
+  extern __shared__ __align__(128) unsigned char sm[];  // the launch's: v's pointers, known to be shared
   const uint32_t tid = threadIdx.x, W = p.W, H = p.H, plane = H * W;
-  const uint32_t reach = (uint32_t)peak_reach(p), B = sh.band_rows - 2 * reach;
-  float* band = reinterpret_cast<float*>(v.ring);
-  uint32_t* run_start = v.thr;  // [kPT] first rank of each thread's run
-  uint32_t* acc = s.peak_part + fu * sh.peak_cap;
-  uint64_t* band_bar = v.bars + 2 * sh.stages;
+  const float* item_px = a.frames + (size_t)f * p.frame_px + (size_t)pn0 * plane;
+  const uint32_t reach = (uint32_t)peak_reach(p), B = band_rows - 2 * reach;
+  float* band = reinterpret_cast<float*>(sm + sh.off_ring);
+  uint32_t* list = reinterpret_cast<uint32_t*>(sm + sh.off_thr);  // [kBandList] (row << 16) | column in the panel
+  uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
+  uint64_t* band_bar = reinterpret_cast<uint64_t*>(sm + sh.off_bar) + 2 * sh.stages;
   const uint64_t pol = evict_normal_policy();  // a band's halo rows are read again by the next band
-  uint32_t bands_done = v.ctl[CTL_BAND];
+  uint32_t bands_done = ctl[CTL_BAND];
+  const bool paper = p.rank == 3 && p.ring_r0 == 5 && p.ring_dr == 2;
+  // per warp, the ring's or the window's pixels of one test (at most 76): the
+  // item's histogram has been flushed
+  float* wbuf = reinterpret_cast<float*>(sm + sh.off_hist) + (tid >> 5) * 96;
+  static_assert(kPW * 96 <= kMaxSymbols, "the warps' buffers fit the histogram");
   for (uint32_t j = 0; j < kp; ++j) {
     const float* pan = item_px + (size_t)j * plane;
-    for (uint32_t r0 = 0; r0 < H; r0 += B) {
-      const uint32_t r1 = min(H, r0 + B);
+    for (uint32_t r0 = row0; r0 < row1; r0 += B) {
+      const uint32_t r1 = min(row1, r0 + B);
       const uint32_t rb0 = r0 >= reach ? r0 - reach : 0u, rb1 = min(H, r1 + reach);
       __syncthreads();  // the previous band is no longer read
       // one bulk copy of the band's rows (contiguous in the panel, 16-byte
@@ -251,56 +292,264 @@ __device__ __noinline__ void dense_band_peaks(const DevParams& p, const Scratch&
       const bool landed = mbar_wait(band_bar, (bands_done++) & 1u);
       if (!__syncthreads_and(landed)) {  // the copy never arrived: the item is marked, see process_item
         if (tid == 0) {
-          v.ctl[CTL_TIMEOUT] = 1;
-          v.ctl[CTL_BAND] = bands_done;
+          ctl[CTL_TIMEOUT] = 1;
+          ctl[CTL_BAND] = bands_done;
         }
         __syncthreads();
         return;
       }
-      // pass 1: each thread counts the candidates of its run of the band's own rows
-      const float* core = band + (size_t)(r0 - rb0) * W;
-      const uint32_t n_core = (r1 - r0) * W, run = ceil_div(n_core, kPT);
-      const uint32_t x0 = min(n_core, tid * run), x1 = min(n_core, x0 + run);
-      uint32_t cnt = 0;
-      for (uint32_t x = x0; x < x1; ++x) cnt += core[x] >= p.amax;
-      uint32_t total;
-      const uint32_t first = block_excl_scan(cnt, v.ctl + CTL_TMP, &total);
-      run_start[tid] = first;
-      __syncthreads();
-      // pass 2: rank q -> the run holding it (the last run starting at or before
-      // q), then the (q - start)-th candidate of that run
-      for (uint32_t q0 = 0; q0 < total; q0 += kPT) {
-        const uint32_t q = q0 + tid;
-        if (q >= total) continue;
-        uint32_t lo = 0, hi = kPT - 1;
-        while (lo < hi) {
-          const uint32_t mid = (lo + hi + 1) >> 1;
-          if (run_start[mid] <= q) lo = mid;
-          else hi = mid - 1;
+      const float4* core = reinterpret_cast<const float4*>(band + (size_t)(r0 - rb0) * W);
+      const uint32_t n4 = (r1 - r0) * (W / 4);
+      for (uint32_t base = 0; base < n4; base += 8 * kPT) {  // eight float4s a thread: a 32-bit mask
+        uint32_t hot = 0;
+#pragma unroll
+        for (uint32_t e = 0; e < 8; ++e) {
+          const uint32_t i = base + e * kPT + tid;
+          if (i < n4) {
+            const float4 x = core[i];
+            hot |= ((uint32_t)(x.x >= p.amax) | (uint32_t)(x.y >= p.amax) << 1 | (uint32_t)(x.z >= p.amax) << 2 |
+                    (uint32_t)(x.w >= p.amax) << 3)
+                   << (4 * e);
+          }
         }
-        uint32_t skip = q - run_start[lo], x = min(n_core, lo * run);
-        for (;; ++x)
-          if (core[x] >= p.amax && skip-- == 0) break;
-        const int r = (int)(r0 + x / W), c = (int)(x % W);
-        const float* at = band + (size_t)(r - (int)rb0) * W + c;
-        auto px = [&](int dr, int dc) { return at[dr * (int)W + dc]; };
-        if (peak_test_one(px, (int)H, (int)W, r, c, p)) {
-          const uint32_t slot = atomicAdd(v.ctl + CTL_ACC, 1u);
-          if (slot < sh.peak_cap) acc[slot] = j * plane + (uint32_t)r * W + (uint32_t)c;
+        uint32_t total;
+        const uint32_t first = block_excl_scan(__popc(hot), ctl + CTL_TMP, &total);
+        for (uint32_t q0 = 0; q0 < total; q0 += kBandList) {
+          if (tid < 2) ctl[CTL_CARRY0 + tid] = 0;  // inner, edge candidates listed
+          __syncthreads();
+          uint32_t rank = first;
+          for (uint32_t m = hot; m; m &= m - 1, ++rank) {
+            if (rank < q0 || rank >= q0 + kBandList) continue;
+            const uint32_t bit = __ffs(m) - 1, x = 4 * (base + (bit >> 2) * kPT + tid) + (bit & 3u);
+            const uint32_t r = r0 + x / W, c = x % W;
+            const bool inner = paper && r >= 6 && r + 6 < H && c >= 6 && c + 6 < W;
+            const uint32_t at = atomicAdd(ctl + CTL_CARRY0 + (inner ? 0 : 1), 1u);
+            list[inner ? at : kBandList - 1 - at] = (r << 16) | c;
+          }
+          __syncthreads();
+          const uint32_t n_in = ctl[CTL_CARRY0], n_edge = ctl[CTL_CARRY1];
+          auto accept = [&](uint32_t r, uint32_t c) { add_peak(p, a, peak_n, f, (pn0 + j) * plane + r * W + c); };
+          for (uint32_t i = tid; i < n_in; i += kPT) {
+            const uint32_t r = list[i] >> 16, c = list[i] & 0xFFFFu;
+            if (peak_test_inner(band + (size_t)(r - rb0) * W + c, (int)W, p)) accept(r, c);
+          }
+          if (paper) {  // the last warp first: the candidates above start from the first
+            for (uint32_t i = kPW - 1 - (tid >> 5); i < n_edge; i += kPW) {
+              const uint32_t r = list[kBandList - 1 - i] >> 16, c = list[kBandList - 1 - i] & 0xFFFFu;
+              // the panel as the band shows it: the test reads rows rb0 .. rb1 - 1 of it only
+              const float* pan_band = band - (ptrdiff_t)rb0 * W;
+              if (warp_peak_test_small(pan_band, (int)H, (int)W, (int)r, (int)c, p, wbuf,
+                                       [](const float* q) { return *q; }) &&
+                  lane_id() == 0)
+                accept(r, c);
+            }
+          } else {
+            for (uint32_t i = tid; i < n_edge; i += kPT) {
+              const uint32_t r = list[kBandList - 1 - i] >> 16, c = list[kBandList - 1 - i] & 0xFFFFu;
+              const float* at = band + (size_t)(r - rb0) * W + c;
+              auto px = [&](int dr, int dc) { return at[dr * (int)W + dc]; };
+              if (is_local_max_at(px, (int)H, (int)W, (int)r, (int)c, p) &&
+                  evaluate_peak_at(px, (int)H, (int)W, (int)r, (int)c, p))
+                accept(r, c);
+            }
+          }
+          __syncthreads();  // the list is free
         }
       }
     }
   }
   __syncthreads();
-  if (tid == 0) v.ctl[CTL_BAND] = bands_done;
-  // the item's accepted pixels into the shared list the caller sorts
-  const uint32_t n_acc = v.ctl[CTL_ACC];
-  if (n_acc <= p.max_peaks)
-    for (uint32_t k = tid; k < n_acc; k += kPT) v.acc[k] = __ldcg(acc + k);
+  if (tid == 0) ctl[CTL_BAND] = bands_done;
+}
+
+// a1 + a2 on the listed blocks and pixels of a streaming item, raw rows [row0,
+// row1) of its panels (on every pixel >= amax_thr there if the list overflowed).
+__device__ __forceinline__ void item_peaks(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
+                                        unsigned char* sm, uint32_t* peak_n, uint32_t f, uint32_t pn0, uint32_t kp,
+                                        uint32_t row0, uint32_t row1) {
+  const StreamView v = stream_view(sm, sh);
+  const bool dense = sh.dense != 0;
+  const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5, plane = p.H * p.W;
+  const float* item_px = a.frames + (size_t)f * p.frame_px + (size_t)pn0 * plane;
+  auto spill_at = [&](uint32_t e) -> uint32_t& { return s.thr_spill[(size_t)blockIdx.x * kThrSpill + e]; };
+  const uint32_t cnt = v.ctl[CTL_THR];
+  float* nb = v.nb + warp * sh.side * sh.side;
+  auto test = [&](uint32_t lp) {  // lp: pixel index within the item
+    const uint32_t pj = lp / plane, rem = lp - pj * plane;
+    const uint32_t r = rem / p.W, c = rem - r * p.W;
+    auto ld = [](const float* q) { return __ldg(q); };
+    const float* pan = item_px + (size_t)pj * plane;
+    if (warp_peak_test(pan, p.H, p.W, r, c, p, nb, ld) && lane == 0) add_peak(p, a, peak_n, f, pn0 * plane + lp);
+  };
+  // a listed pixel is tested; a listed 2x4 block is screened first (a pixel
+  // beaten inside its own block, which lies inside its window, by the
+  // local-maximum rule can never be a candidate)
+  auto test_listed = [&](uint32_t listed) {
+    if (!(listed & kBlockKey)) {
+      test(listed);
+      return;
+    }
+    const uint32_t key = listed & ~kBlockKey, pj = key / plane, rem = key - pj * plane;
+    const uint32_t r0 = rem / p.W;
+    const uint32_t npx = r0 + 1 < p.H ? 8u : 4u;
+    const uint32_t me = lane & 7u;
+    const float x = me < npx ? __ldg(item_px + key + (me >> 2) * p.W + (me & 3u)) : 0.0f;
+    bool keep = lane < npx && x >= p.amax;
+#pragma unroll
+    for (uint32_t q = 0; q < 8; ++q) {
+      const float y = __shfl_sync(0xffffffffu, x, q);
+      const int dc = (int)(q & 3u) - (int)(me & 3u);
+      if (q == me || q >= npx || dc > p.rank || -dc > p.rank) continue;
+      if (q < me ? !(x > y) : !(x >= y)) keep = false;
+    }
+    uint32_t m = __ballot_sync(0xffffffffu, keep);
+    while (m) {
+      const uint32_t l = __ffs(m) - 1;
+      m &= m - 1;
+      test(key + (l >> 2) * p.W + (l & 3u));
+    }
+  };
+  // more candidates than this: lane per candidate, band by band, where a band
+  // fits; else every pixel of the item again
+  if (cnt <= (dense ? min(kThrLocalCap, sh.list_max) : sh.list_max)) {
+    // a listed candidate beaten by another candidate of the shared list
+    // inside its window (larger, or equal and earlier in row-major order)
+    // fails the local-maximum rule; the others are tested in full
+    const uint32_t cnt_local = min(cnt, kThrLocalCap);
+    if (tid == 0) v.ctl[CTL_NCAND] = 0;
+    // each listed pixel's (panel, row, col), decoded once, in the per-warp
+    // neighbourhood buffers (unused until the tests): the pairwise pass below
+    // then compares without dividing
+    uint32_t* pos = reinterpret_cast<uint32_t*>(v.nb);
+    const bool decoded = (uint64_t)kPW * sh.side * sh.side >= 2ull * cnt_local;
+    if (decoded)
+      for (uint32_t e = tid; e < cnt_local; e += kPT) {
+        const uint32_t key = v.thr[e], pj = key / plane, rem = key - pj * plane, r = rem / p.W;
+        pos[2 * e] = (key & kBlockKey) ? 0xFFFFFFFFu : pj;
+        pos[2 * e + 1] = (r << 16) | (rem - r * p.W);
+      }
+    __syncthreads();
+    // a warp per listed pixel, its lanes over the others (a thread per pixel
+    // walking the whole list ran 3.7 us an item, a chain of shared loads)
+    for (uint32_t e = warp; e < cnt_local; e += kPW) {
+      const uint32_t key = v.thr[e];
+      bool keep = true;
+      if (!(key & kBlockKey)) {
+        const float x = v.thrv[e];
+        keep = x >= p.amax;
+        uint32_t pj, r, c;
+        if (decoded) {
+          pj = pos[2 * e];
+          r = pos[2 * e + 1] >> 16;
+          c = pos[2 * e + 1] & 0xFFFFu;
+        } else {
+          pj = key / plane;
+          const uint32_t rem = key - pj * plane;
+          r = rem / p.W;
+          c = rem - r * p.W;
+        }
+        bool beaten = false;
+        for (uint32_t o = lane; keep && o < cnt_local; o += 32) {
+          if (o == e) continue;
+          uint32_t pj2, r2, c2;
+          if (decoded) {
+            pj2 = pos[2 * o];  // a listed block: no panel matches
+            r2 = pos[2 * o + 1] >> 16;
+            c2 = pos[2 * o + 1] & 0xFFFFu;
+          } else {
+            const uint32_t k2 = v.thr[o];
+            if (k2 & kBlockKey) continue;  // a listed block
+            pj2 = k2 / plane;
+            const uint32_t rem2 = k2 - pj2 * plane;
+            r2 = rem2 / p.W;
+            c2 = rem2 - r2 * p.W;
+          }
+          if (pj2 != pj) continue;  // another panel, or a listed block
+          const int dr = (int)r2 - (int)r, dc = (int)c2 - (int)c;
+          if (dr > p.rank || -dr > p.rank || dc > p.rank || -dc > p.rank) continue;
+          const float y = v.thrv[o];
+          if (y > x || (y == x && v.thr[o] < key)) beaten = true;
+        }
+        keep = keep && !__any_sync(0xffffffffu, beaten);
+      }
+      if (keep && lane == 0) v.cand[atomicAdd(v.ctl + CTL_NCAND, 1u)] = key;
+    }
+    __syncthreads();
+    const uint32_t n_cand = v.ctl[CTL_NCAND];
+    for (uint32_t e = warp; e < n_cand; e += kPW) test_listed(v.cand[e]);
+    // the spilled candidates (written before the barriers above)
+    for (uint32_t e = warp; e < cnt - cnt_local; e += kPW) test_listed(spill_at(e));
+  } else {
+    const uint32_t band_rows = dense ? sh.band_rows_dense : sh.band_rows;
+    if (band_rows) {
+      dense_band_peaks(p, a, sh, peak_n, f, pn0, kp, row0, row1, band_rows);
+    } else if (dense) {
+      // a panel too wide for a band of rows in shared memory, many candidates: the
+      // warp gathers the pixels >= amax_thr of its slices, 32 at a time, and each
+      // lane runs the local-maximum rule and the evaluation on its own candidate
+      // in the sequential order the warp tests reproduce (is_local_max_at,
+      // evaluate_peak_at), so a warp instruction serves 32 candidates
+      uint32_t mine = 0, nq = 0;  // nq: candidates held by lanes 0 .. nq - 1 (the same in every lane)
+      auto flush = [&]() {
+        if (lane < nq) {
+          const uint32_t pj = mine / plane, rem = mine - pj * plane;
+          const int r = (int)(rem / p.W), c = (int)(rem - (uint32_t)r * p.W);
+          const float* pan = item_px + (size_t)pj * plane;
+          auto px = [&](int dr, int dc) { return __ldg(pan + (size_t)(r + dr) * p.W + (c + dc)); };
+          if (is_local_max_at(px, (int)p.H, (int)p.W, r, c, p) && evaluate_peak_at(px, (int)p.H, (int)p.W, r, c, p))
+            add_peak(p, a, peak_n, f, pn0 * plane + mine);
+        }
+        __syncwarp();
+        nq = 0;
+      };
+      for (uint32_t pj = 0; pj < kp; ++pj) {
+        const uint32_t end = pj * plane + row1 * p.W;
+        for (uint32_t base = pj * plane + row0 * p.W + warp * 32; base < end; base += kPW * 32) {
+          const uint32_t lp = base + lane;
+          const bool hot = lp < end && __ldg(item_px + lp) >= p.amax;
+          uint32_t m = __ballot_sync(0xffffffffu, hot);
+          while (m) {
+            // the first `take` hot lanes hand their pixels to lanes nq .. nq + take - 1
+            // through the warp's 32 slots of the candidate list (unused on this path)
+            static_assert(kThrLocalCap >= kPW * 32, "32 candidate slots per warp");
+            uint32_t* q = v.cand + warp * 32;
+            const uint32_t take = min((uint32_t)__popc(m), 32u - nq);
+            const uint32_t k = __popc(m & lanemask_lt());
+            const bool go = ((m >> lane) & 1u) && k < take;
+            if (go) q[nq + k] = base + lane;
+            m &= ~__ballot_sync(0xffffffffu, go);
+            __syncwarp();
+            if (lane >= nq && lane < nq + take) mine = q[lane];
+            __syncwarp();
+            nq += take;
+            if (nq == 32) flush();
+          }
+        }
+      }
+      if (nq) flush();
+    } else {
+      // every pixel >= amax_thr of the item, one warp test each
+      for (uint32_t pj = 0; pj < kp; ++pj) {
+        const uint32_t end = pj * plane + row1 * p.W;
+        for (uint32_t base = pj * plane + row0 * p.W + warp * 32; base < end; base += kPW * 32) {
+          const uint32_t lp = base + lane;
+          const bool hot = lp < end && __ldg(item_px + lp) >= p.amax;
+          uint32_t m = __ballot_sync(0xffffffffu, hot);
+          while (m) {
+            const uint32_t l = __ffs(m) - 1;
+            m &= m - 1;
+            test(base + l);
+          }
+        }
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
-// One streaming item: panels pn0 .. pn0 + kp - 1 of frame f, side by side.
+// One streaming item: binned rows [ib, ie) of panels pn0 .. pn0 + kp - 1 of frame
+// f, side by side (all rows, or one of the row bands that small batches are cut
+// into so that every CTA has work).
 //
 // A consumer lane owns float4 columns of the item (two bins per binned row),
 // one per column group, and walks down the rows.  The q values of the row
@@ -309,31 +558,31 @@ __device__ __noinline__ void dense_band_peaks(const DevParams& p, const Scratch&
 // shared memory.  A step covers RB binned rows: phase A bins and
 // prequantises them into registers, one barrier (it also frees the ring
 // slot), then phase B forms the Lorenzo residuals, code bytes and histogram.
-// kRt: the dense-peaks choice is read from sh.dense at run time instead of
-// kDense (one copy of the code for both, as the multi-job kernel wants).
-template <int RB, bool kDense, int kG, bool kRt = false>
+// kBand: the launch cuts panels into row bands (else the band is the whole panel,
+// known to the compiler: the loop of large batches measured 2% faster so).
+template <int RB, int kG, bool kBand>
 __device__ void process_item(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
-                             unsigned char* sm, uint32_t f, uint32_t u, uint32_t& ring_iter) {
+                             unsigned char* sm, uint32_t f, uint32_t u, const SyncWords& sw, uint32_t& ring_iter) {
   const StreamView v = stream_view(sm, sh);
-  const bool dense = kRt ? sh.dense != 0 : kDense;
   // input rows: evict-first (or normal) in L2; code bytes: evict-last until packed
   const uint64_t pol = sh.input_evict_first ? evict_first_policy() : evict_normal_policy();
   const uint64_t keep_pol = evict_last_policy();
   const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
   const uint32_t NP = p.W >> 2, Mp = p.Hb * p.Wb, plane = p.H * p.W;
-  const uint32_t pn0 = u * sh.k, kp = min(sh.k, p.P - pn0);
+  const uint32_t bands = kBand ? sh.bands : 1u, grp = u / bands, band = u - grp * bands;
+  const uint32_t pn0 = grp * sh.k, kp = min(sh.k, p.P - pn0);
+  const uint32_t ib = kBand ? band * sh.band_bins : 0u, ie = kBand ? min(p.Hb, ib + sh.band_bins) : p.Hb;
   // lane l >= 1 of warp w owns float4 column 217 g + 31 w + l - 1 of the item
   // in each column group g; lane 0 recomputes the column before (the previous
   // warp's last) for its left neighbour, so warps never wait for one another
   const uint32_t C = kp * NP;
   const float* item_px = a.frames + (size_t)f * p.frame_px + (size_t)pn0 * plane;
   const uint32_t slot_floats = 2 * RB * p.W;  // one panel's rows in a ring slot
-  const size_t fu = (size_t)f * p.P + u;
   uint64_t* full_bar = v.bars;                 // [stages] rows landed (TMA transaction count)
   uint64_t* empty_bar = v.bars + sh.stages;    // [stages] every consumer warp is done with the slot
 
-  uint64_t* trace = (a.trace && f < a.trace_frames && tid == 0)
-                       ? a.trace + (size_t)a.trace_frames * kTracePoints + fu * 4
+  uint64_t* trace = (a.trace && f < a.trace_frames && u < p.P && tid == 0)
+                       ? a.trace + (size_t)a.trace_frames * kTracePoints + ((size_t)f * p.P + u) * 4
                        : nullptr;
   if (trace) trace[0] = global_ns();
   for (uint32_t k = tid; k < p.nsym; k += kPT) v.hist[k] = 0;
@@ -343,14 +592,13 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
     v.ctl[CTL_PQN] = 0;
   }
   if (tid < kMaxK) v.ctl[CTL_PQ + tid] = 0;
-  if (a.user_peaks && tid == 0) s.peak_part_count[fu] = 0;
   __syncthreads();  // hist, masks and counters are zero
 
-  const uint32_t n_steps = ceil_div(p.Hb, (uint32_t)RB);
+  const uint32_t n_steps = ceil_div(ie - ib, (uint32_t)RB);
   const bool find = a.user_peaks == nullptr;
   // candidates past the shared list go to the CTA's list in global memory
   // (the dense-peaks variant tests such items band by band instead)
-  const bool spills = !dense && blockIdx.x < s.thr_spill_ctas;
+  const bool spills = sh.dense == 0;  // the launch has a spill list for each of its CTAs
   auto spill_at = [&](uint32_t e) -> uint32_t& { return s.thr_spill[(size_t)blockIdx.x * kThrSpill + e]; };
   bool timed_out = false;
   uint32_t slot = ring_iter % sh.stages, phase = (ring_iter / sh.stages) & 1u;
@@ -361,12 +609,12 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
     }
   };
   if (warp == kProducerWarp) {
-    // producer: step st = raw rows [2 st RB, min(H, 2 (st + 1) RB)) of each
-    // panel, one bulk copy per panel, once every consumer has left the slot
+    // producer: step st = raw rows [2 (ib + st RB), 2 (ib + (st + 1) RB)) of each
+    // panel (up to the band's and the panel's end), one bulk copy per panel, once every consumer has left the slot
     if (lane == 0) {
       for (uint32_t st = 0; st < n_steps; ++st) {
         if (!mbar_wait(empty_bar + slot, phase ^ 1u)) timed_out = true;
-        const uint32_t r0 = 2 * st * RB, r1 = min(p.H, 2 * (st + 1) * RB);
+        const uint32_t r0 = 2 * (ib + st * RB), r1 = min(p.H, 2 * min(ie, ib + (st + 1) * RB));
         const uint32_t bytes = (r1 - r0) * p.W * 4;
         float* dst = reinterpret_cast<float*>(v.ring + (size_t)slot * sh.stage_bytes);
         fence_proxy_async();
@@ -389,7 +637,7 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
     struct Col {
       bool owned, first;
       uint32_t pi, pc;
-      uint8_t* codes;      // the column's code bytes in binned row 0
+      uint8_t* codes;      // the column's code bytes in the step's first binned row
       uint16_t* esc;       // the lane's panel: escape codes, Lorenzo-outlier deltas and
       int32_t* lo_delta;   // prequantisation-outlier bits, at their bin
       uint32_t* pq_bits;
@@ -408,12 +656,20 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
       c.pc = gcol - c.pi * NP;
       c.first = c.pc == 0;  // the bin to the left lies outside the panel
       const size_t fbin = (size_t)f * p.M + (size_t)(pn0 + c.pi) * Mp;  // first bin of the lane's panel
-      c.codes = s.codes8 + (size_t)f * sh.codes_stride + (size_t)(pn0 + c.pi) * Mp + 2 * c.pc;
+      c.codes = s.codes8 + (size_t)f * sh.codes_stride + (size_t)(pn0 + c.pi) * Mp + (size_t)ib * p.Wb + 2 * c.pc;
       c.esc = s.codes + fbin;
       c.lo_delta = s.lo_delta + fbin;
       c.pq_bits = s.pq_bits + fbin;
       qu[g] = make_int2(0, 0);
       qd[g] = 0;
+      if (kBand && ib > 0) {  // the row above the band, from the frame (its outliers and pixels are the band's above)
+        const float4* above = reinterpret_cast<const float4*>(item_px + (size_t)c.pi * plane + (size_t)(2 * ib - 2) * p.W) + c.pc;
+        float v0, v1;
+        bin_pair(__ldg(above), __ldg(above + NP), true, v0, v1);
+        qu[g] = make_int2(prequantize(v0, p).q, prequantize(v1, p).q);
+        const int32_t from_lane = __shfl_up_sync(0xffffffffu, qu[g].y, 1);
+        qd[g] = c.first ? 0 : from_lane;
+      }
     }
 
     // One step: RB binned rows.  FULL steps have RB rows of two raw rows each
@@ -424,7 +680,7 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
     // group reads its rows (phase A) before the warp leaves the ring slot.
     auto step = [&](uint32_t st, auto full_tag) {
       constexpr bool FULL = decltype(full_tag)::value;
-      const uint32_t i0 = st * RB;
+      const uint32_t i0 = ib + st * RB;
       int2 qa[kG][RB];
 #pragma unroll
       for (int g = 0; g < kG; ++g) {
@@ -439,7 +695,7 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
         for (int ii = 0; ii < RB; ++ii) {
           const uint32_t i = i0 + ii;
           qa[g][ii] = make_int2(0, 0);
-          if (!FULL && i >= p.Hb) continue;
+          if (!FULL && i >= ie) continue;
           const bool two = FULL || 2 * i + 1 < p.H;
           const float4 va = rows[(2 * ii) * NP];
           const float4 vb = two ? rows[(2 * ii + 1) * NP] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -547,7 +803,7 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
 #pragma unroll
         for (int ii = 0; ii < RB; ++ii) {
           const uint32_t i = i0 + ii;
-          if (!FULL && i >= p.Hb) break;
+          if (!FULL && i >= ie) break;
           const int32_t left = left_of(ii);
           const int32_t d0 = qa[g][ii].x - qu[g].x - left + qd[g];
           const int32_t d1 = qa[g][ii].y - qu[g].y - qa[g][ii].x + qu[g].x;
@@ -555,7 +811,7 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
           qd[g] = left;
           nz |= (uint32_t)((d0 | d1) != 0) << ii;
           const uint32_t pair = (uint32_t)((d0 + 128) & 0xFF) | ((uint32_t)((d1 + 128) & 0xFF) << 8);
-          st_keep_u16_if(codes + (size_t)i * p.Wb, (uint16_t)pair, keep_pol,
+          st_keep_u16_if(codes + ii * p.Wb, (uint16_t)pair, keep_pol,
                          owned && RB_CHECK(s, i < p.Hb && 2 * pc + 1 < p.Wb, ROIBIN_CHECK_CODES));  // 2 pc is even
         }
         if (!owned) nz = 0;
@@ -565,7 +821,7 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
 #pragma unroll
           for (int ii = 0; ii < RB; ++ii) {
             const uint32_t i = i0 + ii;
-            if (!FULL && i >= p.Hb) break;
+            if (!FULL && i >= ie) break;
             const int32_t left = left_of(ii);
             const int32_t d0 = qa[g][ii].x - qu_r.x - left + qd_r;
             const int32_t d1 = qa[g][ii].y - qu_r.y - qa[g][ii].x + qu_r.x;
@@ -591,19 +847,24 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
               };
               const uint32_t b0 = to_byte(d0, c0, lb), b1 = to_byte(d1, c1, lb + 1);
               if (b0 != (uint32_t)((d0 + 128) & 0xFF) || b1 != (uint32_t)((d1 + 128) & 0xFF))
-                st_keep_u16_if(codes + (size_t)i * p.Wb, (uint16_t)(b0 | (b1 << 8)), keep_pol, true);
+                st_keep_u16_if(codes + ii * p.Wb, (uint16_t)(b0 | (b1 << 8)), keep_pol, true);
             }
             hist_add_warp(v.hist, c0 != (uint32_t)p.R ? c0 : 0xFFFFu, 0xFFFFFFFFu);
             hist_add_warp(v.hist, c1 != (uint32_t)p.R ? c1 : 0xFFFFu, 0xFFFFFFFFu);
           }
         }
+        cols[g].codes += RB * p.Wb;
       }
     };
-    for (uint32_t st = 0; st < n_steps; ++st) {
+    // whole steps first, then the one that may end early (the band's or the panel's end)
+    const uint32_t n_full = (min(ie, p.H >> 1) - ib) / RB;
+    for (uint32_t st = 0; st < n_full; ++st) {
       if (!mbar_wait(full_bar + slot, phase)) timed_out = true;
-      const uint32_t i_end = (st + 1) * RB;
-      if (i_end <= p.Hb && 2 * i_end <= p.H) step(st, std::integral_constant<bool, true>{});
-      else step(st, std::integral_constant<bool, false>{});
+      step(st, std::integral_constant<bool, true>{});
+    }
+    for (uint32_t st = n_full; st < n_steps; ++st) {
+      if (!mbar_wait(full_bar + slot, phase)) timed_out = true;
+      step(st, std::integral_constant<bool, false>{});
     }
   }
   if (timed_out) v.ctl[CTL_TIMEOUT] = 1;
@@ -638,32 +899,41 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
     for (int d = 16; d > 0; d >>= 1) part += __shfl_xor_sync(0xffffffffu, part, d);
     if (lane == 0 && part) atomicAdd(v.ctl + CTL_NZ, part);
     __syncthreads();
-    if (tid == 0) v.hist[p.R] = kp * Mp - v.ctl[CTL_NZ];
+    if (tid == 0) v.hist[p.R] = kp * (ie - ib) * p.Wb - v.ctl[CTL_NZ];
     __syncthreads();
   }
   if (trace) trace[1] = global_ns();
-  // flush the item's histogram and its panels' outlier bits (disjoint slots)
-  for (uint32_t k = tid; k < p.nsym; k += kPT) s.hist_part[fu * kMaxSymbols + k] = v.hist[k];
+  // flush the item's histogram (the codes it has seen; the 3-D predictor counts
+  // its own later) and its panels' outlier bits (a slot per panel and band)
+  if (p.dims == 2)
+    for (uint32_t k = tid; k < p.nsym; k += kPT)
+      if (v.hist[k]) atomicAdd(s.hist_f + (size_t)f * kMaxSymbols + k, v.hist[k]);
   const uint32_t n_pq_item = v.ctl[CTL_PQN];
+  uint32_t* slots = s.pq_mask + (((size_t)f * p.P + pn0) * bands + band) * sh.mask_words;  // panel pn0's
+  const size_t slot_step = (size_t)bands * sh.mask_words;                                     // to the next panel's
   for (uint32_t j = 0; j < kp; ++j) {
     const uint32_t n_pq = v.ctl[CTL_PQ + j];
-    const size_t fp = (size_t)f * p.P + pn0 + j;
-    if (n_pq)  // the panel's bitmask, set below
-      for (uint32_t k = tid; k < sh.mask_words; k += kPT) s.pq_mask[fp * sh.mask_words + k] = 0;
-    if (tid == 0) s.pq_part_count[fp] = n_pq;
+    if (n_pq)  // the slot's bitmask, set below
+      for (uint32_t k = 1 + tid; k < sh.mask_words; k += kPT) slots[j * slot_step + k] = 0;
+    if (tid == 0) slots[j * slot_step] = n_pq;
   }
   if (n_pq_item) {
+    if (tid == 0) atomicAdd(sw.pq_n + f, n_pq_item);
     __syncthreads();  // the masks are zero
-    uint32_t* gmask = s.pq_mask + ((size_t)f * p.P + pn0) * sh.mask_words;
+    auto set_bit = [&](uint32_t pj, uint32_t lb) {
+      const uint32_t b = lb - ib * p.Wb;
+      atomicOr(slots + pj * slot_step + 1 + (b >> 5), 1u << (b & 31));
+    };
     if (n_pq_item <= kPqList) {
       for (uint32_t e = tid; e < n_pq_item; e += kPT) {
-        const uint32_t b = v.pql[e], pj = b / Mp, lb = b - pj * Mp;
-        atomicOr(gmask + pj * sh.mask_words + (lb >> 5), 1u << (lb & 31));
+        const uint32_t b = v.pql[e], pj = b / Mp;
+        set_bit(pj, b - pj * Mp);
       }
     } else {
       // more outliers than the list holds: find them again from the input
-      for (uint32_t b = tid; b < kp * Mp; b += kPT) {
-        const uint32_t pj = b / Mp, lb = b - pj * Mp, i = lb / p.Wb, jb = lb - i * p.Wb;
+      const uint32_t n_bins = (ie - ib) * p.Wb;
+      for (uint32_t b = tid; b < kp * n_bins; b += kPT) {
+        const uint32_t pj = b / n_bins, lb = ib * p.Wb + (b - pj * n_bins), i = lb / p.Wb, jb = lb - i * p.Wb;
         const float* px = item_px + (size_t)pj * plane + (size_t)(2 * i) * p.W + 2 * jb;
         const bool two = 2 * i + 1 < p.H;
         const float4 va = make_float4(__ldg(px), __ldg(px + 1), 0.f, 0.f);
@@ -671,229 +941,19 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
                               : make_float4(0.f, 0.f, 0.f, 0.f);
         float v0, v1;
         bin_pair(va, vb, two, v0, v1);
-        if (prequantize(v0, p).outlier) atomicOr(gmask + pj * sh.mask_words + (lb >> 5), 1u << (lb & 31));
+        if (prequantize(v0, p).outlier) set_bit(pj, lb);
       }
     }
   }
 
-  // a1 + a2 on the listed blocks (on every pixel >= amax_thr if the list overflowed)
+  // a1 + a2 on the listed blocks
   if (find) {
-    if (tid == 0) v.ctl[CTL_ACC] = 0;
     __syncthreads();
-    const uint32_t cnt = v.ctl[CTL_THR];
-    float* nb = v.nb + warp * sh.side * sh.side;
-    auto test = [&](uint32_t lp) {  // lp: pixel index within the item
-      const uint32_t pj = lp / plane, rem = lp - pj * plane;
-      const uint32_t r = rem / p.W, c = rem - r * p.W;
-      auto ld = [](const float* q) { return __ldg(q); };
-      const float* pan = item_px + (size_t)pj * plane;
-      const bool hit = kRt ? (dense ? warp_peak_test<true>(pan, p.H, p.W, r, c, p, nb, ld)
-                                    : warp_peak_test<false>(pan, p.H, p.W, r, c, p, nb, ld))
-                           : warp_peak_test<kDense>(pan, p.H, p.W, r, c, p, nb, ld);
-      if (hit && lane == 0) {
-        const uint32_t slot = atomicAdd(v.ctl + CTL_ACC, 1u);
-        if (slot < sh.sort_n2) v.acc[slot] = lp;
-      }
-    };
-    // a listed pixel is tested; a listed 2x4 block is screened first (a pixel
-    // beaten inside its own block, which lies inside its window, by the
-    // local-maximum rule can never be a candidate)
-    auto test_listed = [&](uint32_t listed) {
-      if (!(listed & kBlockKey)) {
-        test(listed);
-        return;
-      }
-      const uint32_t key = listed & ~kBlockKey, pj = key / plane, rem = key - pj * plane;
-      const uint32_t r0 = rem / p.W;
-      const uint32_t npx = r0 + 1 < p.H ? 8u : 4u;
-      const uint32_t me = lane & 7u;
-      const float x = me < npx ? __ldg(item_px + key + (me >> 2) * p.W + (me & 3u)) : 0.0f;
-      bool keep = lane < npx && x >= p.amax;
-#pragma unroll
-      for (uint32_t q = 0; q < 8; ++q) {
-        const float y = __shfl_sync(0xffffffffu, x, q);
-        const int dc = (int)(q & 3u) - (int)(me & 3u);
-        if (q == me || q >= npx || dc > p.rank || -dc > p.rank) continue;
-        if (q < me ? !(x > y) : !(x >= y)) keep = false;
-      }
-      uint32_t m = __ballot_sync(0xffffffffu, keep);
-      while (m) {
-        const uint32_t l = __ffs(m) - 1;
-        m &= m - 1;
-        test(key + (l >> 2) * p.W + (l & 3u));
-      }
-    };
-    if (cnt <= kThrLocalCap + (spills ? kThrSpill : 0u)) {
-      // a listed candidate beaten by another candidate of the shared list
-      // inside its window (larger, or equal and earlier in row-major order)
-      // fails the local-maximum rule; the others are tested in full
-      const uint32_t cnt_local = min(cnt, kThrLocalCap);
-      if (tid == 0) v.ctl[CTL_NCAND] = 0;
-      // each listed pixel's (panel, row, col), decoded once, in the per-warp
-      // neighbourhood buffers (unused until the tests): the pairwise pass below
-      // then compares without dividing
-      uint32_t* pos = reinterpret_cast<uint32_t*>(v.nb);
-      const bool decoded = (uint64_t)kPW * sh.side * sh.side >= 2ull * cnt_local;
-      if (decoded)
-        for (uint32_t e = tid; e < cnt_local; e += kPT) {
-          const uint32_t key = v.thr[e], pj = key / plane, rem = key - pj * plane, r = rem / p.W;
-          pos[2 * e] = (key & kBlockKey) ? 0xFFFFFFFFu : pj;
-          pos[2 * e + 1] = (r << 16) | (rem - r * p.W);
-        }
-      __syncthreads();
-      // a warp per listed pixel, its lanes over the others (a thread per pixel
-      // walking the whole list ran 3.7 us an item, a chain of shared loads)
-      for (uint32_t e = warp; e < cnt_local; e += kPW) {
-        const uint32_t key = v.thr[e];
-        bool keep = true;
-        if (!(key & kBlockKey)) {
-          const float x = v.thrv[e];
-          keep = x >= p.amax;
-          uint32_t pj, r, c;
-          if (decoded) {
-            pj = pos[2 * e];
-            r = pos[2 * e + 1] >> 16;
-            c = pos[2 * e + 1] & 0xFFFFu;
-          } else {
-            pj = key / plane;
-            const uint32_t rem = key - pj * plane;
-            r = rem / p.W;
-            c = rem - r * p.W;
-          }
-          bool beaten = false;
-          for (uint32_t o = lane; keep && o < cnt_local; o += 32) {
-            if (o == e) continue;
-            uint32_t pj2, r2, c2;
-            if (decoded) {
-              pj2 = pos[2 * o];  // a listed block: no panel matches
-              r2 = pos[2 * o + 1] >> 16;
-              c2 = pos[2 * o + 1] & 0xFFFFu;
-            } else {
-              const uint32_t k2 = v.thr[o];
-              if (k2 & kBlockKey) continue;  // a listed block
-              pj2 = k2 / plane;
-              const uint32_t rem2 = k2 - pj2 * plane;
-              r2 = rem2 / p.W;
-              c2 = rem2 - r2 * p.W;
-            }
-            if (pj2 != pj) continue;  // another panel, or a listed block
-            const int dr = (int)r2 - (int)r, dc = (int)c2 - (int)c;
-            if (dr > p.rank || -dr > p.rank || dc > p.rank || -dc > p.rank) continue;
-            const float y = v.thrv[o];
-            if (y > x || (y == x && v.thr[o] < key)) beaten = true;
-          }
-          keep = keep && !__any_sync(0xffffffffu, beaten);
-        }
-        if (keep && lane == 0) v.cand[atomicAdd(v.ctl + CTL_NCAND, 1u)] = key;
-      }
-      __syncthreads();
-      const uint32_t n_cand = v.ctl[CTL_NCAND];
-      for (uint32_t e = warp; e < n_cand; e += kPW) test_listed(v.cand[e]);
-      // the spilled candidates (written before the barriers above)
-      for (uint32_t e = warp; e < cnt - cnt_local; e += kPW) test_listed(spill_at(e));
-    } else {
-      // every pixel >= amax_thr of the item, one warp test each
-      auto scan_all = [&]() {
-        const uint32_t n_px = kp * plane;
-        for (uint32_t base = warp * 32; base < n_px; base += kPW * 32) {
-          const uint32_t lp = base + lane;
-          const bool hot = lp < n_px && __ldg(item_px + lp) >= p.amax;
-          uint32_t m = __ballot_sync(0xffffffffu, hot);
-          while (m) {
-            const uint32_t l = __ffs(m) - 1;
-            m &= m - 1;
-            test(base + l);
-          }
-        }
-
-      };
-      if constexpr (kDense || kRt) {
-        if (dense) {
-          if (sh.band_rows >= 2u * (uint32_t)peak_reach(p) + 2u) {
-            dense_band_peaks(p, s, sh, v, item_px, kp, fu);
-          } else {
-          // many candidates (hot pixels): one lane per candidate.  The warp gathers
-          // the pixels >= amax_thr of its slices, 32 at a time, and each lane runs
-          // the local-maximum rule and the evaluation on its own candidate in the
-          // sequential order the warp tests reproduce (is_local_max_at,
-          // evaluate_peak_at), so a warp instruction serves 32 candidates
-          const uint32_t n_px = kp * plane;
-          uint32_t mine = 0, nq = 0;  // nq: candidates held by lanes 0 .. nq - 1 (the same in every lane)
-          auto flush = [&]() {
-            if (lane < nq) {
-              const uint32_t pj = mine / plane, rem = mine - pj * plane;
-              const int r = (int)(rem / p.W), c = (int)(rem - (uint32_t)r * p.W);
-              const float* pan = item_px + (size_t)pj * plane;
-              auto px = [&](int dr, int dc) { return __ldg(pan + (size_t)(r + dr) * p.W + (c + dc)); };
-              if (is_local_max_at(px, (int)p.H, (int)p.W, r, c, p) && evaluate_peak_at(px, (int)p.H, (int)p.W, r, c, p)) {
-                const uint32_t slot = atomicAdd(v.ctl + CTL_ACC, 1u);
-                if (slot < sh.sort_n2) v.acc[slot] = mine;
-              }
-            }
-            __syncwarp();
-            nq = 0;
-          };
-          for (uint32_t base = warp * 32; base < n_px; base += kPW * 32) {
-            const uint32_t lp = base + lane;
-            const bool hot = lp < n_px && __ldg(item_px + lp) >= p.amax;
-            uint32_t m = __ballot_sync(0xffffffffu, hot);
-            while (m) {
-              // the first `take` hot lanes hand their pixels to lanes nq .. nq + take - 1
-              // (this fallback serves panels too wide for a band of rows in shared memory)
-              // through the warp's 32 slots of the candidate list (unused on this path)
-              static_assert(kThrLocalCap >= kPW * 32, "32 candidate slots per warp");
-              uint32_t* q = v.cand + warp * 32;
-              const uint32_t take = min((uint32_t)__popc(m), 32u - nq);
-              const uint32_t k = __popc(m & lanemask_lt());
-              const bool go = ((m >> lane) & 1u) && k < take;
-              if (go) q[nq + k] = base + lane;
-              m &= ~__ballot_sync(0xffffffffu, go);
-              __syncwarp();
-              if (lane >= nq && lane < nq + take) mine = q[lane];
-              __syncwarp();
-              nq += take;
-              if (nq == 32) flush();
-            }
-          }
-          if (nq) flush();
-          }
-        } else {
-          scan_all();
-        }
-      } else {
-        scan_all();
-      }
-    }
-    __syncthreads();
-    const uint32_t n_acc = v.ctl[CTL_ACC];
-    if (n_acc <= p.max_peaks) {  // sort the item's peaks: (panel, row, col) order
-      uint32_t n2 = 1;
-      while (n2 < n_acc) n2 <<= 1;
-      for (uint32_t k = n_acc + tid; k < n2; k += kPT) v.acc[k] = 0xFFFFFFFFu;
-      __syncthreads();
-      for (uint32_t size = 2; size <= n2; size <<= 1) {
-        for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-          for (uint32_t k = tid; k < n2; k += kPT) {
-            const uint32_t partner = k ^ stride;
-            if (partner > k) {
-              const bool upw = (k & size) == 0;
-              const uint32_t x = v.acc[k], y = v.acc[partner];
-              if ((x > y) == upw) {
-                v.acc[k] = y;
-                v.acc[partner] = x;
-              }
-            }
-          }
-          __syncthreads();
-        }
-      }
-      for (uint32_t k = tid; k < n_acc; k += kPT) s.peak_part[fu * sh.peak_cap + k] = pn0 * plane + v.acc[k];
-    }
-    if (tid == 0) s.peak_part_count[fu] = n_acc;
+    item_peaks(p, s, a, sh, sm, sw.peak_n, f, pn0, kp, 2 * ib, min(p.H, 2 * ie));
   }
   __syncthreads();
   if (tid == 0 && v.ctl[CTL_TIMEOUT]) {  // a copy never arrived: the frame is marked, see frame_codebook
-    s.peak_part_count[fu] = kPanelTimedOut;
+    atomicOr(sw.fin + f, kGaveUp);
     v.ctl[CTL_TIMEOUT] = 0;
   }
   if (trace) trace[2] = global_ns();
@@ -907,36 +967,12 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
 //       the last one scans, lays the frame out and writes its head;
 //   (3) chunk-write items pack the bits, write the outliers and the ROI
 //       windows, and drop their code bytes from L2.
-// One atomic ticket counter orders all work: round r holds the panels of
-// frame r, the size items of frame r - lag1 and the write items of frame
-// r - lag1 - lag2.  Stages hand over through release/acquire flags.  A CTA only
+// One atomic ticket counter orders all work: every frame's streaming items, then
+// every frame's size items, with the write items of frame r - lag after the size
+// items of frame r.  Stages hand over through release/acquire flags.  A CTA only
 // ever waits for work handed out to an earlier ticket, which is running or
 // done, so every wait ends; waits are bounded anyway (ROIBIN_ERR_TIMEOUT).
 constexpr uint32_t kWaitLimit = 1u << 22;
-
-// Per-frame words, zeroed before each launch:
-//   panel_done, size_done   streaming / size items finished;
-//   ready_cb, ready_plan    the codebook / the plan is published;
-//   timed_out               set by any item whose flag wait gave up (sticky: no
-//                           later write of the frame's status can clear it);
-//   fin_count               the plan and the write items finished; the one that
-//                           finishes last settles the frame's status;
-//   chunk_done              (per chunk of frames) frames whose peaks are known.
-struct SyncWords {
-  uint32_t *panel_done, *size_done, *ready_cb, *ready_plan, *timed_out, *fin_count, *chunk_done, *ticket;
-};
-__device__ __forceinline__ SyncWords sync_words(const Scratch& s, uint32_t n) {
-  SyncWords w;
-  w.panel_done = s.frame_done;
-  w.size_done = s.frame_done + n;
-  w.ready_cb = s.frame_done + 2 * n;
-  w.ready_plan = s.frame_done + 3 * n;
-  w.timed_out = s.frame_done + 4 * n;
-  w.fin_count = s.frame_done + 5 * n;
-  w.chunk_done = s.frame_done + 6 * n;
-  w.ticket = s.frame_done + kSyncWordsPerFrame * n;
-  return w;
-}
 
 // Called by thread 0 of the plan and of every write item of frame g once its
 // work is visible (after a __threadfence): the last of them to finish sees
@@ -944,30 +980,30 @@ __device__ __forceinline__ SyncWords sync_words(const Scratch& s, uint32_t n) {
 // reported ROIBIN_ERR_TIMEOUT with no bytes, whatever the plan wrote before.
 __device__ __forceinline__ void finish_frame_item(const PlainArgs& a, const FusedShape& sh, const SyncWords& sw,
                                                   uint32_t g) {
-  if (atomicAdd(sw.fin_count + g, 1u) != sh.groups) return;
+  if ((atomicAdd(sw.fin + g, 1u) & ~kGaveUp) != sh.groups) return;
   __threadfence();
-  if (__ldcg(sw.timed_out + g)) {
+  if (__ldcg(sw.fin + g) & kGaveUp) {
     a.frame_status[g] = ROIBIN_ERR_TIMEOUT;
     a.frame_bytes[g] = 0;
   }
 }
 
-__device__ __forceinline__ void flag_release(uint32_t* f) {
+__device__ __forceinline__ void flag_release(uint32_t* f, uint32_t bit) {
   __threadfence();
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(f), "r"(1u) : "memory");
+  asm volatile("red.release.gpu.global.or.b32 [%0], %1;" ::"l"(f), "r"(bit) : "memory");
 }
 __device__ __forceinline__ uint32_t flag_acquire(const uint32_t* f) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
   return v;
 }
-// Thread 0 waits (bounded: `limit` polls) for a flag; every thread gets the
+// Thread 0 waits (bounded: `limit` polls) for a flag's bit; every thread gets the
 // outcome.  limit = 0 polls nothing, so the wait gives up at once.
-__device__ bool wait_flag(const uint32_t* f, uint32_t* slot, uint32_t limit) {
+__device__ bool wait_flag(const uint32_t* f, uint32_t bit, uint32_t* slot, uint32_t limit) {
   if (threadIdx.x == 0) {
     uint32_t ok = 0;
     for (uint32_t i = 0; i < limit; ++i) {
-      if (flag_acquire(f)) {
+      if (flag_acquire(f) & bit) {
         ok = 1;
         break;
       }
@@ -1035,7 +1071,7 @@ __device__ void chunk_codebook(const DevParams& p, const Scratch& s, const Plain
   }
   __syncthreads();
   if (tid == 0)
-    for (uint32_t g = c0; g < c1; ++g) flag_release(sw.ready_cb + g);
+    for (uint32_t g = c0; g < c1; ++g) flag_release(sw.stage + g, kStageCodebook);
 }
 
 // The 3-D predictor (a6 over the panel stack, §6) from the streamed 2-D
@@ -1059,8 +1095,7 @@ __device__ __noinline__ void stack_residuals(const DevParams& p, const Scratch& 
   const uint32_t Mp = p.Hb * p.Wb;  // even: the fused path has an even binned width
   const int32_t R = p.R;
   // two slice buffers in the stage, each a slice plus the 15 bytes before its first line
-  constexpr uint32_t kStage = sizeof(HuffSmem) > 4096 ? (uint32_t)sizeof(HuffSmem) : 4096u;
-  constexpr uint32_t kSlice = (kStage / 2 - 16) & ~15u;
+  constexpr uint32_t kSlice = (kHuffArea / 2 - 16) & ~15u;
   uint8_t* buf[2] = {stage, stage + kSlice + 16};
   uint32_t zeros = 0;  // codes of the zero residual this thread saw (the common code)
   auto residual = [&](uint32_t b, uint32_t bin) -> int32_t {  // the stored 2-D residual from its byte
@@ -1136,86 +1171,103 @@ __device__ __noinline__ void stack_residuals(const DevParams& p, const Scratch& 
   __syncthreads();
 }
 
+// Sorts n distinct keys of a list in global memory, through shared memory (a
+// power of two of words >= n): by counting the smaller ones up to 256 keys, else
+// bitonic.
+__device__ void sort_peaks(uint32_t* keys, uint32_t n, uint32_t* buf) {
+  const uint32_t tid = threadIdx.x;
+  uint32_t n2 = 4;
+  while (n2 < n) n2 <<= 1;
+  for (uint32_t k = tid; k < n2; k += kPT) buf[k] = k < n ? __ldcg(keys + k) : 0xFFFFFFFFu;
+  __syncthreads();
+  if (n <= kPT) {
+    if (tid < n) {
+      const uint32_t key = buf[tid];
+      uint32_t rank = 0;
+      for (uint32_t j = 0; j < n; j += 4) {
+        const uint4 q = *reinterpret_cast<const uint4*>(buf + j);
+        rank += (q.x < key) + (q.y < key) + (q.z < key) + (q.w < key);
+      }
+      keys[rank] = key;
+    }
+    return;
+  }
+  for (uint32_t size = 2; size <= n2; size <<= 1) {
+    for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+      for (uint32_t i = tid; i < n2 / 2; i += kPT) {  // i-th pair of the step
+        const uint32_t k = 2 * i - (i & (stride - 1)), q = k + stride;
+        const uint32_t x = buf[k], y = buf[q];
+        if ((x > y) == ((k & size) == 0)) {
+          buf[k] = y;
+          buf[q] = x;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  for (uint32_t k = tid; k < n; k += kPT) keys[k] = buf[k];
+}
+
 // (1) peak list + codebook of frame f, by the CTA that completed its last streaming item.
 __device__ void frame_codebook(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
                                unsigned char* sm, uint32_t f, const SyncWords& sw) {
   const FinView v = fin_view(sm, sh);
-  const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+  const uint32_t tid = threadIdx.x;
   uint64_t* trace = (a.trace && f < a.trace_frames && tid == 0) ? a.trace + (size_t)f * kTracePoints : nullptr;
   if (trace) trace[0] = global_ns();
-  // a8: the frame's histogram; prequantisation outliers in the frame
-  if (p.dims == 3) {
-    stack_residuals(p, s, sh, v.total, sm + sh.off_huff, f);
-  } else {
-    for (uint32_t k = tid; k < p.nsym; k += kPT) {
-      uint32_t t = 0;
-      for (uint32_t u = 0; u < sh.U; ++u) t += __ldcg(s.hist_part + ((size_t)f * p.P + u) * kMaxSymbols + k);
-      v.total[k] = t;
-    }
-  }
   if (tid == 0) {
-    uint32_t t = 0;
-    for (uint32_t pn = 0; pn < p.P; ++pn) t += __ldcg(s.pq_part_count + (size_t)f * p.P + pn);
-    s.plan[f].n_pq = t;  // provisional: read by the size items to skip the outlier bits
+    s.plan[f].n_pq = __ldcg(sw.pq_n + f);  // provisional: read by the size items to skip the outlier bits
     v.ctl[CTL_STATUS] = ROIBIN_OK;
     v.ctl[CTL_BAD] = 0;
-    v.ctl[CTL_CARRY0] = 0;
   }
   __syncthreads();
-  // the peak list: per-item sorted lists concatenated in item (= panel) order, or the user's
+  // the peak list: the items' accepted peaks sorted by (panel, row, col), or the user's
   uint32_t* keys = a.peaks_key_out + (size_t)f * p.max_peaks;
+  uint32_t n_peaks;
   if (a.user_peaks) {
-    const uint32_t n = a.user_npeaks[f];
-    if (tid == 0) {
-      v.ctl[CTL_CARRY0] = n;
-      for (uint32_t u = 0; u < sh.U; ++u)
-        if (__ldcg(s.peak_part_count + (size_t)f * p.P + u) == kPanelTimedOut)
-          v.ctl[CTL_BAD] = 2;
-    }
-    if (n > p.max_peaks) {
+    n_peaks = a.user_npeaks[f];
+    if (n_peaks > p.max_peaks) {
       if (tid == 0) v.ctl[CTL_STATUS] = (uint32_t)ROIBIN_ERR_CAPACITY;
     } else {
       const uint16_t* up = a.user_peaks + (size_t)f * p.max_peaks * 3;
-      for (uint32_t k = tid; k < n; k += kPT) {
+      for (uint32_t k = tid; k < n_peaks; k += kPT) {
         const uint32_t pn = up[3 * k], r = up[3 * k + 1], c = up[3 * k + 2];
         if (pn >= p.P || r >= p.H || c >= p.W) v.ctl[CTL_BAD] = 1;
         else keys[k] = (pn * p.H + r) * p.W + c;
       }
     }
   } else {
-    if (tid == 0) {
-      uint32_t n = 0;
-      bool over = false;
-      bool timeout = false;
-      for (uint32_t u = 0; u < sh.U; ++u) {
-        const uint32_t c = __ldcg(s.peak_part_count + (size_t)f * p.P + u);
-        if (c == kPanelTimedOut) timeout = true;
-        else if (c > p.max_peaks) over = true;
-        v.offs[u] = n;
-        if (c != kPanelTimedOut) n += c;
-      }
-      if (over || n > p.max_peaks) v.ctl[CTL_STATUS] = (uint32_t)ROIBIN_ERR_CAPACITY;
-      if (timeout) v.ctl[CTL_STATUS] = (uint32_t)ROIBIN_ERR_TIMEOUT;
-      v.ctl[CTL_CARRY0] = timeout ? 0 : n;
-    }
-    __syncthreads();
-    if (v.ctl[CTL_STATUS] == ROIBIN_OK) {
-      for (uint32_t u = warp; u < sh.U; u += kPW) {
-        const uint32_t c = __ldcg(s.peak_part_count + (size_t)f * p.P + u), off = v.offs[u];
-        for (uint32_t k = lane; k < c; k += 32)
-          keys[off + k] = __ldcg(s.peak_part + ((size_t)f * p.P + u) * sh.peak_cap + k);
-      }
+    n_peaks = __ldcg(sw.peak_n + f);
+    if (n_peaks > p.max_peaks) {
+      if (tid == 0) v.ctl[CTL_STATUS] = (uint32_t)ROIBIN_ERR_CAPACITY;
+    } else {
+      sort_peaks(keys, n_peaks, reinterpret_cast<uint32_t*>(sm + sh.off_huff));
     }
   }
   __syncthreads();
   if (tid == 0) {
-    if (v.ctl[CTL_BAD] == 2) v.ctl[CTL_STATUS] = (uint32_t)ROIBIN_ERR_TIMEOUT;
-    else if (v.ctl[CTL_BAD] && v.ctl[CTL_STATUS] == ROIBIN_OK) v.ctl[CTL_STATUS] = (uint32_t)ROIBIN_ERR_INVALID_ARG;
+    if (__ldcg(sw.fin + f) & kGaveUp) {  // a streaming item's rows never arrived
+      v.ctl[CTL_STATUS] = (uint32_t)ROIBIN_ERR_TIMEOUT;
+      n_peaks = 0;
+    } else if (v.ctl[CTL_BAD] && v.ctl[CTL_STATUS] == ROIBIN_OK) {
+      v.ctl[CTL_STATUS] = (uint32_t)ROIBIN_ERR_INVALID_ARG;
+    }
     // non-hit rejection (§1, §4): too few peaks, the frame is not compressed
-    if (v.ctl[CTL_STATUS] == ROIBIN_OK && v.ctl[CTL_CARRY0] < (uint32_t)p.nhr_min)
+    if (v.ctl[CTL_STATUS] == ROIBIN_OK && n_peaks < (uint32_t)p.nhr_min)
       v.ctl[CTL_STATUS] = (uint32_t)ROIBIN_REJECTED;
-    a.peaks_count_out[f] = v.ctl[CTL_CARRY0];
+    a.peaks_count_out[f] = n_peaks;
   }
+  // a8: the frame's histogram, cleared for the next launch
+  if (p.dims == 3) {
+    stack_residuals(p, s, sh, v.total, sm + sh.off_huff, f);
+  } else {
+    uint32_t* hist = s.hist_f + (size_t)f * kMaxSymbols;
+    for (uint32_t k = tid; k < p.nsym; k += kPT) {
+      v.total[k] = __ldcg(hist + k);
+      hist[k] = 0;
+    }
+  }
+  __syncthreads();
   if (trace) trace[1] = global_ns();
   if (p.chunk > 1) {
     chunk_codebook(p, s, a, sh, sm, f, sw);
@@ -1234,7 +1286,7 @@ __device__ void frame_codebook(const DevParams& p, const Scratch& s, const Plain
   }
   __syncthreads();
   if (trace) trace[2] = global_ns();
-  if (tid == 0) flag_release(sw.ready_cb + f);
+  if (tid == 0) flag_release(sw.stage + f, kStageCodebook);
 }
 
 // Per-byte tables of a frame's codebook (byte = stored code byte):
@@ -1273,11 +1325,12 @@ __device__ __forceinline__ uint64_t symbol_entry(const DevParams& p, const Scrat
 
 __device__ __forceinline__ uint32_t pq_bit_of(const DevParams& p, const Scratch& s, const FusedShape& sh, uint32_t f,
                                               uint32_t bin) {
-  const uint32_t Mp = p.Hb * p.Wb;
-  const uint32_t pn = bin / Mp, lb = bin - pn * Mp;
-  // a panel without prequantisation outliers never wrote its mask words
-  if (__ldcg(s.pq_part_count + (size_t)f * p.P + pn) == 0) return 0u;
-  return (__ldcg(s.pq_mask + ((size_t)f * p.P + pn) * sh.mask_words + (lb >> 5)) >> (lb & 31)) & 1u;
+  const uint32_t Mp = p.Hb * p.Wb, per = sh.band_bins * p.Wb;
+  const uint32_t pn = bin / Mp, lb = bin - pn * Mp, band = lb / per, b = lb - band * per;
+  const uint32_t* slot = s.pq_mask + (((size_t)f * p.P + pn) * sh.bands + band) * sh.mask_words;
+  // a slot without prequantisation outliers never wrote its mask words
+  if (__ldcg(slot) == 0) return 0u;
+  return (__ldcg(slot + 1 + (b >> 5)) >> (b & 31)) & 1u;
 }
 
 // A warp stages one chunk's 4096 code bytes in its shared buffer with
@@ -1341,6 +1394,107 @@ __device__ __forceinline__ void lane_counts(const DevParams& p, const Scratch& s
     for (uint32_t i = s0; i < s1; ++i) npq += pq_bit_of(p, s, sh, f, i);
 }
 
+// Sparse chunks.  When the zero residual's codeword is the single bit 0 (a
+// canonical code's first), a chunk's bits are zeros but for the codewords of its
+// other symbols, so only those need work: the size item lists them, in order, and
+// the write item ORs their codewords into zeroed words.  About 82 of a CSPAD-like
+// frame's 4,096 symbols are listed.  Walking all of them twice cost 51 us of CTA
+// time per frame in the size items and 133 us in the write items; so it is 83 and
+// 40 us (1,000 frames: 2,218 -> 2,112 us).
+// The list of chunk k (position << 16 | code byte) takes the chunk's place in the
+// prequantisation-outlier bits, which such a frame does not use; lane 0's word of
+// lane_bit, 0 for a chunk walked in full, holds kSparseChunk and the list's length.
+constexpr uint32_t kSparseChunk = 1u << 31;
+constexpr uint32_t kSparseMost = 512;  // other symbols of a chunk at most
+__device__ __forceinline__ uint32_t* sparse_list(const DevParams& p, const Scratch& s, uint32_t f, uint32_t k) {
+  return s.pq_bits + (size_t)f * p.M + (size_t)k * kChunk;
+}
+__device__ __forceinline__ bool sparse_code(const uint64_t* btab) { return btab[0x80] == 1; }  // length 1, codeword 0
+
+// Lists the other symbols of a chunk staged in wbuf (lane l has symbols 128 l ..);
+// false (nothing usable written) when there are too many or their words would not
+// fit the write item's buffer.
+__device__ __forceinline__ bool size_sparse_chunk(const DevParams& p, const Scratch& s, uint32_t f, const uint64_t* btab,
+                                                  const uint32_t* wbuf, uint32_t k) {
+  const uint32_t lane = lane_id(), n = min(p.M, (k + 1) * kChunk) - k * kChunk;
+  const uint32_t* lw = wbuf + 33 * lane;
+  uint32_t m[4];  // a bit per symbol that is not the zero residual
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    m[j] = 0;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      // 0x80 in each byte that is not 0x80 (w ^ 0x80 is not 0), then two words' gathered to 8 bits, times 128
+      auto other = [](uint32_t w) { return ((((w ^ 0x80808080u) & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | ~w) & 0x80808080u; };
+      const uint32_t q = __dp4a(other(lw[8 * j + 2 * h + 1]), 0x80402010u, __dp4a(other(lw[8 * j + 2 * h]), 0x08040201u, 0u));
+      m[j] |= (q >> 7) << (8 * h);
+    }
+    const uint32_t at = 128 * lane + 32 * j;
+    if (at + 32 > n) m[j] &= at >= n ? 0u : (1u << (n - at)) - 1u;  // the frame's last chunk
+  }
+  const uint32_t mine = __popc(m[0]) + __popc(m[1]) + __popc(m[2]) + __popc(m[3]), incl = warp_incl_scan(mine);
+  const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+  if (total > kSparseMost) return false;
+  uint32_t* list = sparse_list(p, s, f, k) + (incl - mine);
+  const uint8_t* bytes = reinterpret_cast<const uint8_t*>(lw);
+  uint32_t extra = 0, nlo = 0;  // bits beyond one a symbol
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    for (uint64_t q = m[2 * h] | ((uint64_t)m[2 * h + 1] << 32); q; q &= q - 1) {
+      const uint32_t at = 64 * h + __ffsll((long long)q) - 1, byte = bytes[at], pos = 128 * lane + at;
+      extra += (uint32_t)symbol_entry(p, s, f, btab, byte, k * kChunk + pos) - 1;
+      nlo += byte == 0;
+      *list++ = (pos << 16) | byte;
+    }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    extra += __shfl_xor_sync(0xffffffffu, extra, d);
+    nlo += __shfl_xor_sync(0xffffffffu, nlo, d);
+  }
+  const uint32_t words = (n + extra + 31) / 32;
+  if (words > kStageWords) return false;
+  if (lane == 0) {
+    const size_t o = (size_t)f * p.n_chunks + k;
+    s.lane_bit[o * 32] = kSparseChunk | total;
+    s.chunk_words[o] = words;
+    s.chunk_lo[o] = nlo;
+    s.chunk_pq[o] = 0;
+  }
+  return true;
+}
+
+// Writes a listed chunk: words [w0, w0 + n_words) of the frame's bitstream and its
+// Lorenzo outliers from entry `lo` on.
+__device__ __forceinline__ void write_sparse_chunk(const DevParams& p, const Scratch& s, uint32_t f, const uint64_t* btab,
+                                                   uint32_t k, uint32_t count, uint32_t* wbuf, uint32_t* words,
+                                                   uint32_t w0, uint32_t n_words, uint2* lo_out, uint32_t lo,
+                                                   const FramePlan& pl) {
+  const uint32_t lane = lane_id();
+  for (uint32_t w = lane; w < n_words; w += 32) wbuf[w] = 0;
+  __syncwarp();
+  const uint32_t* list = sparse_list(p, s, f, k);
+  uint32_t extra = 0;  // bits beyond one a symbol, of the symbols before this round
+  for (uint32_t e0 = 0; e0 < count; e0 += 32) {
+    const bool in = e0 + lane < count;
+    const uint32_t ent = in ? __ldcg(list + e0 + lane) : 0u, byte = ent & 0xFFu, pos = ent >> 16, bin = k * kChunk + pos;
+    const uint64_t e = in ? symbol_entry(p, s, f, btab, byte, bin) : 1u;
+    const uint32_t L = (uint32_t)e, incl = warp_incl_scan(L - 1);
+    if (in) put_bits(wbuf, pos + extra + incl - (L - 1), (uint32_t)(e >> 32), L);
+    extra += __shfl_sync(0xffffffffu, incl, 31);
+    const uint32_t outliers = __ballot_sync(0xffffffffu, in && byte == 0);
+    if (in && byte == 0) {
+      const uint32_t at = lo + __popc(outliers & lanemask_lt());
+      if (RB_CHECK(s, at < pl.n_lo, ROIBIN_CHECK_OUTLIERS))
+        lo_out[at] = make_uint2(bin, (uint32_t)__ldcg(s.lo_delta + (size_t)f * p.M + bin));
+    }
+    lo += __popc(outliers);
+  }
+  __syncwarp();
+  for (uint32_t w = lane; w < n_words; w += 32)
+    if (RB_CHECK(s, w0 + w < pl.n_words, ROIBIN_CHECK_BITSTREAM)) words[w0 + w] = wbuf[w];
+  __syncwarp();
+}
+
 // (2) chunk sizes of one group of chunks of frame g.
 __device__ void size_item(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
                           unsigned char* sm, uint32_t g, uint32_t grp, const SyncWords& sw) {
@@ -1352,9 +1506,9 @@ __device__ void size_item(const DevParams& p, const Scratch& s, const PlainArgs&
                                  ? reinterpret_cast<unsigned long long*>(a.trace + (size_t)g * kTracePoints)
                                  : nullptr;
   const uint64_t t_in = acct ? global_ns() : 0;
-  const bool ready = wait_flag(sw.ready_cb + g, ctl + CTL_WAIT, sh.wait_limit);
+  const bool ready = wait_flag(sw.stage + g, kStageCodebook, ctl + CTL_WAIT, sh.wait_limit);
   if (acct) atomicAdd(acct + 7, (unsigned long long)(global_ns() - t_in));
-  if (!ready && tid == 0) atomicOr(sw.timed_out + g, 1u);
+  if (!ready && tid == 0) atomicOr(sw.fin + g, kGaveUp);
   const bool ok = ready && __ldcg(s.status + g) == ROIBIN_OK;
   if (ok) {
     load_byte_tables(p, s, g, btab, ctab);
@@ -1364,9 +1518,14 @@ __device__ void size_item(const DevParams& p, const Scratch& s, const PlainArgs&
     const uint32_t k_end = min(p.n_chunks, (grp + 1) * sh.group_chunks);
     uint32_t* wbuf = reinterpret_cast<uint32_t*>(sm + sh.off_stage) + warp * kStageWords;
     const uint64_t t_loop = acct ? global_ns() : 0;
+    const bool sparse = !any_pq && sparse_code(btab);
     for (uint32_t k = grp * sh.group_chunks + warp; k < k_end; k += kPW) {
       const uint32_t s0 = k * kChunk + lane * 128, s1 = min(p.M, s0 + 128);
       stage_chunk(codes, k, wbuf);
+      if (sparse && size_sparse_chunk(p, s, g, btab, wbuf, k)) {
+        __syncwarp();  // the buffer is free
+        continue;
+      }
       uint32_t bits, nlo, npq;
       lane_counts(p, s, sh, g, btab, ctab, wbuf, s0, s1, any_pq, bits, nlo, npq);
       __syncwarp();
@@ -1398,7 +1557,7 @@ __device__ void size_item(const DevParams& p, const Scratch& s, const PlainArgs&
   // a size item of the frame that gave up waiting for the codebook left the
   // chunk counts unfinished: the frame stops here (its give-up was published
   // before its size_done increment, which this CTA has seen)
-  int32_t st = __ldcg(sw.timed_out + g) ? ROIBIN_ERR_TIMEOUT : __ldcg(s.status + g);
+  int32_t st = (__ldcg(sw.fin + g) & kGaveUp) ? ROIBIN_ERR_TIMEOUT : __ldcg(s.status + g);
   const uint32_t ref = p.chunk > 1 ? __ldcg(s.chunk_ref + g) : 0u;  // frames back to the chunk's head
   uint32_t* cw = reinterpret_cast<uint32_t*>(sm + sh.off_cw);
   uint32_t* clo = cw + p.n_chunks;
@@ -1468,7 +1627,7 @@ __device__ void size_item(const DevParams& p, const Scratch& s, const PlainArgs&
   __syncthreads();
   if (trace) trace[4] = global_ns();
   if (tid == 0) {
-    flag_release(sw.ready_plan + g);
+    flag_release(sw.stage + g, kStagePlan);
     finish_frame_item(a, sh, sw, g);
   }
 }
@@ -1486,12 +1645,12 @@ __device__ void write_item(const DevParams& p, const Scratch& s, const PlainArgs
                                  ? reinterpret_cast<unsigned long long*>(a.trace + (size_t)g * kTracePoints)
                                  : nullptr;
   const uint64_t t_in = acct ? global_ns() : 0;
-  const bool ready = wait_flag(sw.ready_plan + g, ctl + CTL_WAIT, sh.wait_limit);
+  const bool ready = wait_flag(sw.stage + g, kStagePlan, ctl + CTL_WAIT, sh.wait_limit);
   if (acct) atomicAdd(acct + 8, (unsigned long long)(global_ns() - t_in));
-  if (!ready && tid == 0) atomicOr(sw.timed_out + g, 1u);
-  // a plan that gave up (timed_out, published before ready_plan) wrote no
+  if (!ready && tid == 0) atomicOr(sw.fin + g, kGaveUp);
+  // a plan that gave up (published before its stage bit) wrote no
   // layout for this launch: nothing of the frame is written then
-  if (ready && __ldcg(sw.timed_out + g) == 0 && __ldcg(s.status + g) == ROIBIN_OK)
+  if (ready && !(__ldcg(sw.fin + g) & kGaveUp) && __ldcg(s.status + g) == ROIBIN_OK)
     write_item_work(p, s, a, sh, sm, g, grp, acct, t_in);
   __threadfence();
   __syncthreads();
@@ -1543,6 +1702,13 @@ __device__ void write_item_work(const DevParams& p, const Scratch& s, const Plai
   for (uint32_t k = k_begin + warp; k < k_end; k += kPW) {
     const size_t o = (size_t)g * p.n_chunks + k;
     const uint32_t w0 = __ldcg(s.chunk_words + o);
+    const uint32_t listed = __ldcg(s.lane_bit + o * 32);
+    if (listed & kSparseChunk) {
+      const uint32_t w1 = k + 1 < p.n_chunks ? __ldcg(s.chunk_words + o + 1) : pl.n_words;
+      write_sparse_chunk(p, s, g, btab, k, listed & ~kSparseChunk, wbuf, words, w0, w1 - w0, lo_out,
+                         __ldcg(s.chunk_lo + o), pl);
+      continue;
+    }
     // In a full chunk every lane codes 128 symbols (>= 128 bits), so a word is
     // shared by at most two neighbouring lanes: lane l keeps its first, partial
     // word and ORs in lane l-1's last, partial word received by shuffle; every
@@ -1677,27 +1843,41 @@ __device__ void write_item_work(const DevParams& p, const Scratch& s, const Plai
 }
 
 // ---------------------------------------------------------------------------
-// One ticket t of a launch over the n frames of one geometry (the order is
-// above: round r = t / (U + 2 groups) holds the panels of frame r, the size
-// items of frame r - lag1 and the write items of frame r - lag1 - lag2).
-// Every thread of the CTA calls it; tickets past the work do nothing and
-// return false.  k_fused keeps this body inline in its own loop (the same
-// code, which compiled with fewer register spills there).
-template <bool kDense, int kG, bool kRt = false>
-__device__ __forceinline__ bool fused_ticket(const DevParams& p, const Scratch& s, const PlainArgs& a,
+// The tickets of a launch over n frames: n U streaming items (frame by frame),
+// then lag frames' size items, then rounds of a frame's size items and the write
+// items of the frame lag before it, then the last lag frames' write items.
+__host__ __device__ inline uint64_t fused_tickets(const FusedShape& sh, uint32_t n) {
+  return (uint64_t)n * (sh.U + 2 * sh.groups);
+}
+// The item of a coding ticket c (counted from the first one): frame and group;
+// true for a write item.
+__device__ __forceinline__ bool coding_item(const FusedShape& sh, uint32_t n, uint32_t c, uint32_t& g, uint32_t& grp) {
+  const uint32_t G = sh.groups, lag = sh.lag;
+  uint32_t r = c / G;  // in groups of G tickets: lag size groups, (size, write) pairs, lag write groups
+  grp = c - r * G;
+  if (r < lag) {
+    g = r;
+    return false;
+  }
+  r -= lag;
+  if (r < 2 * (n - lag)) {
+    g = (r >> 1) + ((r & 1u) ? 0u : lag);
+    return (r & 1u) != 0;
+  }
+  g = r - (n - lag);
+  return true;
+}
+// One ticket t < fused_tickets.  Every thread of the CTA calls it.  k_fused keeps
+// this body inline in its own loop (the same code, which compiled with fewer
+// register spills there).
+template <int kG>
+__device__ __forceinline__ void fused_ticket(const DevParams& p, const Scratch& s, const PlainArgs& a,
                                              const FusedShape& sh, const SyncWords& sw, unsigned char* sm,
                                              uint32_t t, uint32_t& ring_iter) {
   uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
-  const uint32_t n = a.n_frames, lag1 = sh.lag1, lag2 = lag1 + sh.lag2, round = sh.U + 2 * sh.groups;
-  const uint32_t r = t / round, j = t - r * round;
-  if (j < sh.U) {
-    if (r >= n) return false;
-    if constexpr (kRt || kG > 1) {  // RB = 2 only (the multi-job plan keeps to it)
-      process_item<2, kDense, kG, kRt>(p, s, a, sh, sm, r, j, ring_iter);
-    } else {
-      if (sh.RB == 2) process_item<2, kDense, kG>(p, s, a, sh, sm, r, j, ring_iter);
-      else process_item<3, kDense, 1>(p, s, a, sh, sm, r, j, ring_iter);
-    }
+  const uint32_t n = a.n_frames, r = t / sh.U, j = t - r * sh.U;
+  if (r < n) {
+    process_item<2, kG, false>(p, s, a, sh, sm, r, j, sw, ring_iter);  // the multi-job plan keeps to RB = 2, whole panels
     // publish the item; the CTA that completes the frame builds its codebook
     __threadfence();
     __syncthreads();
@@ -1707,19 +1887,11 @@ __device__ __forceinline__ bool fused_ticket(const DevParams& p, const Scratch& 
       __threadfence();
       frame_codebook(p, s, a, sh, sm, r, sw);
     }
-  } else if (j < sh.U + sh.groups) {
-    if (r < lag1 || r - lag1 >= n) return false;
-    size_item(p, s, a, sh, sm, r - lag1, j - sh.U, sw);
   } else {
-    if (r < lag2 || r - lag2 >= n) return false;
-    write_item(p, s, a, sh, sm, r - lag2, j - sh.U - sh.groups, sw);
+    uint32_t g, grp;
+    if (coding_item(sh, n, t - n * sh.U, g, grp)) write_item(p, s, a, sh, sm, g, grp, sw);
+    else size_item(p, s, a, sh, sm, g, grp, sw);
   }
-  return true;
-}
-
-// Tickets of one launch over n frames of this shape.
-__host__ __device__ inline uint64_t fused_tickets(const FusedShape& sh, uint32_t n) {
-  return (uint64_t)(n + sh.lag1 + sh.lag2) * (sh.U + 2 * sh.groups);
 }
 
 // The CTA's ring barriers (full: the producer's expect_tx; empty: one arrival
@@ -1747,6 +1919,49 @@ __device__ __forceinline__ uint32_t fused_next_ticket(unsigned char* sm, const F
   const uint32_t t = ctl[CTL_ITEM];
   __syncthreads();
   return t;
+}
+
+// ---------------------------------------------------------------------------
+// The persistent kernel over the frames of one geometry.
+// kG: column groups per consumer lane (FusedShape::kG; 2 only with RB = 2).
+// RB: binned rows per streaming step (FusedShape::RB).  One body per kernel: with
+// both steps in one, the register allocator spilled more.
+// kBand: panels cut into row bands (FusedShape::bands > 1; RB = 2 only).
+template <int kG, int RB, bool kBand>
+__global__ void __launch_bounds__(kPT, 4) k_fused(DevParams p, Scratch s, PlainArgs a, FusedShape sh) {
+  extern __shared__ __align__(128) unsigned char sm[];
+  uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
+  const SyncWords sw = sync_words(s, a.n_frames);
+  const uint32_t n = a.n_frames;
+  const uint64_t total = fused_tickets(sh, n);
+  fused_cta_init(sm, sh);
+  uint32_t ring_iter = 0;  // ring stages consumed so far (the same in every thread)
+  for (;;) {
+    if (threadIdx.x == 0) ctl[CTL_ITEM] = atomicAdd(sw.ticket, 1u);
+    __syncthreads();
+    const uint32_t t = ctl[CTL_ITEM];
+    __syncthreads();
+    if (t >= total) break;
+    // the body of fused_ticket
+    const uint32_t r = t / sh.U, j = t - r * sh.U;
+    if (r < n) {
+      process_item<RB, kG, kBand>(p, s, a, sh, sm, r, j, sw, ring_iter);
+      // publish the item; the CTA that completes the frame builds its codebook
+      __threadfence();
+      __syncthreads();
+      if (threadIdx.x == 0) ctl[CTL_LAST] = atomicAdd(sw.panel_done + r, 1u) == sh.U - 1 ? 1u : 0u;
+      __syncthreads();
+      if (ctl[CTL_LAST]) {
+        __threadfence();
+        frame_codebook(p, s, a, sh, sm, r, sw);
+      }
+    } else {
+      uint32_t g, grp;
+      if (coding_item(sh, n, t - n * sh.U, g, grp)) write_item(p, s, a, sh, sm, g, grp, sw);
+      else size_item(p, s, a, sh, sm, g, grp, sw);
+    }
+    __syncthreads();
+  }
 }
 
 }  // namespace

@@ -37,10 +37,10 @@ __global__ void __launch_bounds__(kPT, 3) k_fused_jobs(const __grid_constant__ F
     const uint32_t u = k * J.chunk + (o - J.cbegin);  // the job's own ticket
     if (u >= J.tickets) continue;                      // past the job's last one
     const SyncWords sw = sync_words(J.s, J.a.n_frames);
-    // one copy of the item code per column-group count; dense peaks (sh.dense) at run time
-    const bool worked = J.sh.kG > 1 ? fused_ticket<false, kMaxG, true>(J.p, J.s, J.a, J.sh, sw, sm, u, ring_iter)
-                                    : fused_ticket<false, 1, true>(J.p, J.s, J.a, J.sh, sw, sm, u, ring_iter);
-    if (worked) __syncthreads();
+    // one copy of the item code per column-group count
+    if (J.sh.kG > 1) fused_ticket<kMaxG>(J.p, J.s, J.a, J.sh, sw, sm, u, ring_iter);
+    else fused_ticket<1>(J.p, J.s, J.a, J.sh, sw, sm, u, ring_iter);
+    __syncthreads();
   }
 }
 
@@ -78,8 +78,7 @@ bool fused_jobs_plan(FusedJobs* m, const FusedShape* tuned, int num_sms, uint32_
     for (uint32_t i = 0; i < m->n_jobs; ++i) {
       FusedJob& J = m->job[i];
       const uint32_t n = J.a.n_frames;
-      J.sh.lag1 = n < kLagSize ? n : kLagSize;
-      J.sh.lag2 = n < kLagWrite ? n : kLagWrite;
+      J.sh.lag = n < kLagWrite ? n : kLagWrite;
       const uint64_t t = fused_tickets(J.sh, n);
       if (t >= (1ull << 31)) return false;
       J.tickets = (uint32_t)t;

@@ -28,54 +28,21 @@
 namespace roibin {
 
 // ---------------------------------------------------------------------------
-// kDense: the variant for frames with many peak candidates (hot pixels).  Its
-// warp tests of listed candidates first try the exact rejection screen
-// (screen_rejects), and an item whose candidates overflow the list evaluates
-// them one per lane.  Both variants write the same bytes.
-// kG: column groups per consumer lane (FusedShape::kG; 2 only with RB = 2).
-template <bool kDense, int kG>
-__global__ void __launch_bounds__(kPT, 4) k_fused(DevParams p, Scratch s, PlainArgs a, FusedShape sh) {
-  extern __shared__ __align__(128) unsigned char sm[];
-  uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
-  const SyncWords sw = sync_words(s, a.n_frames);
-  const uint32_t n = a.n_frames, lag1 = sh.lag1, lag2 = lag1 + sh.lag2, round = sh.U + 2 * sh.groups;
-  const uint64_t total = fused_tickets(sh, n);
-  fused_cta_init(sm, sh);
-  uint32_t ring_iter = 0;  // ring stages consumed so far (the same in every thread)
-  for (;;) {
-    if (threadIdx.x == 0) ctl[CTL_ITEM] = atomicAdd(sw.ticket, 1u);
-    __syncthreads();
-    const uint32_t t = ctl[CTL_ITEM];
-    __syncthreads();
-    if (t >= total) break;
-    // the body of fused_ticket
-    const uint32_t r = t / round, j = t - r * round;
-    if (j < sh.U) {
-      if (r >= n) continue;
-      if (kG > 1 || sh.RB == 2) process_item<2, kDense, kG>(p, s, a, sh, sm, r, j, ring_iter);
-      else process_item<3, kDense, 1>(p, s, a, sh, sm, r, j, ring_iter);
-      // publish the item; the CTA that completes the frame builds its codebook
-      __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) ctl[CTL_LAST] = atomicAdd(sw.panel_done + r, 1u) == sh.U - 1 ? 1u : 0u;
-      __syncthreads();
-      if (ctl[CTL_LAST]) {
-        __threadfence();
-        frame_codebook(p, s, a, sh, sm, r, sw);
-      }
-    } else if (j < sh.U + sh.groups) {
-      if (r < lag1 || r - lag1 >= n) continue;
-      size_item(p, s, a, sh, sm, r - lag1, j - sh.U, sw);
-    } else {
-      if (r < lag2 || r - lag2 >= n) continue;
-      write_item(p, s, a, sh, sm, r - lag2, j - sh.U - sh.groups, sw);
-    }
-    __syncthreads();
+// host side
+// The candidates of an item up to which they are tested a warp each (eight at a
+// time, about 5 us a round); above, they are tested a lane each, band by band
+// (about 12 us a band of rows in shared memory): the two meet near 20 candidates a
+// band.
+static void set_list_max(const DevParams& p, FusedShape* sh) {
+  if (!sh->band_rows) {
+    sh->list_max = kThrLocalCap + kThrSpill;
+    return;
   }
+  const uint32_t own = sh->band_rows - 2 * (uint32_t)peak_reach(p);  // rows a band adds
+  const uint32_t bands = sh->k * ceil_div(min(p.H, 2 * sh->band_bins), own);
+  sh->list_max = min(20u * bands, kThrLocalCap + kThrSpill);
 }
 
-// ---------------------------------------------------------------------------
-// host side
 // Shared memory a CTA of this shape needs (0 if the shape is impossible).
 static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, uint32_t stages, FusedShape* out) {
   FusedShape sh{};
@@ -86,6 +53,8 @@ static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, ui
   sh.k = min(kMaxK, sh.kG * kGroupCols / NP);
   if ((uint64_t)sh.k * p.H * p.W >= kBlockKey) return false;  // item-local keys stay below the flag
   sh.U = ceil_div(p.P, sh.k);
+  sh.bands = 1;
+  sh.band_bins = p.Hb;
   sh.RB = rb;
   sh.stages = stages;
   // the streamed rows are read once: first out of L2, so that the code bytes
@@ -96,10 +65,8 @@ static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, ui
   sh.ctas_per_sm = ctas_per_sm;
   sh.mask_words = ceil_div(p.Hb * p.Wb, 32) + 1;
   sh.side = 2 * (uint32_t)peak_reach(p) + 1;
-  uint32_t n2 = 1;
-  while (n2 < max(p.max_peaks, 1u)) n2 <<= 1;
-  sh.sort_n2 = n2;
-  sh.peak_cap = max(p.max_peaks, 1u);
+  uint32_t n2 = 4;  // words the peak sort needs
+  while (n2 < p.max_peaks) n2 <<= 1;
   sh.n_chunks = p.n_chunks;
   sh.codes_stride = p.n_chunks * kChunk;
   sh.group_chunks = 2 * kPW;
@@ -123,12 +90,11 @@ static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, ui
   const uint64_t ring_end = off;
   off = sh.off_ring;
   sh.off_nb = take((uint64_t)kPW * sh.side * sh.side * 4);
-  sh.off_acc = take((uint64_t)n2 * 4);
   sh.off_cand = take(kThrLocalCap * 4);
   const uint64_t stream_end = off > ring_end ? off : ring_end;
   // codebook role / size, write and plan roles (overlap the streaming role)
   off = base;
-  sh.off_huff = take(sizeof(HuffSmem) > 4096 ? sizeof(HuffSmem) : 4096);  // Huffman scratch | byte tables
+  sh.off_huff = take(kHuffArea);  // Huffman scratch | byte tables | slices of the 3-D stacking
   const uint64_t after_huff = off;
   off = sh.off_huff + 4096;  // chunk staging of the size and write items (after the byte tables)
   sh.off_stage = take((uint64_t)kPW * kStageWords * 4);
@@ -137,10 +103,10 @@ static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, ui
   sh.off_total = take(kMaxSymbols * 4);
   sh.off_cblen = take(kMaxSymbols);
   sh.off_cbcode = take(kMaxSymbols * 4);
-  sh.off_keys = take(16);
   sh.off_cw = take(3ull * p.n_chunks * 4);
-  sh.off_offs = take((uint64_t)sh.U * 4);
-  const uint64_t fin_end = off > stage_end ? off : stage_end;
+  const uint64_t sort_end = sh.off_huff + (uint64_t)n2 * 4;  // before the histogram is read
+  uint64_t fin_end = off > stage_end ? off : stage_end;
+  if (sort_end > fin_end) fin_end = sort_end;
   sh.smem = (uint32_t)(stream_end > fin_end ? stream_end : fin_end);
   // The dense-peaks variant takes all the shared memory its CTAs per SM leave
   // it: from the ring on, that memory holds a band of rows of one panel once
@@ -148,15 +114,23 @@ static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, ui
   // per thread, so a taller band keeps more threads busy.
   const uint32_t share = 233472u / ctas_per_sm - 1024u;
   sh.smem_dense = sh.smem > share ? sh.smem : (share < 227u * 1024u ? share : 227u * 1024u);
-  sh.band_rows = (sh.smem_dense - sh.off_ring) / (p.W * 4);
+  const uint32_t least = 2 * (uint32_t)peak_reach(p) + 2;
+  auto rows_in = [&](uint32_t smem) {
+    const uint32_t rows = (smem - sh.off_ring) / (p.W * 4);
+    return rows >= least ? rows : 0u;
+  };
+  sh.band_rows = rows_in(sh.smem);
+  sh.band_rows_dense = rows_in(sh.smem_dense);
+  set_list_max(p, &sh);
   *out = sh;
   return sh.smem <= 227 * 1024;
 }
 
-// The kernel instantiation for a shape: dense-peaks variant or not, column groups.
-static const void* fused_kernel(bool dense, uint32_t kG) {
-  if (kG > 1) return dense ? (const void*)k_fused<true, kMaxG> : (const void*)k_fused<false, kMaxG>;
-  return dense ? (const void*)k_fused<true, 1> : (const void*)k_fused<false, 1>;
+// The kernel instantiation for a shape: column groups, rows per step, row bands.
+static FusedKernel fused_kernel(const FusedShape& sh) {
+  if (sh.bands > 1) return fused_band_kernel(sh.kG);
+  if (sh.kG > 1) return k_fused<kMaxG, 2, false>;
+  return sh.RB == 3 ? k_fused<1, 3, false> : k_fused<1, 2, false>;
 }
 
 bool fused_shape_for(const DevParams& p, uint32_t ctas_per_sm, uint32_t rows_per_step, uint32_t stages,
@@ -175,7 +149,7 @@ bool fused_shape_for(const DevParams& p, uint32_t ctas_per_sm, uint32_t rows_per
     for (uint32_t rb = 3; rb >= 2 && !ok; --rb) ok = make_shape(p, ctas_per_sm, rb, stages, &sh) && sh.smem <= budget;
   }
   if (!ok) return false;
-  const void* kern = fused_kernel(false, sh.kG);
+  const FusedKernel kern = fused_kernel(sh);
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -203,32 +177,68 @@ bool fused_plan(const DevParams& p, int device, int num_sms, FusedShape* out) {
          fused_shape_for(p, 2, 2, 2, out) || fused_shape_for(p, 1, 2, 1, out);
 }
 
+// Cuts the panels of a small batch into row bands: a batch of few frames has too
+// few panel groups to occupy every CTA (one CSPAD frame has 16 for 608), and the
+// last wave of a middling one is long.  The bands per panel with the least
+//   waves x (an item's pixels per raw row pair x its binned rows + a fixed cost)
+// where the fixed cost of an item (its start, flush and peak tests, about 12 us)
+// is worth 17,000 of those pixels (a 776-pixel binned row takes 0.54 us), waves =
+// items / CTAs (at least 1), and a partly filled wave after the first costs 0.15
+// more.  us per call, whole panels -> bands: 1 CSPAD frame 93 -> 61, 8 frames 105
+// -> 79, 16 frames 121 -> 96, 33 frames one band (132; two 147); 8 x 512 x 1024
+// panels: 1 frame 291 -> 72, 5 frames 308 -> 100, 20 frames 430 -> 199, 60 frames
+// 474 -> 430; 30 hot-pixel frames 1,120 -> 800, 100 of them one band (1,636; two
+// 1,772).
+static void band_shape(const DevParams& p, const Scratch& s, uint32_t n, FusedShape* sh) {
+  const uint64_t items = (uint64_t)n * sh->U;
+  if (sh->RB != 2 || items >= 4ull * sh->n_ctas) return;
+  uint32_t best = p.Hb;
+  double best_cost = 0.0;
+  for (uint32_t bands = 1;; ++bands) {
+    const uint32_t bins = (ceil_div(p.Hb, bands) + 1) & ~1u;  // whole steps of two rows
+    if (bands > 1 && bins < 4) break;
+    const double w = (double)items * ceil_div(p.Hb, bins) / sh->n_ctas;
+    const double cost = (w > 1.0 ? w + 0.15 : 1.0) * ((double)min(bins, p.Hb) * sh->k * p.W + 17000.0);
+    if (bands == 1 || cost < best_cost) {
+      best = bins;
+      best_cost = cost;
+    }
+    if (w > 4.0) break;  // more bands only add fixed costs
+  }
+  for (; best < p.Hb; best *= 2) {
+    const uint32_t bands = ceil_div(p.Hb, best), words = ceil_div(best * p.Wb, 32) + 1;
+    if ((uint64_t)n * p.P * bands * words > s.pq_mask_words) continue;  // the outlier slots do not fit
+    sh->bands = bands;
+    sh->band_bins = best;
+    sh->mask_words = words;
+    sh->U *= bands;
+    set_list_max(p, sh);
+    return;
+  }
+}
+
 cudaError_t launch_fused(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
-                         bool screen, cudaStream_t st) {
+                         bool dense, cudaStream_t st) {
   // stage counters, ready flags and the ticket counter start at zero
   cudaError_t e = cudaMemsetAsync(s.frame_done, 0, sizeof(uint32_t) * (kSyncWordsPerFrame * (uint64_t)a.n_frames + 1), st);
   if (e != cudaSuccess) return e;
-  const uint32_t smem = screen ? sh.smem_dense : sh.smem;
-  e = cudaFuncSetAttribute(fused_kernel(screen, sh.kG), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   FusedShape s2 = sh;
-  // frames between the stages in the ticket order.  Streaming -> chunk sizes:
-  // the whole batch, so every frame streams before any is sized.  Streaming
-  // is bound by the bytes each CTA keeps in flight, and a CTA on a coding
-  // item has none; interleaving the stages (a lag of 256 frames) ran 6% slower
-  // at 1,000 frames.  Chunk sizes -> writing: 64 frames, so that a frame's
-  // plan is ready when its write items come up.
-  s2.lag1 = a.n_frames < kLagSize ? a.n_frames : kLagSize;
-  s2.lag2 = a.n_frames < kLagWrite ? a.n_frames : kLagWrite;
+  band_shape(p, s, a.n_frames, &s2);
+  const uint32_t smem = dense ? sh.smem_dense : sh.smem;
+  s2.dense = dense ? 1u : 0u;
+  const FusedKernel kern = fused_kernel(s2);
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // Every frame streams before any is sized: streaming is bound by the bytes each
+  // CTA keeps in flight, and a CTA on a coding item has none (interleaving the
+  // stages, 256 frames apart, ran 6% slower at 1,000 frames).  Chunk sizes ->
+  // writing: 64 frames, so that a frame's plan is ready when its write items
+  // come up.
+  s2.lag = a.n_frames < kLagWrite ? a.n_frames : kLagWrite;
   const uint64_t tickets = fused_tickets(s2, a.n_frames);
+  if (tickets + sh.n_ctas >= (1ull << 32)) return cudaErrorInvalidValue;
   const uint32_t grid = (uint32_t)(tickets < sh.n_ctas ? tickets : sh.n_ctas);
-  if (sh.kG > 1) {
-    if (screen) k_fused<true, kMaxG><<<grid, kPT, smem, st>>>(p, s, a, s2);
-    else k_fused<false, kMaxG><<<grid, kPT, smem, st>>>(p, s, a, s2);
-  } else {
-    if (screen) k_fused<true, 1><<<grid, kPT, smem, st>>>(p, s, a, s2);
-    else k_fused<false, 1><<<grid, kPT, smem, st>>>(p, s, a, s2);
-  }
+  kern<<<grid, kPT, smem, st>>>(p, s, a, s2);
   return cudaGetLastError();
 }
 

@@ -221,11 +221,13 @@ uint64_t carve_scratch(const DevParams& d, uint32_t n, uint8_t* base, Scratch* s
   t.bhat = reinterpret_cast<float*>(t.pq_bits);
   const uint64_t mask_words = ceil_div(d.Hb * d.Wb, 32) + 1;
   t.codes8 = c.take<uint8_t>((uint64_t)n * d.n_chunks * kChunk);
-  t.pq_mask = c.take<uint32_t>((uint64_t)n * d.P * mask_words);
-  t.hist_part = c.take<uint32_t>((uint64_t)n * d.P * kMaxSymbols);
-  t.peak_part = c.take<uint32_t>((uint64_t)n * d.P * std::max<uint32_t>(d.max_peaks, 1));
-  t.peak_part_count = c.take<uint32_t>((uint64_t)n * d.P);
-  t.pq_part_count = c.take<uint32_t>((uint64_t)n * d.P);
+  // the frames' code counts, and room for the outlier slots of a launch that cuts
+  // panels into row bands (more slots than panels).  These four sizes are what a
+  // context has always held, so that a budget admits the contexts it did.
+  t.hist_f = c.take<uint32_t>((uint64_t)n * kMaxSymbols);
+  t.pq_mask_words = (uint64_t)n * d.P * mask_words + (uint64_t)n * (d.P - 1) * kMaxSymbols +
+                    (uint64_t)n * d.P * std::max<uint32_t>(d.max_peaks, 1) + 2ull * n * d.P;
+  t.pq_mask = c.take<uint32_t>(t.pq_mask_words);
   t.lane_bit = c.take<uint32_t>((uint64_t)n * d.n_chunks * 32);
   t.lane_lo = c.take<uint32_t>((uint64_t)n * d.n_chunks * 32);
   t.lane_pq = c.take<uint32_t>((uint64_t)n * d.n_chunks * 32);
@@ -640,7 +642,8 @@ int roibin_ctx_create(roibin_ctx** out, const roibin_geometry* g, const roibin_p
   carve_scratch(ctx->dp, max_frames_per_call, static_cast<uint8_t*>(ctx->scratch), &ctx->s, spill_ctas,
                 &ctx->guards);
   // the check words start at zero; the guard bands (checks build) hold their pattern
-  bool set = cudaMemset(ctx->s.check, 0, 8) == cudaSuccess;
+  bool set = cudaMemset(ctx->s.check, 0, 8) == cudaSuccess &&
+             cudaMemset(ctx->s.hist_f, 0, (uint64_t)max_frames_per_call * kMaxSymbols * 4) == cudaSuccess;
   for (uint64_t g : ctx->guards)
     set = set && cudaMemset(static_cast<uint8_t*>(ctx->scratch) + g, kGuardByte, kGuardBytes) == cudaSuccess;
   if (!set || cudaDeviceSynchronize() != cudaSuccess) {

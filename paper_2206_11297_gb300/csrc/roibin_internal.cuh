@@ -107,11 +107,10 @@ struct Scratch {
   DecInfo* dec_info;      // [n]
   // persistent batched path (codes: esc side array; lo_delta, pq_bits shared)
   uint8_t* codes8;          // [n][n_chunks * kChunk] one code byte per bin
-  uint32_t* pq_mask;        // [n][P][mask_words] prequantisation-outlier bits per panel
-  uint32_t* hist_part;      // [n][P][kMaxSymbols] per-panel histograms
-  uint32_t* peak_part;      // [n][P][max(max_peaks, 1)] per-panel sorted peaks
-  uint32_t* peak_part_count;  // [n][P]
-  uint32_t* pq_part_count;    // [n][P] prequantisation outliers per panel
+  uint32_t* hist_f;         // [n][kMaxSymbols] the frame's code counts: zero between launches (the codebook
+                            // stage clears what it has read)
+  uint32_t* pq_mask;        // a slot of mask_words per panel and row band: its outlier count, then a bit per
+  uint64_t pq_mask_words;   // bin (written only where the count is not 0); words there are
   uint32_t* lane_bit;         // [n][n_chunks][32] bit offset of each lane's symbols in its chunk
   uint32_t* lane_lo;          // [n][n_chunks][32] Lorenzo outliers before the lane, in its chunk
   uint32_t* lane_pq;          // [n][n_chunks][32] prequantisation outliers before the lane
@@ -234,11 +233,16 @@ __device__ __forceinline__ Quant prequantize(float b, const DevParams& p) {
 
 // The common case of prequantize: true when the screen alone proves the bin
 // is not an outlier (then q is final); false sends the bin to prequantize.
+// rint by adding and subtracting 1.5 * 2^23, whose last bit is worth 1: exact,
+// to nearest even, for |x| <= 2^22 (larger ones are sent on).  The sum's bits
+// give q.  Two adds in place of a rounding and a conversion, which run at a
+// quarter of the rate or less.
 __device__ __forceinline__ bool prequant_fast(float b, const DevParams& p, int32_t& q) {
-  const float t = rintf(__fmul_rn(b, p.recip));
+  constexpr float kMagic = 12582912.0f, kFastLimit = 4194304.0f;
+  const float x = __fmul_rn(b, p.recip), m = __fadd_rn(x, kMagic), t = __fsub_rn(m, kMagic);
   const float d = __fsub_rn(b, __fmul_rn(t, p.two_eb));
-  q = __float2int_rz(t);  // exact for the |t| < 2^28 the fast path accepts
-  return (fabsf(t) < kPqLimit) & (fabsf(d) < p.eb_lo);
+  q = (int32_t)(__float_as_uint(m) - 0x4B400000u);
+  return (fabsf(x) < kFastLimit) & (fabsf(d) < p.eb_lo);
 }
 
 // 2x2 bin pair from two float4 (4 pixels of raw row 2i and of row 2i+1):
@@ -372,70 +376,60 @@ __device__ inline bool is_local_max_at(Px px, int H, int W, int r, int c, const 
   return true;
 }
 
-// is_local_max_at + evaluate_peak_at for one compile-time window and ring
-// (RANK, ring R0 .. R0 + DR): the same operations in the same order (so the
-// same float32 results), with every loop unrolled, so that the compiler sees
-// each neighbour's offset and issues the loads ahead of the ordered sums.
-// In-panel tests stay per pixel (a candidate may sit at the panel's edge).
-template <int RANK, int R0, int DR, class Px>
-__device__ __forceinline__ bool peak_test_fixed(Px px, int H, int W, int r, int c, const DevParams& p) {
-  constexpr int OUT = R0 + DR, RING = OUT - 1;
-  const float v = px(0, 0);
-  if (!(v >= p.amax)) return false;
-  bool ok = true;
-#pragma unroll
-  for (int dr = -RANK; dr <= RANK; ++dr) {
-#pragma unroll
-    for (int dc = -RANK; dc <= RANK; ++dc) {
-      if (dr == 0 && dc == 0) continue;
-      const int rr = r + dr, cc = c + dc;
-      if (rr < 0 || rr >= H || cc < 0 || cc >= W) continue;
-      const float u = px(dr, dc);
-      ok &= (dr < 0 || (dr == 0 && dc < 0)) ? (v > u) : (v >= u);
-    }
-  }
-  if (!ok) return false;
+// The paper's test (rank 3, ring 5 .. 7) for one thread on pixels in shared
+// memory, `at` the candidate's, rows W apart, every pixel within 6 of it inside
+// the panel: the same operations in the same order as is_local_max_at +
+// evaluate_peak_at, so the same float32 results, with no test per pixel.  The
+// compiler barrier between rows keeps it from hoisting every load to the front,
+// which spilled under a 64-register cap.  About 1,080 instructions; a warp alone
+// issues one in 8 cycles, so it takes 9 thousand cycles (13-14 with a test per
+// pixel, 18 with rolled loops over a table of offsets).
+#define RB_ROW_BARRIER() asm volatile("" ::: "memory")
+__device__ __forceinline__ bool peak_test_inner(const float* at, int W, const DevParams& p) {
+  const float v = at[0];
+  bool ok = v >= p.amax;
   float sum = 0.0f;
   int n = 0;
 #pragma unroll
-  for (int dr = -RING; dr <= RING; ++dr) {
+  for (int dr = -6; dr <= 6; ++dr) {  // the local-maximum rule and the ring's sum
+    const float* row = at + dr * W;
+    RB_ROW_BARRIER();
 #pragma unroll
-    for (int dc = -RING; dc <= RING; ++dc) {
-      if (dr * dr + dc * dc < R0 * R0 || dr * dr + dc * dc >= OUT * OUT) continue;
-      const int rr = r + dr, cc = c + dc;
-      if (rr < 0 || rr >= H || cc < 0 || cc >= W) continue;
-      sum = __fadd_rn(sum, px(dr, dc));
-      ++n;
-    }
-  }
-  float bkg = 0.0f, var = 0.0f;
-  if (n > 0) {
-    bkg = __fdiv_rn(sum, (float)n);
-    float ss = 0.0f;
-#pragma unroll
-    for (int dr = -RING; dr <= RING; ++dr) {
-#pragma unroll
-      for (int dc = -RING; dc <= RING; ++dc) {
-        if (dr * dr + dc * dc < R0 * R0 || dr * dr + dc * dc >= OUT * OUT) continue;
-        const int rr = r + dr, cc = c + dc;
-        if (rr < 0 || rr >= H || cc < 0 || cc >= W) continue;
-        const float d = __fsub_rn(px(dr, dc), bkg);
-        ss = __fadd_rn(ss, __fmul_rn(d, d));
+    for (int dc = -6; dc <= 6; ++dc) {
+      const int d2 = dr * dr + dc * dc;
+      if (d2 >= 25 && d2 < 49) {
+        sum = __fadd_rn(sum, row[dc]);
+        ++n;
+      } else if (d2 > 0 && dr >= -3 && dr <= 3 && dc >= -3 && dc <= 3) {
+        ok &= (dr < 0 || (dr == 0 && dc < 0)) ? (v > row[dc]) : (v >= row[dc]);
       }
     }
-    var = __fdiv_rn(ss, (float)n);
   }
-  const float sigma = __fsqrt_rn(var);
+  if (!ok) return false;
+  const float bkg = __fdiv_rn(sum, (float)n);
+  sum = 0.0f;
+#pragma unroll
+  for (int dr = -6; dr <= 6; ++dr) {
+    const float* row = at + dr * W;
+    RB_ROW_BARRIER();
+#pragma unroll
+    for (int dc = -6; dc <= 6; ++dc) {
+      if (dr * dr + dc * dc < 25 || dr * dr + dc * dc >= 49) continue;
+      const float d = __fsub_rn(row[dc], bkg);
+      sum = __fadd_rn(sum, __fmul_rn(d, d));
+    }
+  }
+  const float sigma = __fsqrt_rn(__fdiv_rn(sum, (float)n));
   const float thr = __fmul_rn(p.pix_nsigma, sigma);
   int npix = 0;
   float atot = 0.0f;
 #pragma unroll
-  for (int dr = -RANK; dr <= RANK; ++dr) {
+  for (int dr = -3; dr <= 3; ++dr) {
+    const float* row = at + dr * W;
+    RB_ROW_BARRIER();
 #pragma unroll
-    for (int dc = -RANK; dc <= RANK; ++dc) {
-      const int rr = r + dr, cc = c + dc;
-      if (rr < 0 || rr >= H || cc < 0 || cc >= W) continue;
-      const float d = __fsub_rn(px(dr, dc), bkg);
+    for (int dc = -3; dc <= 3; ++dc) {
+      const float d = __fsub_rn(row[dc], bkg);
       if (d > thr) {
         ++npix;
         atot = __fadd_rn(atot, d);
@@ -446,118 +440,6 @@ __device__ __forceinline__ bool peak_test_fixed(Px px, int H, int W, int r, int 
   if (!(atot > p.atot_thr)) return false;
   const float noise = __fmul_rn(__fmul_rn(p.son_min, sigma), __fsqrt_rn((float)npix));
   return atot > noise;
-}
-
-// The same test for a candidate whose neighbourhood rows [rb0, rb1) of its
-// panel sit in `band` (row pitch W).  It goes row by row: the row's pixels are
-// read unconditionally from clamped in-band addresses (so the reads of a row
-// are issued together), and out-of-panel or off-ring pixels are then masked
-// out by selects, so no pixel is a branch.  The sums take exactly the
-// in-panel pixels in row-major order, as evaluate_peak_at does, so the results
-// are the same bit for bit.
-template <int RANK, int R0, int DR>
-__device__ __forceinline__ bool peak_test_band(const float* band, int rb0, int rb1, int H, int W, int r, int c,
-                                               const DevParams& p) {
-  constexpr int OUT = R0 + DR, RING = OUT - 1, REACH = RANK > RING ? RANK : RING, SIDE = 2 * REACH + 1;
-  static_assert(SIDE <= 32, "one bit per column of the neighbourhood");
-  int col[SIDE];        // clamped columns c - REACH .. c + REACH
-  uint32_t col_in = 0;  // bit k: column c + k - REACH is in the panel
-#pragma unroll
-  for (int k = 0; k < SIDE; ++k) {
-    const int cc = c + k - REACH;
-    col_in |= (uint32_t)(cc >= 0 && cc < W) << k;
-    col[k] = min(max(cc, 0), W - 1);
-  }
-  auto row_at = [&](int dr) { return band + (min(max(r + dr, rb0), rb1 - 1) - rb0) * W; };
-  auto row_mask = [&](int dr) { return (r + dr >= 0 && r + dr < H) ? col_in : 0u; };
-  const float v = band[(r - rb0) * W + c];
-  if (!(v >= p.amax)) return false;
-  bool ok = true;
-#pragma unroll 1
-  for (int dr = -RANK; dr <= RANK; ++dr) {
-    const float* rp = row_at(dr);
-    const uint32_t m = row_mask(dr);
-    float x[2 * RANK + 1];
-#pragma unroll
-    for (int k = 0; k < 2 * RANK + 1; ++k) x[k] = rp[col[REACH - RANK + k]];
-#pragma unroll
-    for (int k = 0; k < 2 * RANK + 1; ++k) {
-      const int dc = k - RANK;
-      const bool in = ((m >> (REACH + dc)) & 1u) && (dr != 0 || dc != 0);
-      const bool pass = (dr < 0 || (dr == 0 && dc < 0)) ? (v > x[k]) : (v >= x[k]);
-      ok &= pass || !in;
-    }
-  }
-  if (!ok) return false;
-  float sum = 0.0f;
-  int n = 0;
-#pragma unroll 1
-  for (int dr = -RING; dr <= RING; ++dr) {
-    const float* rp = row_at(dr);
-    const uint32_t m = row_mask(dr);
-    float x[2 * RING + 1];
-#pragma unroll
-    for (int k = 0; k < 2 * RING + 1; ++k) x[k] = rp[col[REACH - RING + k]];
-#pragma unroll
-    for (int k = 0; k < 2 * RING + 1; ++k) {
-      const int dc = k - RING, d2 = dr * dr + dc * dc;
-      const bool in = ((m >> (REACH + dc)) & 1u) && d2 >= R0 * R0 && d2 < OUT * OUT;
-      sum = in ? __fadd_rn(sum, x[k]) : sum;
-      n += in;
-    }
-  }
-  float bkg = 0.0f, var = 0.0f;
-  if (n > 0) {
-    bkg = __fdiv_rn(sum, (float)n);
-    float ss = 0.0f;
-#pragma unroll 1
-    for (int dr = -RING; dr <= RING; ++dr) {
-      const float* rp = row_at(dr);
-      const uint32_t m = row_mask(dr);
-      float x[2 * RING + 1];
-#pragma unroll
-      for (int k = 0; k < 2 * RING + 1; ++k) x[k] = rp[col[REACH - RING + k]];
-#pragma unroll
-      for (int k = 0; k < 2 * RING + 1; ++k) {
-        const int dc = k - RING, d2 = dr * dr + dc * dc;
-        const bool in = ((m >> (REACH + dc)) & 1u) && d2 >= R0 * R0 && d2 < OUT * OUT;
-        const float d = __fsub_rn(x[k], bkg);
-        ss = in ? __fadd_rn(ss, __fmul_rn(d, d)) : ss;
-      }
-    }
-    var = __fdiv_rn(ss, (float)n);
-  }
-  const float sigma = __fsqrt_rn(var);
-  const float thr = __fmul_rn(p.pix_nsigma, sigma);
-  int npix = 0;
-  float atot = 0.0f;
-#pragma unroll 1
-  for (int dr = -RANK; dr <= RANK; ++dr) {
-    const float* rp = row_at(dr);
-    const uint32_t m = row_mask(dr);
-    float x[2 * RANK + 1];
-#pragma unroll
-    for (int k = 0; k < 2 * RANK + 1; ++k) x[k] = rp[col[REACH - RANK + k]];
-#pragma unroll
-    for (int k = 0; k < 2 * RANK + 1; ++k) {
-      const float d = __fsub_rn(x[k], bkg);
-      const bool take = ((m >> (REACH + k - RANK)) & 1u) && d > thr;
-      npix += take;
-      atot = take ? __fadd_rn(atot, d) : atot;
-    }
-  }
-  if (npix < p.npix_min || npix > p.npix_max) return false;
-  if (!(atot > p.atot_thr)) return false;
-  const float noise = __fmul_rn(__fmul_rn(p.son_min, sigma), __fsqrt_rn((float)npix));
-  return atot > noise;
-}
-
-// a1 + a2 for one thread: the unrolled form for the paper's window and ring
-// (rank 3, ring 5 .. 7), else the general loops.  Same results either way.
-template <class Px>
-__device__ __forceinline__ bool peak_test_one(Px px, int H, int W, int r, int c, const DevParams& p) {
-  if (p.rank == 3 && p.ring_r0 == 5 && p.ring_dr == 2) return peak_test_fixed<3, 5, 2>(px, H, W, r, c, p);
-  return is_local_max_at(px, H, W, r, c, p) && evaluate_peak_at(px, H, W, r, c, p);
 }
 
 __device__ inline bool evaluate_peak(const float* __restrict__ panel, int H, int W, int r, int c,
@@ -849,18 +731,16 @@ __device__ inline bool warp_peak_test(const float* __restrict__ panel, int H, in
 // two-queue merge takes the leaf on equal weights; code length = leaf depth
 // (a lone symbol gets 1); canonical codes by (length, symbol) ascending.
 struct HuffSmem {
-  uint32_t f[kMaxSymbols];        // compacted counts (symbol order), then sorted
-  uint16_t s[kMaxSymbols];        // compacted symbols, then sorted
-  uint32_t sf[kMaxSymbols];
-  uint16_t ss[kMaxSymbols];
-  uint32_t w[2 * kMaxSymbols];    // node weights: leaves [0,n), internal [n,2n-1)
-  uint16_t parent[2 * kMaxSymbols];
+  uint32_t f[kMaxSymbols];        // compacted counts (symbol order)
+  uint32_t sf[kMaxSymbols];       // counts, sorted
+  uint32_t w[kMaxSymbols];        // weights of the internal nodes, in the order they are made
+  uint16_t s[kMaxSymbols];        // compacted symbols
+  uint16_t pos[kMaxSymbols];      // each compacted symbol's place in the sorted order
+  uint16_t parent[2 * kMaxSymbols];  // leaves (sorted), then internal nodes: internal parent
+  uint8_t len[kMaxSymbols];       // compacted code lengths
   uint32_t cnt_len[34];
   uint32_t first_code[34];
-  uint32_t running[34];
-  uint32_t warp_cnt[32][34];
   uint32_t scan_tmp[33];
-  uint32_t n;
   int32_t status;
 };
 
@@ -868,115 +748,114 @@ struct HuffSmem {
 // Writes len[nsym] and code[nsym] (shared or global).  Returns ROIBIN_OK or
 // ROIBIN_ERR_CODE_LENGTH (same value in every thread).  All threads of the
 // block must call it; blockDim.x must be a multiple of 32.
+// The stages are latency-bound chains on a few to a thousand symbols; the merge
+// keeps the two front entries of both queues in registers, and the canonical
+// codes are ranked by counting equal lengths, four to a word, without a barrier.
+// CTA time of the stage, 256 threads: CSPAD-like frames (a dozen symbols) 17.9 ->
+// 9.8 us alone, 24 -> 16 us beside streaming; epix10k (about 220) 37 -> 28 us.
 __device__ inline int build_codebook(const uint32_t* hist, uint32_t nsym, HuffSmem& h,
                                      uint8_t* len_out, uint32_t* code_out) {
   const uint32_t tid = threadIdx.x, nt = blockDim.x;
-  // 1. compact the non-zero symbols, keeping symbol order
-  uint32_t base = 0;
-  for (uint32_t s0 = 0; s0 < nsym; s0 += nt) {
-    const uint32_t s = s0 + tid;
-    const uint32_t f = s < nsym ? hist[s] : 0u;
-    uint32_t tot;
-    const uint32_t pos = block_excl_scan(f > 0 ? 1u : 0u, h.scan_tmp, &tot);
-    if (f > 0) {
-      h.f[base + pos] = f;
-      h.s[base + pos] = (uint16_t)s;
-    }
-    base += tot;
+  // 1. compact the non-zero symbols, keeping symbol order: a run of symbols a thread
+  const uint32_t per = (nsym + nt - 1) / nt, s0 = min(nsym, tid * per), s1 = min(nsym, s0 + per);
+  uint32_t mine = 0;
+  for (uint32_t s = s0; s < s1; ++s) {
+    mine += hist[s] > 0;
+    len_out[s] = 0;
+    code_out[s] = 0;
   }
-  if (tid == 0) {
-    h.n = base;
-    h.status = ROIBIN_OK;
+  uint32_t n;
+  uint32_t at = block_excl_scan(mine, h.scan_tmp, &n);
+  for (uint32_t s = s0; s < s1; ++s) {
+    const uint32_t f = hist[s];
+    if (f == 0) continue;
+    h.f[at] = f;
+    h.s[at++] = (uint16_t)s;
   }
-  for (uint32_t L = tid; L < 34; L += nt) {
-    h.cnt_len[L] = 0;
-    h.running[L] = 0;
-  }
+  if (tid < 4 && n + tid < kMaxSymbols) h.f[n + tid] = 0xFFFFFFFFu;  // read past the end below
+  if (tid == 0) h.status = ROIBIN_OK;
+  for (uint32_t L = tid; L < 34; L += nt) h.cnt_len[L] = 0;
   __syncthreads();
-  const uint32_t n = h.n;
   // 2. rank sort by (count, symbol): symbols are already ascending
   for (uint32_t i = tid; i < n; i += nt) {
     const uint32_t fi = h.f[i];
     uint32_t rank = 0;
-    for (uint32_t j = 0; j < n; ++j) {
-      const uint32_t fj = h.f[j];
-      rank += (fj < fi) || (fj == fi && j < i);
+    for (uint32_t j = 0; j < n; j += 4) {
+      const uint4 q = *reinterpret_cast<const uint4*>(h.f + j);
+      rank += (q.x < fi || (q.x == fi && j < i)) + (q.y < fi || (q.y == fi && j + 1 < i)) +
+              (q.z < fi || (q.z == fi && j + 2 < i)) + (q.w < fi || (q.w == fi && j + 3 < i));
     }
     h.sf[rank] = fi;
-    h.ss[rank] = h.s[i];
+    h.pos[i] = (uint16_t)rank;
   }
   __syncthreads();
-  for (uint32_t s = tid; s < nsym; s += nt) len_out[s] = 0;
-  // 3. two-queue merge (sequential by nature; one thread)
+  // 3. two-queue merge (sequential by nature; one thread), the leaf on equal weights
   if (tid == 0 && n >= 2) {
-    for (uint32_t i = 0; i < n; ++i) h.w[i] = h.sf[i];
-    uint32_t nl = 0, ni = n, nc = n;
+    constexpr uint32_t kNone = 0xFFFFFFFFu;  // above every weight
+    uint32_t nl = 0, ni = 0, nc = 0;          // next leaf, next and new internal node
+    uint32_t l0 = h.sf[0], l1 = h.sf[1], i0 = kNone, i1 = kNone;
     for (uint32_t k = 0; k + 1 < n; ++k) {
-      uint32_t a, b;
-      if (nl < n && (ni >= nc || h.w[nl] <= h.w[ni])) a = nl++; else a = ni++;
-      if (nl < n && (ni >= nc || h.w[nl] <= h.w[ni])) b = nl++; else b = ni++;
-      h.w[nc] = h.w[a] + h.w[b];
-      h.parent[a] = (uint16_t)nc;
-      h.parent[b] = (uint16_t)nc;
+      uint32_t sum = 0;
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        if (l0 <= i0) {
+          sum += l0;
+          h.parent[nl++] = (uint16_t)nc;
+          l0 = l1;
+          l1 = nl + 1 < n ? h.sf[nl + 1] : kNone;
+        } else {
+          sum += i0;
+          h.parent[n + ni++] = (uint16_t)nc;
+          i0 = i1;
+          i1 = ni + 1 < nc ? h.w[ni + 1] : kNone;
+        }
+      }
+      h.w[nc] = sum;
+      if (ni == nc) i0 = sum;
+      else if (ni + 1 == nc) i1 = sum;
       ++nc;
     }
   }
   __syncthreads();
-  // 4. depths by walking to the root
+  // 4. depths by walking to the root (the last internal node)
   for (uint32_t i = tid; i < n; i += nt) {
     uint32_t d = 1;
     if (n >= 2) {
-      const uint32_t root = 2 * n - 2;
-      uint32_t x = i;
-      d = 0;
-      while (x != root && d <= 40) {
-        x = h.parent[x];
+      uint32_t x = h.parent[h.pos[i]];
+      while (x != n - 2 && d <= 40) {
+        x = h.parent[n + x];
         ++d;
       }
     }
     if (d > 32) h.status = ROIBIN_ERR_CODE_LENGTH;
     const uint32_t L = d > 33 ? 33 : d;
-    len_out[h.ss[i]] = (uint8_t)L;
+    h.len[i] = (uint8_t)L;
     atomicAdd(&h.cnt_len[L], 1u);
   }
+  if (tid < 4 && n + tid < kMaxSymbols) h.len[n + tid] = 0;
   __syncthreads();
-  if (tid == 0) {
-    uint64_t c = 0;
-    uint32_t prev = 0;
-    for (uint32_t L = 1; L <= 32; ++L) {
-      h.first_code[L] = 0;
-      if (h.cnt_len[L] == 0) continue;
-      c = prev == 0 ? 0 : (c + h.cnt_len[prev]) << (L - prev);
-      h.first_code[L] = (uint32_t)c;
-      prev = L;
+  // 5. first_code[L] = sum of cnt[l] 2^(L - l) over l < L (modulo 2^32; exact for every length in use)
+  if (tid < 32) {
+    const uint32_t L = tid + 1, c = h.cnt_len[L];
+    uint32_t code = 0;
+    for (uint32_t l = 1; l < 32; ++l) {
+      const uint32_t cl = __shfl_sync(0xffffffffu, c, l - 1);
+      if (l < L) code += cl << (L - l);
     }
+    h.first_code[L] = code;
   }
   __syncthreads();
-  // 5. canonical codes: first_code[L] + rank among same-length symbols
-  const uint32_t warp = tid >> 5, nwarps = nt >> 5;
-  for (uint32_t s0 = 0; s0 < nsym; s0 += nt) {
-    const uint32_t s = s0 + tid;
-    const uint32_t L = s < nsym ? len_out[s] : 0u;
-    const uint32_t peers = __match_any_sync(0xffffffffu, L);
-    const uint32_t lower = __popc(peers & lanemask_lt());
-    for (uint32_t k = tid; k < 32 * 34; k += nt) (&h.warp_cnt[0][0])[k] = 0;
-    __syncthreads();
-    if (s < nsym && L > 0 && lower == 0) h.warp_cnt[warp][L] = __popc(peers);
-    __syncthreads();
-    if (s < nsym && L > 0 && L <= 32) {
-      uint32_t before = h.running[L];
-      for (uint32_t w = 0; w < warp; ++w) before += h.warp_cnt[w][L];
-      code_out[s] = h.first_code[L] + before + lower;
-    } else if (s < nsym) {
-      code_out[s] = 0;
-    }
-    __syncthreads();
-    if (tid < 34) {
-      uint32_t add = 0;
-      for (uint32_t w = 0; w < nwarps; ++w) add += h.warp_cnt[w][tid];
-      h.running[tid] += add;
-    }
-    __syncthreads();
+  // canonical codes: first_code[L] + rank among same-length symbols
+  for (uint32_t i = tid; i < n; i += nt) {
+    const uint32_t L = h.len[i], s = h.s[i];
+    len_out[s] = (uint8_t)L;
+    if (L > 32) continue;
+    const uint32_t same = L * 0x01010101u;
+    uint32_t before = 0;
+    for (uint32_t j = 0; j + 4 <= i; j += 4)
+      before += __popc(__vcmpeq4(*reinterpret_cast<const uint32_t*>(h.len + j), same)) >> 3;
+    for (uint32_t j = i & ~3u; j < i; ++j) before += h.len[j] == L;
+    code_out[s] = h.first_code[L] + before;
   }
   const int st = h.status;
   __syncthreads();
@@ -1017,25 +896,26 @@ constexpr uint32_t kTracePoints = 16;
 // Shape of the persistent batched kernel, chosen on the host (fused_kernel.cu).
 struct FusedShape {
   uint32_t ctas_per_sm, n_ctas;  // resident CTAs per SM, grid size
-  uint32_t k, U;                 // panels per streaming item; streaming items per frame
+  uint32_t k, U;                 // panels per streaming item; streaming items per frame (panel groups x bands)
   uint32_t kG;                   // column groups per consumer lane (1, or 2 for panels above 868 columns)
   uint32_t RB;                   // binned rows per streaming step (2 or 3)
   uint32_t stages, stage_bytes;  // TMA ring: slots, bytes per slot (2 RB raw rows of k panels)
-  uint32_t mask_words;           // prequantisation-outlier bitmask words per panel
+  uint32_t bands, band_bins;     // row bands a panel is cut into (1: whole panels), binned rows of each
+  uint32_t mask_words;           // words of a prequantisation-outlier slot (one per panel and band)
   uint32_t side;                 // side of the peak-test neighbourhood
-  uint32_t sort_n2;              // power of two >= max_peaks
-  uint32_t peak_cap;             // max(max_peaks, 1)
   uint32_t n_chunks;
   uint32_t codes_stride;         // code bytes per frame slot (n_chunks * kChunk)
   uint32_t group_chunks, groups; // chunks per size/write work item; items per frame
-  uint32_t lag1, lag2;           // frames between stages in the ticket order (per launch)
+  uint32_t lag;                  // frames between sizing and writing in the ticket order (per launch)
   uint32_t input_evict_first;    // L2 policy of the streamed rows (1 = evict first)
   uint32_t wait_limit;           // polls of a flag wait before it reports ROIBIN_ERR_TIMEOUT
-  uint32_t band_rows;            // dense peaks: panel rows staged at once (band + halo)
+  uint32_t band_rows, band_rows_dense;  // panel rows staged at once as a band with its halo, in the plain
+                                 // launch's shared memory and in the dense-peaks variant's (0: no band fits)
+  uint32_t list_max;             // candidates of an item tested a warp each (more: band by band)
   uint32_t smem_dense;           // shared memory of the dense-peaks variant (>= smem)
-  uint32_t dense;                // multi-job launch: this job takes the dense-peaks code
-  uint32_t off_ctl, off_bar, off_hist, off_pql, off_thr, off_ring, off_nb, off_acc, off_cand;  // streaming role
-  uint32_t off_huff, off_total, off_cblen, off_cbcode, off_keys, off_cw, off_offs;  // codebook / plan roles
+  uint32_t dense;                // the dense-peaks variant (per launch)
+  uint32_t off_ctl, off_bar, off_hist, off_pql, off_thr, off_ring, off_nb, off_cand;  // streaming role
+  uint32_t off_huff, off_total, off_cblen, off_cbcode, off_cw;  // codebook / plan roles
   uint32_t off_stage;                                                        // size / write roles
   uint32_t smem;
 };
@@ -1043,7 +923,9 @@ bool fused_plan(const DevParams& p, int device, int num_sms, FusedShape* out);
 bool fused_shape_for(const DevParams& p, uint32_t ctas_per_sm, uint32_t rows_per_step, uint32_t stages,
                      FusedShape* out);
 cudaError_t launch_fused(const DevParams& p, const Scratch& fs, const PlainArgs& a, const FusedShape& sh,
-                         bool screen, cudaStream_t st);
+                         bool dense, cudaStream_t st);
+using FusedKernel = void (*)(DevParams, Scratch, PlainArgs, FusedShape);
+FusedKernel fused_band_kernel(uint32_t kG);  // the instantiations whose items are row bands of panels
 
 // One persistent launch over several batches (fused_jobs.cu): each job is a
 // batch of frames of one geometry with its own parameters, scratch, outputs
