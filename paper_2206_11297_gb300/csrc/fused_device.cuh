@@ -24,6 +24,7 @@ constexpr uint32_t kProducerWarp = 7;   // the warp whose lane 0 issues the row 
 constexpr uint32_t kThrLocalCap = 256;
 constexpr uint32_t kBlockKey = 1u << 31;  // a listed 2x4 block (else a listed candidate pixel)
 constexpr uint32_t kPqList = 128;  // prequantisation outliers an item lists before rescanning
+constexpr uint32_t kStackSlice = 896;  // bins of every panel a stack item takes: 32 panels' slices fit kHuffArea
 constexpr uint32_t kHuffArea = 29 * 1024;  // bytes of the Huffman scratch and of what shares its place
 static_assert(sizeof(HuffSmem) <= kHuffArea, "the Huffman scratch fits its area");
 constexpr uint32_t kLagWrite = 64;  // see launch_fused
@@ -207,8 +208,9 @@ __device__ __forceinline__ FinView fin_view(unsigned char* sm, const FusedShape&
 }
 
 // Per-frame words, zeroed before each launch:
-//   panel_done, size_done   streaming / size items finished;
-//   stage                   bit 0: the codebook is published, bit 1: the plan is;
+//   panel_done, size_done   streaming (then stack) / size items finished;
+//   stage                   bit 0: the codebook is published, bit 1: the plan is,
+//                           bit 2: the frame has streamed (3-D predictor);
 //   fin                     the plan and the write items finished (the one that
 //                           finishes last settles the frame's status); bit 31 is
 //                           set by any item that gave up waiting (sticky: no later
@@ -218,7 +220,7 @@ __device__ __forceinline__ FinView fin_view(unsigned char* sm, const FusedShape&
 struct SyncWords {
   uint32_t *panel_done, *size_done, *stage, *fin, *chunk_done, *peak_n, *pq_n, *ticket;
 };
-constexpr uint32_t kStageCodebook = 1u, kStagePlan = 2u, kGaveUp = 1u << 31;
+constexpr uint32_t kStageCodebook = 1u, kStagePlan = 2u, kStageStreamed = 4u, kGaveUp = 1u << 31;
 __device__ __forceinline__ SyncWords sync_words(const Scratch& s, uint32_t n) {
   SyncWords w;
   w.panel_done = s.frame_done;
@@ -1074,103 +1076,6 @@ __device__ void chunk_codebook(const DevParams& p, const Scratch& s, const Plain
     for (uint32_t g = c0; g < c1; ++g) flag_release(sw.stage + g, kStageCodebook);
 }
 
-// The 3-D predictor (a6 over the panel stack, §6) from the streamed 2-D
-// residuals: the 3-D residual of a bin is, exactly in integers, its 2-D
-// residual minus the 2-D residual of the same bin in the panel before (the
-// panel's own residual for the first panel).  One CTA rewrites the frame's
-// code bytes, escape codes and Lorenzo-outlier deltas in place.  A bin's new
-// value depends only on the same bin of the panel below, so the panel's bins
-// are taken in slices, and a slice goes from the last panel down: the slice of
-// the panel below is read into shared memory (16-byte loads of whole lines),
-// the panel's new bytes are written from there, and that slice becomes the
-// next step's own.  The frame's histogram of the new codes goes to `total`.
-// `stage` is the Huffman scratch (unused until the codebook is built).
-__device__ __noinline__ void stack_residuals(const DevParams& p, const Scratch& s, const FusedShape& sh, uint32_t* total,
-                                             unsigned char* stage, uint32_t f) {
-  const uint32_t tid = threadIdx.x, lane = lane_id();
-  for (uint32_t k = tid; k < p.nsym; k += kPT) total[k] = 0;
-  uint8_t* codes = s.codes8 + (size_t)f * sh.codes_stride;  // 16-byte aligned (whole chunks per frame)
-  uint16_t* esc = s.codes + (size_t)f * p.M;
-  int32_t* lo = s.lo_delta + (size_t)f * p.M;
-  const uint32_t Mp = p.Hb * p.Wb;  // even: the fused path has an even binned width
-  const int32_t R = p.R;
-  // two slice buffers in the stage, each a slice plus the 15 bytes before its first line
-  constexpr uint32_t kSlice = (kHuffArea / 2 - 16) & ~15u;
-  uint8_t* buf[2] = {stage, stage + kSlice + 16};
-  uint32_t zeros = 0;  // codes of the zero residual this thread saw (the common code)
-  auto residual = [&](uint32_t b, uint32_t bin) -> int32_t {  // the stored 2-D residual from its byte
-    if (b == 0) return lo[bin];
-    if (b == 255) return (int32_t)esc[bin] - R;
-    return (int32_t)b - 128;
-  };
-  auto count = [&](uint32_t c) {
-    if (c == (uint32_t)R) ++zeros;
-    else atomicAdd(total + c, 1u);
-  };
-  // bytes [from, from + len) of the frame's codes into b (byte i at b[(from & 15) + i])
-  auto load = [&](uint8_t* b, uint32_t from, uint32_t len) {
-    const uint32_t a = from & ~15u, words = (from - a + len + 15) / 16;
-    const uint4* src = reinterpret_cast<const uint4*>(codes + a);
-    for (uint32_t w = tid; w < words; w += kPT) reinterpret_cast<uint4*>(b)[w] = __ldcg(src + w);
-  };
-  __syncthreads();
-  for (uint32_t x0 = 0; x0 < Mp; x0 += kSlice) {
-    const uint32_t len = min(kSlice, Mp - x0);  // even (Mp and kSlice are)
-    uint32_t cur = 0;
-    load(buf[cur], (p.P - 1) * Mp + x0, len);
-    for (uint32_t pn = p.P - 1; pn >= 1; --pn) {
-      const uint32_t at = pn * Mp + x0, below_at = at - Mp;
-      load(buf[cur ^ 1u], below_at, len);
-      __syncthreads();  // both slices are in shared memory
-      const uint8_t* cb8 = buf[cur] + (at & 15u);
-      const uint8_t* bb8 = buf[cur ^ 1u] + (below_at & 15u);
-      for (uint32_t i = 2 * tid; i < len; i += 2 * kPT) {  // two bins a thread: 2-byte aligned in the frame
-        // the common case: both bins hold the zero residual in both panels, so
-        // the new residuals are zero too and the stored bytes stay as they are
-        if (*reinterpret_cast<const uint16_t*>(cb8 + i) == 0x8080u &&
-            *reinterpret_cast<const uint16_t*>(bb8 + i) == 0x8080u) {
-          zeros += 2;
-          continue;
-        }
-        uint32_t pair = 0;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const uint32_t bin = at + i + j;
-          const uint32_t cb = cb8[i + j], bb = bb8[i + j];
-          int32_t d3;
-          if (cb != 0 && cb != 255 && bb != 0 && bb != 255) d3 = (int32_t)cb - (int32_t)bb;  // both ordinary
-          else d3 = (int32_t)((uint32_t)residual(cb, bin) - (uint32_t)residual(bb, bin - Mp));  // as the oracle's int64 -> int32
-          const uint32_t c = quant_code(d3, R);
-          uint32_t y;
-          if (c == 0) {
-            lo[bin] = d3;
-            y = 0;
-          } else if (d3 >= -127 && d3 <= 126) {
-            y = (uint32_t)(d3 + 128);
-          } else {
-            esc[bin] = (uint16_t)c;
-            y = 255;
-          }
-          pair |= y << (8 * j);
-          count(c);
-        }
-        *reinterpret_cast<uint16_t*>(codes + at + i) = (uint16_t)pair;
-      }
-      __syncthreads();  // the slice is done before its buffer takes the next panel's
-      cur ^= 1u;
-    }
-    __syncthreads();  // a single panel: its slice has just been read
-    // the first panel keeps its 2-D residuals: only counted
-    const uint8_t* cb8 = buf[cur] + (x0 & 15u);
-    for (uint32_t i = tid; i < len; i += kPT) count(quant_code(residual(cb8[i], x0 + i), R));
-    __syncthreads();
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) zeros += __shfl_xor_sync(0xffffffffu, zeros, o);
-  if (lane == 0 && zeros) atomicAdd(total + R, zeros);
-  __syncthreads();
-}
-
 // Sorts n distinct keys of a list in global memory, through shared memory (a
 // power of two of words >= n): by counting the smaller ones up to 256 keys, else
 // bitonic.
@@ -1258,14 +1163,10 @@ __device__ void frame_codebook(const DevParams& p, const Scratch& s, const Plain
     a.peaks_count_out[f] = n_peaks;
   }
   // a8: the frame's histogram, cleared for the next launch
-  if (p.dims == 3) {
-    stack_residuals(p, s, sh, v.total, sm + sh.off_huff, f);
-  } else {
-    uint32_t* hist = s.hist_f + (size_t)f * kMaxSymbols;
-    for (uint32_t k = tid; k < p.nsym; k += kPT) {
-      v.total[k] = __ldcg(hist + k);
-      hist[k] = 0;
-    }
+  uint32_t* hist = s.hist_f + (size_t)f * kMaxSymbols;
+  for (uint32_t k = tid; k < p.nsym; k += kPT) {
+    v.total[k] = __ldcg(hist + k);
+    hist[k] = 0;
   }
   __syncthreads();
   if (trace) trace[1] = global_ns();
@@ -1287,6 +1188,122 @@ __device__ void frame_codebook(const DevParams& p, const Scratch& s, const Plain
   __syncthreads();
   if (trace) trace[2] = global_ns();
   if (tid == 0) flag_release(sw.stage + f, kStageCodebook);
+}
+
+// (1a) The 3-D predictor (a6 over the panel stack, §6) from the streamed 2-D
+// residuals: the 3-D residual of a bin is, exactly in integers, its 2-D residual
+// minus the 2-D residual of the same bin in the panel before (the panel's own
+// residual for the first panel).  A bin's new value depends only on the same bin of
+// the panel below, so a frame's bins are cut into slices, one work item each: bins
+// [x0, x0 + len) of every panel.  The item reads the slice of as many panels as
+// fit shared memory at once (16-byte loads of whole lines), from the last panels
+// down, and each thread walks two bins down the panels, rewriting code bytes,
+// escape codes and Lorenzo-outlier deltas in place (it reads a panel's old values
+// one step before it replaces them).  The codes it has seen go to the frame's
+// histogram.  One CTA per frame, slice after slice and panel after panel with two
+// barriers each, took 386 us a frame: 40 CSPAD-like frames 390 -> 176 us.
+__device__ void stack_slice(const DevParams& p, const Scratch& s, const FusedShape& sh, unsigned char* sm, uint32_t f,
+                            uint32_t slice) {
+  const uint32_t tid = threadIdx.x, lane = lane_id();
+  uint32_t* total = reinterpret_cast<uint32_t*>(sm + sh.off_total);
+  uint8_t* stage = sm + sh.off_huff;
+  for (uint32_t k = tid; k < p.nsym; k += kPT) total[k] = 0;
+  uint8_t* codes = s.codes8 + (size_t)f * sh.codes_stride;  // 16-byte aligned (whole chunks per frame)
+  uint16_t* esc = s.codes + (size_t)f * p.M;
+  int32_t* lo = s.lo_delta + (size_t)f * p.M;
+  const uint32_t Mp = p.Hb * p.Wb;  // even: the fused path has an even binned width
+  const int32_t R = p.R;
+  const uint32_t x0 = slice * kStackSlice, len = min(kStackSlice, Mp - x0);  // both even
+  constexpr uint32_t kRow = kStackSlice + 32;  // a panel's slice and the bytes before its first line
+  constexpr uint32_t kPanels = kHuffArea / kRow;
+  uint32_t zeros = 0;  // codes of the zero residual this thread saw (the common code)
+  auto residual = [&](uint32_t b, uint32_t bin) -> int32_t {  // the stored 2-D residual from its byte
+    if (b == 0) return lo[bin];
+    if (b == 255) return (int32_t)esc[bin] - R;
+    return (int32_t)b - 128;
+  };
+  auto count = [&](uint32_t c) {
+    if (c == (uint32_t)R) ++zeros;
+    else atomicAdd(total + c, 1u);
+  };
+  for (uint32_t top = p.P; top > 0;) {
+    const uint32_t first = top > kPanels ? top - kPanels : 0u;  // panels first .. top - 1 are in shared memory
+    __syncthreads();
+    const uint32_t words = (15 + len + 15) / 16;  // of 16 bytes, whatever the panel's first byte
+    for (uint32_t i = tid; i < (top - first) * words; i += kPT) {
+      const uint32_t j = i / words, w = i - j * words, from = ((first + j) * Mp + x0) & ~15u;
+      if (from + 16 * w < sh.codes_stride)
+        reinterpret_cast<uint4*>(stage + j * kRow)[w] = __ldcg(reinterpret_cast<const uint4*>(codes + from) + w);
+    }
+    __syncthreads();
+    auto pair_at = [&](uint32_t pn, uint32_t i) {
+      return (uint32_t) * reinterpret_cast<const uint16_t*>(stage + (pn - first) * kRow + ((pn * Mp + x0) & 15u) + i);
+    };
+    const uint32_t last = first > 0 ? first + 1 : 1u;  // the lowest panel whose panel below is here
+    for (uint32_t i = 2 * tid; i < len; i += 2 * kPT) {  // two bins a thread: 2-byte aligned in the frame
+      uint32_t cur = pair_at(top - 1, i);
+      for (uint32_t pn = top - 1; pn >= last; --pn) {
+        const uint32_t below = pair_at(pn - 1, i);
+        // the common case: both bins hold the zero residual in both panels, so
+        // the new residuals are zero too and the stored bytes stay as they are
+        if (cur == 0x8080u && below == 0x8080u) {
+          zeros += 2;
+          continue;
+        }
+        uint32_t pair = 0;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const uint32_t bin = pn * Mp + x0 + i + j;
+          const uint32_t cb = (cur >> (8 * j)) & 0xFFu, bb = (below >> (8 * j)) & 0xFFu;
+          int32_t d3;
+          if (cb != 0 && cb != 255 && bb != 0 && bb != 255) d3 = (int32_t)cb - (int32_t)bb;  // both ordinary
+          else d3 = (int32_t)((uint32_t)residual(cb, bin) - (uint32_t)residual(bb, bin - Mp));  // as the oracle's int64 -> int32
+          const uint32_t c = quant_code(d3, R);
+          uint32_t y;
+          if (c == 0) {
+            lo[bin] = d3;
+            y = 0;
+          } else if (d3 >= -127 && d3 <= 126) {
+            y = (uint32_t)(d3 + 128);
+          } else {
+            esc[bin] = (uint16_t)c;
+            y = 255;
+          }
+          pair |= y << (8 * j);
+          count(c);
+        }
+        *reinterpret_cast<uint16_t*>(codes + pn * Mp + x0 + i) = (uint16_t)pair;
+        cur = below;
+      }
+      if (first == 0)  // the first panel keeps its 2-D residuals: only counted
+        for (int j = 0; j < 2; ++j) count(quant_code(residual((cur >> (8 * j)) & 0xFFu, x0 + i + j), R));
+    }
+    top = first > 0 ? first + 1 : 0u;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) zeros += __shfl_xor_sync(0xffffffffu, zeros, o);
+  if (lane == 0 && zeros) atomicAdd(total + R, zeros);
+  __syncthreads();
+  for (uint32_t k = tid; k < p.nsym; k += kPT)
+    if (total[k]) atomicAdd(s.hist_f + (size_t)f * kMaxSymbols + k, total[k]);
+}
+
+// A stack item: its slice once the frame has streamed; the one that finishes last
+// builds the frame's codebook.
+__device__ void stack_item(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
+                           unsigned char* sm, uint32_t f, uint32_t slice, const SyncWords& sw) {
+  uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
+  const bool ready = wait_flag(sw.stage + f, kStageStreamed, ctl + CTL_WAIT, sh.wait_limit);
+  if (ready) stack_slice(p, s, sh, sm, f, slice);
+  else if (threadIdx.x == 0) atomicOr(sw.fin + f, kGaveUp);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) ctl[CTL_LAST] = atomicAdd(sw.panel_done + f, 1u) == sh.U + sh.stack - 1 ? 1u : 0u;
+  __syncthreads();
+  if (ctl[CTL_LAST]) {
+    __threadfence();
+    frame_codebook(p, s, a, sh, sm, f, sw);
+  }
 }
 
 // Per-byte tables of a frame's codebook (byte = stored code byte):
@@ -1843,11 +1860,11 @@ __device__ void write_item_work(const DevParams& p, const Scratch& s, const Plai
 }
 
 // ---------------------------------------------------------------------------
-// The tickets of a launch over n frames: n U streaming items (frame by frame),
-// then lag frames' size items, then rounds of a frame's size items and the write
+// The tickets of a launch over n frames: n U streaming items (frame by frame), the
+// stack items of the 3-D predictor, then lag frames' size items, then rounds of a frame's size items and the write
 // items of the frame lag before it, then the last lag frames' write items.
 __host__ __device__ inline uint64_t fused_tickets(const FusedShape& sh, uint32_t n) {
-  return (uint64_t)n * (sh.U + 2 * sh.groups);
+  return (uint64_t)n * (sh.U + sh.stack + 2 * sh.groups);
 }
 // The item of a coding ticket c (counted from the first one): frame and group;
 // true for a write item.
@@ -1867,6 +1884,33 @@ __device__ __forceinline__ bool coding_item(const FusedShape& sh, uint32_t n, ui
   g = r - (n - lag);
   return true;
 }
+// After a streaming item of frame f: publishes it; the CTA that completes the frame
+// builds its codebook, or with the 3-D predictor lets its stack items go.
+__device__ __forceinline__ void streamed(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
+                                         const SyncWords& sw, unsigned char* sm, uint32_t f) {
+  uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) ctl[CTL_LAST] = atomicAdd(sw.panel_done + f, 1u) == sh.U - 1 ? 1u : 0u;
+  __syncthreads();
+  if (!ctl[CTL_LAST]) return;
+  __threadfence();
+  if (sh.stack == 0) frame_codebook(p, s, a, sh, sm, f, sw);
+  else if (threadIdx.x == 0) flag_release(sw.stage + f, kStageStreamed);
+}
+// The item of a ticket after the streaming ones (c counted from the first of them).
+__device__ __forceinline__ void later_item(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
+                                           const SyncWords& sw, unsigned char* sm, uint32_t c) {
+  const uint32_t n = a.n_frames;
+  if (c < n * sh.stack) {
+    const uint32_t f = c / sh.stack;
+    stack_item(p, s, a, sh, sm, f, c - f * sh.stack, sw);
+    return;
+  }
+  uint32_t g, grp;
+  if (coding_item(sh, n, c - n * sh.stack, g, grp)) write_item(p, s, a, sh, sm, g, grp, sw);
+  else size_item(p, s, a, sh, sm, g, grp, sw);
+}
 // One ticket t < fused_tickets.  Every thread of the CTA calls it.  k_fused keeps
 // this body inline in its own loop (the same code, which compiled with fewer
 // register spills there).
@@ -1874,23 +1918,12 @@ template <int kG>
 __device__ __forceinline__ void fused_ticket(const DevParams& p, const Scratch& s, const PlainArgs& a,
                                              const FusedShape& sh, const SyncWords& sw, unsigned char* sm,
                                              uint32_t t, uint32_t& ring_iter) {
-  uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
   const uint32_t n = a.n_frames, r = t / sh.U, j = t - r * sh.U;
   if (r < n) {
     process_item<2, kG, false>(p, s, a, sh, sm, r, j, sw, ring_iter);  // the multi-job plan keeps to RB = 2, whole panels
-    // publish the item; the CTA that completes the frame builds its codebook
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) ctl[CTL_LAST] = atomicAdd(sw.panel_done + r, 1u) == sh.U - 1 ? 1u : 0u;
-    __syncthreads();
-    if (ctl[CTL_LAST]) {
-      __threadfence();
-      frame_codebook(p, s, a, sh, sm, r, sw);
-    }
+    streamed(p, s, a, sh, sw, sm, r);
   } else {
-    uint32_t g, grp;
-    if (coding_item(sh, n, t - n * sh.U, g, grp)) write_item(p, s, a, sh, sm, g, grp, sw);
-    else size_item(p, s, a, sh, sm, g, grp, sw);
+    later_item(p, s, a, sh, sw, sm, t - n * sh.U);
   }
 }
 
@@ -1946,19 +1979,9 @@ __global__ void __launch_bounds__(kPT, 4) k_fused(DevParams p, Scratch s, PlainA
     const uint32_t r = t / sh.U, j = t - r * sh.U;
     if (r < n) {
       process_item<RB, kG, kBand>(p, s, a, sh, sm, r, j, sw, ring_iter);
-      // publish the item; the CTA that completes the frame builds its codebook
-      __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) ctl[CTL_LAST] = atomicAdd(sw.panel_done + r, 1u) == sh.U - 1 ? 1u : 0u;
-      __syncthreads();
-      if (ctl[CTL_LAST]) {
-        __threadfence();
-        frame_codebook(p, s, a, sh, sm, r, sw);
-      }
+      streamed(p, s, a, sh, sw, sm, r);
     } else {
-      uint32_t g, grp;
-      if (coding_item(sh, n, t - n * sh.U, g, grp)) write_item(p, s, a, sh, sm, g, grp, sw);
-      else size_item(p, s, a, sh, sm, g, grp, sw);
+      later_item(p, s, a, sh, sw, sm, t - n * sh.U);
     }
     __syncthreads();
   }

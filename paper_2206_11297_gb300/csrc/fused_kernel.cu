@@ -53,6 +53,7 @@ static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, ui
   sh.k = min(kMaxK, sh.kG * kGroupCols / NP);
   if ((uint64_t)sh.k * p.H * p.W >= kBlockKey) return false;  // item-local keys stay below the flag
   sh.U = ceil_div(p.P, sh.k);
+  sh.stack = p.dims == 3 ? ceil_div(p.Hb * p.Wb, kStackSlice) : 0u;
   sh.bands = 1;
   sh.band_bins = p.Hb;
   sh.RB = rb;

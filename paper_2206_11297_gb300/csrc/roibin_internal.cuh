@@ -900,6 +900,7 @@ struct FusedShape {
   uint32_t kG;                   // column groups per consumer lane (1, or 2 for panels above 868 columns)
   uint32_t RB;                   // binned rows per streaming step (2 or 3)
   uint32_t stages, stage_bytes;  // TMA ring: slots, bytes per slot (2 RB raw rows of k panels)
+  uint32_t stack;                // stack items per frame (3-D predictor; else 0)
   uint32_t bands, band_bins;     // row bands a panel is cut into (1: whole panels), binned rows of each
   uint32_t mask_words;           // words of a prequantisation-outlier slot (one per panel and band)
   uint32_t side;                 // side of the peak-test neighbourhood
