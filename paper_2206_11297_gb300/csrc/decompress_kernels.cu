@@ -68,6 +68,13 @@ __device__ bool read_header(const uint32_t* hdr, const DevParams& p, uint64_t ba
   return ok;
 }
 
+// [2][P] first entry of each panel in the frame's Lorenzo and prequantisation
+// outlier lists (in the compressor's outlier slots, free while decompressing: two
+// words a panel at least).
+__device__ __forceinline__ uint32_t* dec_list_starts(const Scratch& s, const DevParams& p, uint32_t f) {
+  return s.pq_mask + (size_t)f * 2 * p.P;
+}
+
 // parse: one block per frame.  Reads the header and the code lengths (its own,
 // or those of its chunk's head, back_ref frames earlier in the call), builds
 // the canonical decoding tables and the prefix table, checks that both outlier
@@ -206,8 +213,7 @@ __global__ void __launch_bounds__(256) k_dec_parse(DevParams p, Scratch s, DecAr
   for (int list = 0; list < 2; ++list) {
     const uint2* v = reinterpret_cast<const uint2*>(base + (list == 0 ? di.pl.off_lo : di.pl.off_pq));
     const uint32_t n = list == 0 ? di.pl.n_lo : di.pl.n_pq;
-    uint32_t* start = (list == 0 ? reinterpret_cast<uint32_t*>(s.dq) : reinterpret_cast<uint32_t*>(s.bhat)) +
-                      (size_t)f * p.M;
+    uint32_t* start = dec_list_starts(s, p, f) + (list == 0 ? 0 : p.P);
     if (n == 0)
       for (uint32_t q = threadIdx.x; q < p.P; q += blockDim.x) start[q] = 0;
     for (uint32_t e = threadIdx.x; e < n; e += blockDim.x) {
@@ -270,7 +276,7 @@ __global__ void k_dec_rows(DevParams p, Scratch s, DecArgs a) {
 }
 
 // cols: prefix sum down each column of a binned panel, then b^ = fl(q * 2eb)
-// (dequant), or the sums back in place for the 3-D inverse (k_dec_stack).
+// (dequant), or the sums back in place for the 3-D inverse (k_dec_stack_out).
 __global__ void k_dec_cols(DevParams p, Scratch s, DecArgs a, int dequant) {
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
@@ -289,21 +295,69 @@ __global__ void k_dec_cols(DevParams p, Scratch s, DecArgs a, int dequant) {
 }
 
 // stack (3-D inverse, last axis): prefix sum across the panels at each binned
-// position of the 2-D sums, then b^ = fl(q * 2eb).  The three axes' prefix
-// sums commute, so rows, columns, then panels inverts the 3-D predictor.
-__global__ void k_dec_stack(DevParams p, Scratch s, DecArgs a) {
+// position of their 2-D sums, b^ = fl(q * 2eb) and the bin's pixels.  The three
+// axes' prefix sums commute, so rows, columns, then panels inverts the 3-D
+// predictor.  kVec: bin 2 x 2, W % 4 == 0, 16-byte aligned frames: a thread takes
+// two bins and stores a float4 on each of their rows; else a thread takes a pixel
+// column of a binned row.  Four panels' sums are read ahead.  HBM-bound: the sums
+// in and the pixels out, once each; with k_dec_panel<true> it replaces a pass
+// each over the int32 sums for rows, columns, panels and up-sampling: 40 CSPAD-like
+// frames 226 -> 125 us.
+template <bool kVec>
+__global__ void __launch_bounds__(256) k_dec_stack_out(DevParams p, Scratch s, DecArgs a) {
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
-  const uint32_t plane = p.Hb * p.Wb;
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= plane) return;
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, cols = kVec ? p.W / 4 : p.W;
+  const uint32_t i = t / cols, c = t - i * cols;
+  if (i >= p.Hb) return;
   const float two_eb = s.dec_info[f].two_eb;
-  const uint32_t* dq = reinterpret_cast<const uint32_t*>(s.dq + (size_t)f * p.M);
-  float* bh = s.bhat + (size_t)f * p.M;
-  uint32_t q = 0;
-  for (uint32_t pn = 0; pn < p.P; ++pn) {
-    q += dq[(size_t)pn * plane + t];
-    bh[(size_t)pn * plane + t] = __fmul_rn((float)(int32_t)q, two_eb);
+  const uint32_t plane = p.Hb * p.Wb;
+  const uint32_t* dq = reinterpret_cast<const uint32_t*>(s.dq) + (size_t)f * p.M + (size_t)i * p.Wb;
+  const uint32_t r0 = i * p.bh, r1 = min(p.H, r0 + p.bh);
+  float* out = a.out + (size_t)f * p.frame_px + (size_t)r0 * p.W;
+  uint32_t q0 = 0, q1 = 0;
+  constexpr uint32_t U = 4;
+  for (uint32_t p0 = 0; p0 < p.P; p0 += U) {
+    uint2 v[U];
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      v[u] = make_uint2(0u, 0u);
+      if (p0 + u < p.P) {
+        const uint32_t* at = dq + (size_t)(p0 + u) * plane;
+        if (kVec) v[u] = __ldcs(reinterpret_cast<const uint2*>(at) + c);
+        else v[u].x = __ldg(at + c / p.bw);
+      }
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      if (p0 + u >= p.P) break;
+      q0 += v[u].x;
+      q1 += v[u].y;
+      const float b0 = __fmul_rn((float)(int32_t)q0, two_eb), b1 = __fmul_rn((float)(int32_t)q1, two_eb);
+      float* px = out + (size_t)(p0 + u) * p.H * p.W;
+      for (uint32_t r = r0; r < r1; ++r, px += p.W) {
+        if (kVec) __stcs(reinterpret_cast<float4*>(px) + c, make_float4(b0, b0, b1, b1));
+        else __stcs(px + c, b0);
+      }
+    }
+  }
+}
+
+// The prequantisation outliers' pixels, over those of k_dec_stack_out (the lists
+// were checked by the parse step).
+__global__ void k_dec_pq_pixels(DevParams p, Scratch s, DecArgs a) {
+  const uint32_t f = blockIdx.y;
+  if (s.status[f] != ROIBIN_OK) return;
+  const DecInfo& di = s.dec_info[f];
+  const uint2* pq = reinterpret_cast<const uint2*>(a.in + di.base + di.pl.off_pq);
+  const uint32_t plane = p.Hb * p.Wb;
+  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < di.pl.n_pq; e += gridDim.x * blockDim.x) {
+    const uint2 v = pq[e];
+    const uint32_t pn = v.x / plane, b = v.x - pn * plane, i = b / p.Wb, j = b - i * p.Wb;
+    const uint32_t r1 = min(p.H, (i + 1) * p.bh), c1 = min(p.W, (j + 1) * p.bw);
+    float* panel = a.out + (size_t)f * p.frame_px + (size_t)pn * p.H * p.W;
+    for (uint32_t r = i * p.bh; r < r1; ++r)
+      for (uint32_t c = j * p.bw; c < c1; ++c) panel[(size_t)r * p.W + c] = __uint_as_float(v.y);
   }
 }
 
@@ -892,6 +946,8 @@ __device__ __forceinline__ uint32_t place_strip_outliers(const uint2* v, uint32_
 // k_dec_roi then overwrites the pixels of the ROI windows.
 // The 2-D prefix sum wraps modulo 2^32 in any order, so column-then-row equals
 // the row-then-column definition.
+// kSums (3-D predictor): the panel's 2-D sums go to s.dq instead of pixels;
+// k_dec_stack_out adds them up across the panels and writes the pixels.
 // The symbols of the next strip arrive by a 1-D TMA bulk copy (a 16-byte
 // aligned superset of the strip) while the block works on the current one.
 constexpr int kPanelThreads = 256;
@@ -904,6 +960,7 @@ __host__ __device__ inline uint32_t panel_sym_bytes(uint32_t Wb, uint32_t sb) { 
 __host__ __device__ inline uint32_t panel_smem_bytes(uint32_t Wb, uint32_t sb) {
   return panel_sym_offset(Wb, sb) + panel_sym_bytes(Wb, sb) + 16;
 }
+template <bool kSums>
 __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scratch s, DecArgs a, uint32_t sb,
                                                                 uint32_t lg_seg, int vec4) {
   extern __shared__ __align__(16) int32_t sm[];  // carry[Wb], tile[sb][Wb], symbols, mbarrier
@@ -929,8 +986,8 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
   const uint8_t* base = a.in + di.base;
   const uint2* lo = reinterpret_cast<const uint2*>(base + di.pl.off_lo);
   const uint2* pq = reinterpret_cast<const uint2*>(base + di.pl.off_pq);
-  const uint32_t* lo_start = reinterpret_cast<const uint32_t*>(s.dq) + (size_t)f * p.M;
-  const uint32_t* pq_start = reinterpret_cast<const uint32_t*>(s.bhat) + (size_t)f * p.M;
+  const uint32_t* lo_start = dec_list_starts(s, p, f);
+  const uint32_t* pq_start = lo_start + p.P;
   uint32_t lo_cur = lo_start[pn], pq_cur = pq_start[pn];
   const uint32_t lo_end = pn + 1 < p.P ? lo_start[pn + 1] : di.pl.n_lo;
   const uint32_t pq_end = pn + 1 < p.P ? pq_start[pn + 1] : di.pl.n_pq;
@@ -1032,8 +1089,28 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
     }
     __syncthreads();
     // prequantisation outliers in this strip (the same answer in every thread)
-    const bool any_pq = pq_cur != pq_end && pq[pq_cur].x < sb1;
-    if (vec4 && !any_pq) {
+    const bool any_pq = !kSums && pq_cur != pq_end && pq[pq_cur].x < sb1;
+    if constexpr (kSums) {
+      // a warp per row, two bins a lane, as below
+      uint32_t* out = reinterpret_cast<uint32_t*>(s.dq) + (size_t)f * p.M + sb0;
+      for (uint32_t i = threadIdx.x >> 5; i < nr; i += kPanelThreads / 32) {
+        const uint32_t* row = tile + i * Wb;
+        uint32_t run = 0;
+        for (uint32_t j0 = 0; j0 < Wb; j0 += 64) {
+          const uint32_t j = j0 + 2 * lane;
+          const uint32_t x = j < Wb ? row[j] : 0u, y = j + 1 < Wb ? row[j + 1] : 0u;
+          const uint32_t incl = warp_incl_scan(x + y);
+          const uint32_t q0 = run + incl - y, q1 = run + incl;
+          run += __shfl_sync(0xffffffffu, incl, 31);
+          if (vec4) {  // even rows and panels: 8-byte aligned
+            if (j < Wb) *reinterpret_cast<uint2*>(out + i * Wb + j) = make_uint2(q0, q1);
+          } else {
+            if (j < Wb) out[i * Wb + j] = q0;
+            if (j + 1 < Wb) out[i * Wb + j + 1] = q1;
+          }
+        }
+      }
+    } else if (vec4 && !any_pq) {
       // a warp per row: row prefix sums by shuffles, two bins a lane, and from the
       // registers b^ = fl(q * 2eb) straight to the row's pixels (one float4 on each
       // of its pixel rows; streaming stores: the kernel never reads them back)
@@ -1111,7 +1188,7 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
     }
     __syncthreads();
   }
-  if (lo_cur != lo_end || pq_cur != pq_end) bad = true;
+  if (lo_cur != lo_end || (!kSums && pq_cur != pq_end)) bad = true;
   if (timed_out) {
     if (threadIdx.x == 0) s.status[f] = ROIBIN_ERR_TIMEOUT;
     return;
@@ -1191,18 +1268,24 @@ cudaError_t launch_dec_rows(const DevParams& p, const Scratch& s, const DecArgs&
   k_dec_rows<<<grid, 256, 0, st>>>(p, s, a);
   return cudaGetLastError();
 }
-cudaError_t launch_dec_cols(const DevParams& p, const Scratch& s, const DecArgs& a, bool dequant, cudaStream_t st) {
+cudaError_t launch_dec_cols(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   dim3 grid(ceil_div(p.P * p.Wb, 128), a.n_frames);
-  k_dec_cols<<<grid, 128, 0, st>>>(p, s, a, dequant ? 1 : 0);
+  k_dec_cols<<<grid, 128, 0, st>>>(p, s, a, p.dims == 2 ? 1 : 0);
   return cudaGetLastError();
 }
 cudaError_t launch_dec_carry(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  if (p.dims == 3) {
-    dim3 grid(ceil_div(p.Hb * p.Wb, 256), a.n_frames);
-    k_dec_stack<<<grid, 256, 0, st>>>(p, s, a);
-  } else {
-    k_dec_chain<<<a.n_frames, kChainThreads, 0, st>>>(p, s, a);
-  }
+  k_dec_chain<<<a.n_frames, kChainThreads, 0, st>>>(p, s, a);
+  return cudaGetLastError();
+}
+cudaError_t launch_dec_stack_out(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
+  const bool vec = p.bh == 2 && p.bw == 2 && (p.W % 4) == 0 && (reinterpret_cast<uintptr_t>(a.out) % 16) == 0;
+  const dim3 grid(ceil_div(p.Hb * (vec ? p.W / 4 : p.W), 256), a.n_frames);
+  if (vec) k_dec_stack_out<true><<<grid, 256, 0, st>>>(p, s, a);
+  else k_dec_stack_out<false><<<grid, 256, 0, st>>>(p, s, a);
+  return cudaGetLastError();
+}
+cudaError_t launch_dec_pq_pixels(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
+  k_dec_pq_pixels<<<dim3(16, a.n_frames), 256, 0, st>>>(p, s, a);
   return cudaGetLastError();
 }
 cudaError_t launch_dec_pq(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
@@ -1236,17 +1319,19 @@ uint32_t dec_panel_rows(const DevParams& p) {
   const uint32_t strips = ceil_div(p.Hb, most);
   return ceil_div(p.Hb, strips);
 }
-cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
+cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs& a, bool sums, cudaStream_t st) {
   const uint32_t sb = dec_panel_rows(p);
   if (sb == 0) return cudaErrorInvalidValue;
-  const bool vec4 = p.bw == 2 && (p.W % 4) == 0 && (reinterpret_cast<uintptr_t>(a.out) % 16) == 0;
+  // sums: pairs of them are stored together when the binned rows are even
+  const bool vec4 = sums ? (p.Wb % 2) == 0 : p.bw == 2 && (p.W % 4) == 0 && (reinterpret_cast<uintptr_t>(a.out) % 16) == 0;
   const size_t smem = panel_smem_bytes(p.Wb, sb);
   // row segments: the most lanes per row that still give every row of a strip
   // its own lanes (sb <= 32, so at least 8)
   uint32_t lg_seg = 5;
   while (lg_seg > 0 && (sb << lg_seg) > (uint32_t)kPanelThreads) --lg_seg;
   dim3 grid(p.P, a.n_frames);
-  k_dec_panel<<<grid, kPanelThreads, smem, st>>>(p, s, a, sb, lg_seg, vec4 ? 1 : 0);
+  if (sums) k_dec_panel<true><<<grid, kPanelThreads, smem, st>>>(p, s, a, sb, lg_seg, vec4 ? 1 : 0);
+  else k_dec_panel<false><<<grid, kPanelThreads, smem, st>>>(p, s, a, sb, lg_seg, vec4 ? 1 : 0);
   return cudaGetLastError();
 }
 cudaError_t launch_roi_mask(const DevParams& p, const uint16_t* peaks, const uint32_t* npeaks, uint32_t n,

@@ -892,22 +892,35 @@ int roibin_decompress(roibin_ctx* ctx, const uint8_t* d_in, uint64_t in_bytes, c
   if (resolved_dec_path(ctx) == ROIBIN_DEC_PANEL) {
     if ((e = timed(ctx, K_DEC_DECODE, st, [&] { return launch_dec_decode(p, s, a, false, st); })) != cudaSuccess)
       return cuda_status(e);
-    if ((e = timed(ctx, K_DEC_PANEL, st, [&] { return launch_dec_panel(p, s, a, st); })) != cudaSuccess)
+    ctx->last_launches++;  // the decode step is two kernels: sparse frames, then dense ones
+    if ((e = timed(ctx, K_DEC_PANEL, st, [&] { return launch_dec_panel(p, s, a, false, st); })) != cudaSuccess)
       return cuda_status(e);
     if ((e = timed(ctx, K_DEC_ROI, st, [&] { return launch_dec_roi(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
     return dec_finish(ctx, a, st);
   }
-  if ((e = timed(ctx, K_DEC_DECODE, st, [&] { return launch_dec_decode(p, s, a, true, st); })) != cudaSuccess) return cuda_status(e);
-  if ((e = timed(ctx, K_DEC_LORENZO, st, [&] { return launch_dec_lorenzo(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
-  if ((e = timed(ctx, K_DEC_ROWS, st, [&] { return launch_dec_rows(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
-  // the inverse predictor after the row sums: down the columns (2-D), then
-  // across the panels (3-D); or the carry from row to row (1-D)
-  if (p.dims >= 2)
-    if ((e = timed(ctx, K_DEC_COLS, st, [&] { return launch_dec_cols(p, s, a, p.dims == 2, st); })) != cudaSuccess)
-      return cuda_status(e);
-  if (p.dims != 2)
-    if ((e = timed(ctx, K_DEC_CARRY, st, [&] { return launch_dec_carry(p, s, a, st); })) != cudaSuccess)
-      return cuda_status(e);
+  if (p.dims == 3 && dec_panel_rows(p)) {
+    // the 3-D predictor: the panels' 2-D sums by the panel kernel
+    if ((e = timed(ctx, K_DEC_DECODE, st, [&] { return launch_dec_decode(p, s, a, false, st); })) != cudaSuccess) return cuda_status(e);
+    ctx->last_launches++;  // the decode step is two kernels: sparse frames, then dense ones
+    if ((e = timed(ctx, K_DEC_PANEL, st, [&] { return launch_dec_panel(p, s, a, true, st); })) != cudaSuccess) return cuda_status(e);
+  } else {
+    if ((e = timed(ctx, K_DEC_DECODE, st, [&] { return launch_dec_decode(p, s, a, true, st); })) != cudaSuccess) return cuda_status(e);
+    if ((e = timed(ctx, K_DEC_LORENZO, st, [&] { return launch_dec_lorenzo(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
+    if ((e = timed(ctx, K_DEC_ROWS, st, [&] { return launch_dec_rows(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
+    // the inverse predictor after the row sums: down the columns (2-D and 3-D), or
+    // the carry from row to row (1-D)
+    if (p.dims >= 2)
+      e = timed(ctx, K_DEC_COLS, st, [&] { return launch_dec_cols(p, s, a, st); });
+    else
+      e = timed(ctx, K_DEC_CARRY, st, [&] { return launch_dec_carry(p, s, a, st); });
+    if (e != cudaSuccess) return cuda_status(e);
+  }
+  if (p.dims == 3) {  // across the panels, straight to pixels
+    if ((e = timed(ctx, K_DEC_CARRY, st, [&] { return launch_dec_stack_out(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
+    if ((e = timed(ctx, K_DEC_PQ, st, [&] { return launch_dec_pq_pixels(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
+    if ((e = timed(ctx, K_DEC_ROI, st, [&] { return launch_dec_roi(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
+    return dec_finish(ctx, a, st);
+  }
   if ((e = timed(ctx, K_DEC_PQ, st, [&] { return launch_dec_pq(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
   if ((e = timed(ctx, K_DEC_UPSAMPLE, st, [&] { return launch_dec_upsample(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
   if ((e = timed(ctx, K_DEC_ROI, st, [&] { return launch_dec_roi(p, s, a, st); })) != cudaSuccess) return cuda_status(e);

@@ -98,10 +98,8 @@ struct Scratch {
   FramePlan* plan;        // [n]
   int32_t* status;        // [n]
   // decompression (aliases lo_delta / pq_bits: a context runs one call at a time)
-  int32_t* dq;            // [n][M] delta, then q (multi-pass); the panel path keeps
-                          // [n][P] first Lorenzo outlier of each panel at dq + f * M
-  float* bhat;            // [n][M] (multi-pass); the panel path keeps [n][P] first
-                          // prequantisation outlier of each panel at bhat + f * M
+  int32_t* dq;            // [n][M] delta, then q (multi-pass); 2-D sums (3-D predictor)
+  float* bhat;            // [n][M] (multi-pass)
   uint32_t* dec_table;    // [n][kDecTableWords] canonical decoding tables
   uint32_t* dec_zero;     // [n] code-0 symbols decoded
   DecInfo* dec_info;      // [n]
@@ -1030,7 +1028,7 @@ cudaError_t launch_dec_parse(const DevParams& p, const Scratch& s, const DecArgs
 cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArgs& a, bool deltas, cudaStream_t st);
 cudaError_t launch_dec_lorenzo(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_dec_rows(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
-cudaError_t launch_dec_cols(const DevParams& p, const Scratch& s, const DecArgs& a, bool dequant, cudaStream_t st);
+cudaError_t launch_dec_cols(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_dec_carry(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_dec_pq(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_dec_upsample(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
@@ -1042,7 +1040,10 @@ cudaError_t launch_dec_finish(const Scratch& s, const DecArgs& a, cudaStream_t s
 // the panel path: decode through the prefix table into symbols, then one block
 // per (frame, panel) rebuilds the panel strip by strip
 uint32_t dec_panel_rows(const DevParams& p);  // binned rows per strip; 0: panel path unavailable
-cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
+// sums (3-D predictor): the panels' 2-D sums to s.dq, for launch_dec_stack_out, instead of pixels
+cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs& a, bool sums, cudaStream_t st);
+cudaError_t launch_dec_stack_out(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
+cudaError_t launch_dec_pq_pixels(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_roi_mask(const DevParams& p, const uint16_t* peaks, const uint32_t* npeaks,
                             uint32_t n, uint8_t* mask, cudaStream_t st);
 cudaError_t launch_pack(const uint8_t* src, uint64_t stride, const uint64_t* sizes, const uint64_t* offsets,

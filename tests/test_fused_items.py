@@ -64,3 +64,19 @@ def test_listed_chunks(others, last, kind):
     assert np.abs(f).max() < 2 ** 24
     params = rb.default_params(amax_thr=1e30, max_peaks=0)
     assert_parity(f[None], params, rb.PATH_FUSED, check_decompress=False)
+
+
+@pytest.mark.parametrize("path", [rb.PATH_FUSED, rb.PATH_PLAIN])
+@pytest.mark.parametrize("geom", [(70, 9, 36), (33, 4, 8), (3, 2, 1736)])
+def test_panel_stacks(geom, path):
+    # more panels than a stack item holds at once; slices cut inside a panel
+    f = frames_of(geom, 2, seed=sum(geom))
+    f[0].reshape(-1)[::11] = 4000.0   # outliers and escapes on both sides of a slice
+    assert_parity(f, rb.default_params(atot_thr=300.0, lorenzo_dims=3, abs_eb=1.0, max_peaks=8192), path)
+
+
+@pytest.mark.parametrize("geom,bin_w", [((3, 5, 8200), 2), ((4, 6, 27), 2), ((2, 7, 30), 3)])
+def test_stack_decompression_of_odd_and_wide_rows(geom, bin_w):
+    f = frames_of(geom, 2, seed=sum(geom))
+    f[1].reshape(-1)[::97] = 1e30
+    assert_parity(f, rb.default_params(atot_thr=300.0, lorenzo_dims=3, bin_w=bin_w), rb.PATH_PLAIN)
