@@ -32,7 +32,6 @@
 namespace roibin {
 
 constexpr uint32_t kRoiWarps = 8;   // windows per block and pass (coding kernels)
-constexpr uint32_t kRoiBlocks = 8;  // blocks per frame (coding kernels)
 
 __device__ __forceinline__ uint32_t roi_order(float x) {
   const uint32_t u = __float_as_uint(x);
@@ -53,6 +52,27 @@ __device__ __forceinline__ bool roi_frame_live(const PlainArgs& a, uint32_t f) {
   return st == ROIBIN_OK || (st == ROIBIN_ERR_CAPACITY && a.frame_bytes[f] > 0);
 }
 
+// (row, column) of element e = lane, lane + 32, ... of a window w wide, stepped by 32
+// elements at a time (two divisions in all).
+struct RoiStep {
+  int i, j, step_i, step_j, w;
+  __device__ __forceinline__ explicit RoiStep(int w_) : w(w_) {
+    const int lane = (int)lane_id();
+    i = lane / w;
+    j = lane - i * w;
+    step_i = 32 / w;
+    step_j = 32 - step_i * w;
+  }
+  __device__ __forceinline__ void next() {
+    i += step_i;
+    j += step_j;
+    if (j >= w) {
+      j -= w;
+      ++i;
+    }
+  }
+};
+
 // A warp stages window k of frame f (its order bits; 0.0f past the panel edge).
 __device__ __forceinline__ void roi_stage(const DevParams& p, const PlainArgs& a, const Scratch& s, uint32_t f,
                                           uint32_t k, uint32_t* mm) {
@@ -61,17 +81,18 @@ __device__ __forceinline__ void roi_stage(const DevParams& p, const PlainArgs& a
   const int r0 = (int)(rem / p.W) - p.roi_h / 2, c0 = (int)(rem % p.W) - p.roi_w / 2;
   const float* panel = a.frames + (size_t)f * p.frame_px + (size_t)pn * plane;
   const int win = p.roi_h * p.roi_w, lane = (int)lane_id();
-  for (int base = 0; base < win; base += 12 * 32) {  // 12 loads in flight per lane, then the stores
-    float vals[12];
+  RoiStep at(p.roi_w);
+  for (int base = 0; base < win; base += 10 * 32) {  // 10 loads in flight per lane (a 17 x 17 window), then the stores
+    float vals[10];
 #pragma unroll
-    for (int u = 0; u < 12; ++u) {
-      const int e = base + u * 32 + lane;
-      const int rr = r0 + e / p.roi_w, cc = c0 + e % p.roi_w;
-      const bool in = e < win && rr >= 0 && rr < (int)p.H && cc >= 0 && cc < (int)p.W;
+    for (int u = 0; u < 10; ++u) {
+      const int rr = r0 + at.i, cc = c0 + at.j;
+      const bool in = base + u * 32 + lane < win && rr >= 0 && rr < (int)p.H && cc >= 0 && cc < (int)p.W;
       vals[u] = in ? __ldg(panel + (size_t)rr * p.W + cc) : 0.0f;
+      at.next();
     }
 #pragma unroll
-    for (int u = 0; u < 12; ++u) {
+    for (int u = 0; u < 10; ++u) {
       const int e = base + u * 32 + lane;
       if (e < win) mm[e] = roi_order(vals[u]);
     }
@@ -79,11 +100,11 @@ __device__ __forceinline__ void roi_stage(const DevParams& p, const PlainArgs& a
   __syncwarp();
 }
 
-// Folded residual of element e of a staged window of width w.
-__device__ __forceinline__ uint32_t roi_residual(const uint32_t* mm, int e, int w) {
-  const int i = e / w, j = e - i * w;
+// Folded residual of element e = at.i * w + at.j of a staged window of width w.
+__device__ __forceinline__ uint32_t roi_residual(const uint32_t* mm, int e, const RoiStep& at) {
   uint32_t pred = 0x80000000u;
-  if (e > 0) pred = (i > 0 ? mm[e - w] : 0u) + (j > 0 ? mm[e - 1] : 0u) - (i > 0 && j > 0 ? mm[e - w - 1] : 0u);
+  if (e > 0)
+    pred = (at.i > 0 ? mm[e - at.w] : 0u) + (at.j > 0 ? mm[e - 1] : 0u) - (at.i > 0 && at.j > 0 ? mm[e - at.w - 1] : 0u);
   return roi_fold((int32_t)(mm[e] - pred));
 }
 
@@ -102,9 +123,10 @@ __global__ void __launch_bounds__(kRoiWarps * 32) k_roi_classes(DevParams p, Scr
   for (uint32_t k = blockIdx.x * kRoiWarps + warp; k < n; k += gridDim.x * kRoiWarps) {
     for (uint32_t c = lane; c < kRoiClasses; c += 32) wc[warp][c] = 0;
     roi_stage(p, a, s, f, k, mm);
-    for (uint32_t e0 = 0; e0 < win; e0 += 32) {  // lanes with the same class add once
+    RoiStep at(p.roi_w);
+    for (uint32_t e0 = 0; e0 < win; e0 += 32, at.next()) {  // lanes with the same class add once
       const uint32_t e = e0 + lane;
-      const uint32_t c = e < win ? roi_class(roi_residual(mm, (int)e, p.roi_w)) : kRoiClasses;
+      const uint32_t c = e < win ? roi_class(roi_residual(mm, (int)e, at)) : kRoiClasses;
       const uint32_t peers = __match_any_sync(0xffffffffu, c);
       if (c < kRoiClasses && (peers & lanemask_lt()) == 0) atomicAdd(&wc[warp][c], (uint32_t)__popc(peers));
     }
@@ -254,12 +276,13 @@ __global__ void __launch_bounds__(kRoiWarps * 32) k_roi_write(DevParams p, Scrat
     for (uint32_t w = lane; w < w1 - w0; w += 32) wb[w] = 0;  // every bit lands below w1 - w0
     __syncwarp();
     uint32_t pos = 0;  // bits of the window before this round
-    for (uint32_t e0 = 0; e0 < win; e0 += 32) {
+    RoiStep step(p.roi_w);
+    for (uint32_t e0 = 0; e0 < win; e0 += 32, step.next()) {
       const uint32_t e = e0 + lane;
       uint64_t v = 0;
       uint32_t L = 0;
       if (e < win) {
-        const uint32_t z = roi_residual(mm, (int)e, p.roi_w), c = roi_class(z);
+        const uint32_t z = roi_residual(mm, (int)e, step), c = roi_class(z);
         L = len[c];
         v = cw[c];
         if (c > 1) {  // the codeword, then the c - 1 bits below the leading one
@@ -304,7 +327,12 @@ cudaError_t launch_roi_code(const DevParams& p, const Scratch& s, const PlainArg
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(s.roi_hist, 0, sizeof(uint32_t) * kRoiClasses * a.n_frames, st);
   if (e != cudaSuccess) return e;
-  const dim3 grid(kRoiBlocks, a.n_frames);
+  // windows are independent: about 4,096 blocks in all (several waves of the 152 SMs),
+  // at least 8 and at most 128 a frame.  The three kernels on 30 epix10k frames of
+  // 3,600 windows: 701 us with 8 blocks a frame, 424 us so, 348 us with the windows'
+  // elements stepped instead of divided (RoiStep).
+  const uint32_t per_frame = std::max<uint32_t>(8, std::min<uint32_t>(128, 4096 / a.n_frames));
+  const dim3 grid(std::min<uint32_t>(per_frame, ceil_div(std::max<uint32_t>(p.max_peaks, 1), kRoiWarps)), a.n_frames);
   k_roi_classes<<<grid, kRoiWarps * 32, smem, st>>>(p, s, a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_roi_plan<<<a.n_frames, kRoiPlanThreads, sizeof(HuffSmem), st>>>(p, s, a);
