@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256) k_dec_parse(DevParams p, Scratch s, DecAr
   __shared__ int ok;
   __shared__ uint64_t len_at;  // byte offset of the code lengths in the input
   __shared__ uint32_t cnt[34], first[34], idx0[34];
-  __shared__ uint8_t lens[kMaxSymbols];
+  __shared__ __align__(4) uint8_t lens[kMaxSymbols];
   __shared__ uint16_t order[kMaxSymbols];
   __shared__ uint32_t nsym_s;
   __shared__ int sparse;
@@ -181,28 +181,32 @@ __global__ void __launch_bounds__(256) k_dec_parse(DevParams p, Scratch s, DecAr
   for (uint32_t k = threadIdx.x; k < nsym_s; k += blockDim.x) {
     const uint32_t L = lens[k];
     if (L == 0 || L > 32) continue;
+    const uint32_t same = L * 0x01010101u;  // four lengths a word
     uint32_t rank = 0;
-    for (uint32_t j = 0; j < k; ++j) rank += lens[j] == L;
+    for (uint32_t j = 0; j + 4 <= k; j += 4)
+      rank += __popc(__vcmpeq4(*reinterpret_cast<const uint32_t*>(lens + j), same)) >> 3;
+    for (uint32_t j = k & ~3u; j < k; ++j) rank += lens[j] == L;
     tab[102 + idx0[L] + rank] = k;
     order[idx0[L] + rank] = (uint16_t)k;
   }
   __syncthreads();
-  // prefix table: the shortest code that matches the top bits of the entry,
-  // as the bit-serial decoder would find it
+  // prefix table.  Canonical codes grow with their length: entry e starts with a
+  // code of at most L bits when it is below end[L], the first 12-bit value past
+  // those codes, so its code's length is 1 + the ends it has reached.
   if (ok) {
+    uint32_t end[kDecLutBits + 1];
+    end[0] = 0;
+#pragma unroll
+    for (uint32_t L = 1; L <= kDecLutBits; ++L) end[L] = cnt[L] ? (first[L] + cnt[L]) << (kDecLutBits - L) : end[L - 1];
     for (uint32_t w = threadIdx.x; w < kDecLutWords; w += blockDim.x) {
       uint32_t word = 0;
+#pragma unroll
       for (uint32_t h = 0; h < 2; ++h) {
         const uint32_t e = 2 * w + h;
-        uint32_t ent = 0;
-        for (uint32_t L = 1; L <= kDecLutBits; ++L) {
-          const uint32_t code = e >> (kDecLutBits - L);
-          if (cnt[L] && code >= first[L] && code - first[L] < cnt[L]) {
-            ent = (L << 10) | order[idx0[L] + code - first[L]];
-            break;
-          }
-        }
-        word |= ent << (16 * h);
+        uint32_t L = 1;
+#pragma unroll
+        for (uint32_t l = 1; l <= kDecLutBits; ++l) L += e >= end[l];
+        if (L <= kDecLutBits) word |= ((L << 10) | order[idx0[L] + (e >> (kDecLutBits - L)) - first[L]]) << (16 * h);
       }
       tab[kDecCanonWords + w] = word;
     }
@@ -960,9 +964,14 @@ __host__ __device__ inline uint32_t panel_sym_bytes(uint32_t Wb, uint32_t sb) { 
 __host__ __device__ inline uint32_t panel_smem_bytes(uint32_t Wb, uint32_t sb) {
   return panel_sym_offset(Wb, sb) + panel_sym_bytes(Wb, sb) + 16;
 }
+// A panel's rows may be split over blocks of `rows` binned rows (a multiple of sb),
+// when a small batch has too few panels: a block then starts from the column sums
+// of all rows above its own, taken from the frame's symbols (a sparse frame's
+// lists, or a thread per column over the symbol array).
+// One CSPAD-like frame: 26 -> 7.4 us.
 template <bool kSums>
 __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scratch s, DecArgs a, uint32_t sb,
-                                                                uint32_t lg_seg, int vec4) {
+                                                                uint32_t rows, uint32_t lg_seg, int vec4) {
   extern __shared__ __align__(16) int32_t sm[];  // carry[Wb], tile[sb][Wb], symbols, mbarrier
   __shared__ int go;
   const uint32_t pn = blockIdx.x, f = blockIdx.y;
@@ -989,8 +998,25 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
   const uint32_t* lo_start = dec_list_starts(s, p, f);
   const uint32_t* pq_start = lo_start + p.P;
   uint32_t lo_cur = lo_start[pn], pq_cur = pq_start[pn];
-  const uint32_t lo_end = pn + 1 < p.P ? lo_start[pn + 1] : di.pl.n_lo;
-  const uint32_t pq_end = pn + 1 < p.P ? pq_start[pn + 1] : di.pl.n_pq;
+  uint32_t lo_end = pn + 1 < p.P ? lo_start[pn + 1] : di.pl.n_lo;
+  uint32_t pq_end = pn + 1 < p.P ? pq_start[pn + 1] : di.pl.n_pq;
+  const uint32_t row0 = blockIdx.z * rows, row1 = min(Hb, row0 + rows);  // the block's binned rows
+  const uint32_t lo_first = lo_cur;
+  if (gridDim.z > 1) {  // the block's part of the panel's outliers
+    auto below = [&](const uint2* v, uint32_t from, uint32_t to, uint32_t bin) {  // first entry at or past bin
+      while (from < to) {
+        const uint32_t mid = (from + to) >> 1;
+        if (v[mid].x < bin) from = mid + 1;
+        else to = mid;
+      }
+      return from;
+    };
+    const uint32_t b0 = pb + row0 * Wb, b1 = pb + row1 * Wb;
+    lo_end = below(lo, lo_cur, lo_end, b1);
+    lo_cur = below(lo, lo_cur, lo_end, b0);
+    pq_end = below(pq, pq_cur, pq_end, b1);
+    pq_cur = below(pq, pq_cur, pq_end, b0);
+  }
   uint32_t* carry = reinterpret_cast<uint32_t*>(sm);
   uint32_t* tile = carry + Wb;
   float* tilef = reinterpret_cast<float*>(tile);
@@ -1002,7 +1028,7 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
   // strip r0's symbols: bytes [2 (pb + r0 Wb), 2 (pb + (r0 + nr) Wb)) of fsym,
   // copied from the 16-byte boundary below to the one above
   auto fetch = [&](uint32_t r0) {
-    const uint32_t nr = min(sb, Hb - r0);
+    const uint32_t nr = min(sb, row1 - r0);
     const uint32_t b0 = 2 * (pb + r0 * Wb), b1 = 2 * (pb + (r0 + nr) * Wb);
     const uint32_t a0 = b0 & ~15u, a1 = (b1 + 15) & ~15u;
     fence_proxy_async();
@@ -1020,7 +1046,7 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
   const uint32_t zsym = s.dec_table[(size_t)f * kDecTableWords + 102];
   const uint32_t fillv = zsym ? (uint32_t)((int32_t)zsym - R) : (uint32_t)kSentinel;
   const uint32_t* counts = dec_list_count(s, p, f);
-  if (threadIdx.x == 0 && !sparse) fetch(0);
+  if (threadIdx.x == 0 && !sparse) fetch(row0);
   uint32_t phase = 0;
   bool timed_out = false;  // uniform: set after a barrier
   float* panel = a.out + (size_t)f * p.frame_px + (size_t)pn * H * W;
@@ -1032,11 +1058,46 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
   const uint32_t W4 = W / 4;
   const uint32_t dr = vec4 ? blockDim.x / W4 : 0, dc = vec4 ? blockDim.x - dr * W4 : 0;
   bool bad = false;
-  for (uint32_t j = threadIdx.x; j < Wb; j += blockDim.x) carry[j] = 0;
   const uint32_t lane = lane_id();
+  // column sums of the rows above the block's
+  const uint32_t above = pb + row0 * Wb;  // bins pb .. above - 1
+  if (sparse || row0 == 0) {
+    for (uint32_t j = threadIdx.x; j < Wb; j += blockDim.x) carry[j] = fillv * row0;
+    __syncthreads();
+    if (row0 > 0) {
+      // the listed symbols in place of the fill; a code 0's value is its outlier's
+      for (uint32_t k = pb / kChunk; k <= (above - 1) / kChunk; ++k) {
+        const uint32_t* list = dec_list(s, p, f, k);
+        const uint32_t cnt = min(counts[k], kDecSparseMax), kb = k * kChunk;
+        for (uint32_t e = threadIdx.x; e < cnt; e += blockDim.x) {
+          const uint32_t v = list[e], x = kb + (v >> 16), u = v & 0xFFFFu;
+          if (x >= pb && x < above)
+            atomicAdd(carry + (x - pb) % Wb, (u ? (uint32_t)((int32_t)u - R) : (uint32_t)kSentinel) - fillv);
+        }
+      }
+    }
+  } else {
+    const uint16_t* u16 = reinterpret_cast<const uint16_t*>(fsym) + pb;
+    for (uint32_t j = threadIdx.x; j < Wb; j += blockDim.x) {
+      uint32_t q = 0;
+#pragma unroll 8
+      for (uint32_t i = 0; i < row0; ++i) {
+        const uint32_t u = __ldg(u16 + (size_t)i * Wb + j);
+        q += u ? (uint32_t)((int32_t)u - R) : (uint32_t)kSentinel;
+      }
+      carry[j] = q;
+    }
+    __syncthreads();
+  }
+  if (row0 > 0)  // outliers above: the sentinel's value goes
+    for (uint32_t e = lo_first + threadIdx.x; e < lo_cur; e += blockDim.x) {
+      const uint2 x = lo[e];
+      if (x.x >= pb) atomicAdd(carry + (x.x - pb) % Wb, x.y - (uint32_t)kSentinel);
+      else bad = true;
+    }
   __syncthreads();
-  for (uint32_t r0 = 0; r0 < Hb; r0 += sb) {
-    const uint32_t nr = min(sb, Hb - r0), nb = nr * Wb;
+  for (uint32_t r0 = row0; r0 < row1; r0 += sb) {
+    const uint32_t nr = min(sb, row1 - r0), nb = nr * Wb;
     const uint32_t sb0 = pb + r0 * Wb, sb1 = sb0 + nb;
     // symbols -> deltas (code 0: sentinel until its outlier arrives)
     if (sparse) {
@@ -1069,7 +1130,7 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
         break;
       }
       // the buffer is free: the next strip's symbols come in behind this one
-      if (threadIdx.x == 0 && r0 + sb < Hb) fetch(r0 + sb);
+      if (threadIdx.x == 0 && r0 + sb < row1) fetch(r0 + sb);
     }
     if (lo_cur != lo_end)
       lo_cur = place_strip_outliers(lo, lo_cur, lo_end, sb1, [&](uint32_t x, uint32_t y) {
@@ -1320,8 +1381,18 @@ uint32_t dec_panel_rows(const DevParams& p) {
   return ceil_div(p.Hb, strips);
 }
 cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs& a, bool sums, cudaStream_t st) {
-  const uint32_t sb = dec_panel_rows(p);
+  uint32_t sb = dec_panel_rows(p);
   if (sb == 0) return cudaErrorInvalidValue;
+  // few panels: strips of fewer rows, a block each, until about four blocks an SM
+  // have work (at least four rows, as every block reads the symbols above its own)
+  uint32_t rows = p.Hb;
+  const uint32_t panels = p.P * a.n_frames;
+  if (panels < 304) {
+    const uint32_t parts = std::max<uint32_t>(1, std::min<uint32_t>(608 / panels, p.Hb / 4));
+    rows = ceil_div(p.Hb, parts);
+    sb = ceil_div(rows, ceil_div(rows, sb));
+    rows = ceil_div(rows, sb) * sb;
+  }
   // sums: pairs of them are stored together when the binned rows are even
   const bool vec4 = sums ? (p.Wb % 2) == 0 : p.bw == 2 && (p.W % 4) == 0 && (reinterpret_cast<uintptr_t>(a.out) % 16) == 0;
   const size_t smem = panel_smem_bytes(p.Wb, sb);
@@ -1329,9 +1400,9 @@ cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs
   // its own lanes (sb <= 32, so at least 8)
   uint32_t lg_seg = 5;
   while (lg_seg > 0 && (sb << lg_seg) > (uint32_t)kPanelThreads) --lg_seg;
-  dim3 grid(p.P, a.n_frames);
-  if (sums) k_dec_panel<true><<<grid, kPanelThreads, smem, st>>>(p, s, a, sb, lg_seg, vec4 ? 1 : 0);
-  else k_dec_panel<false><<<grid, kPanelThreads, smem, st>>>(p, s, a, sb, lg_seg, vec4 ? 1 : 0);
+  dim3 grid(p.P, a.n_frames, ceil_div(p.Hb, rows));
+  if (sums) k_dec_panel<true><<<grid, kPanelThreads, smem, st>>>(p, s, a, sb, rows, lg_seg, vec4 ? 1 : 0);
+  else k_dec_panel<false><<<grid, kPanelThreads, smem, st>>>(p, s, a, sb, rows, lg_seg, vec4 ? 1 : 0);
   return cudaGetLastError();
 }
 cudaError_t launch_roi_mask(const DevParams& p, const uint16_t* peaks, const uint32_t* npeaks, uint32_t n,
