@@ -4,7 +4,7 @@
 //   parse (header, layout, decoding tables) -> decode (chunk-parallel
 //   canonical Huffman) -> lorenzo outliers -> row prefix sums -> column prefix
 //   sums + dequantisation -> prequantisation outliers -> up-sampling -> ROI
-//   restoration -> status
+//   windows and status (k_dec_windows, roi_coder.cu)
 //
 // Every index taken from the stream is bounds-checked; a failed check marks
 // the frame ROIBIN_ERR_CORRUPT_STREAM and skips the access.
@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(256) k_dec_parse(DevParams p, Scratch s, DecAr
   DecInfo di = {};
   if (threadIdx.x == 0) {
     s.dec_zero[f] = 0;
+    s.thr_count[f] = 0;  // blocks of k_dec_windows done with the frame
     ok = 1;
     const uint64_t base = a.offsets[f];
     if ((base & 15u) != 0 || base + kHeaderBytes > a.in_bytes) ok = 0;
@@ -445,62 +446,6 @@ __global__ void k_dec_upsample(DevParams p, Scratch s, DecArgs a, int vec4) {
     const uint32_t rowg = (uint32_t)(e / p.W), c = (uint32_t)(e - (uint64_t)rowg * p.W);
     const uint32_t pn = rowg / p.H, r = rowg - pn * p.H;
     out[e] = bh[((size_t)pn * p.Hb + r / p.bh) * p.Wb + c / p.bw];
-  }
-}
-
-// One warp writes the in-panel pixels of the roi_h x roi_w window `src`, centred
-// on (r, c), into `panel`.  Ten loads a lane are in flight before the stores, so a
-// 17 x 17 window costs one round trip; (row, column) of the lane's elements are
-// stepped, not divided.
-__device__ __forceinline__ void warp_restore_roi(const float* __restrict__ src, int roi_h, int roi_w, float* panel, int H,
-                                                 int W, int r, int c) {
-  constexpr int U = 10;
-  const int win = roi_h * roi_w, lane = (int)lane_id(), r0 = r - roi_h / 2, c0 = c - roi_w / 2;
-  const int step_r = 32 / roi_w, step_c = 32 - step_r * roi_w;
-  int qr = lane / roi_w, qc = lane - qr * roi_w;
-  for (int e0 = lane; e0 < win + lane; e0 += 32 * U) {
-    float v[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = e0 + 32 * u < win ? __ldg(src + e0 + 32 * u) : 0.0f;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int rr = r0 + qr, cc = c0 + qc;
-      if (e0 + 32 * u < win && rr >= 0 && rr < H && cc >= 0 && cc < W) panel[(size_t)rr * W + cc] = v[u];
-      qr += step_r;
-      qc += step_c;
-      if (qc >= roi_w) {
-        qc -= roi_w;
-        ++qr;
-      }
-    }
-  }
-}
-
-// roi: restore every in-panel ROI pixel from the stream (one warp per peak), on
-// both paths; a ROI section after the bitstream is restored by k_dec_roi_coded.
-// Inside the panel kernel the windows were one block's work per panel, each warp
-// looking at every peak of the frame in turn: 60 epix10k frames of 3,000 windows,
-// most of them on three panels, took 1,190 us there (108 us without windows), and
-// 87 us here.
-__global__ void k_dec_roi(DevParams p, Scratch s, DecArgs a) {
-  const uint32_t f = blockIdx.y;
-  if (s.status[f] != ROIBIN_OK) return;
-  const DecInfo& di = s.dec_info[f];
-  const uint8_t* base = a.in + di.base;
-  const uint16_t* pk = reinterpret_cast<const uint16_t*>(base + di.pl.off_peaks);
-  const float* roi = reinterpret_cast<const float*>(base + di.pl.off_roi);
-  const uint32_t win = (uint32_t)(di.roi_h * di.roi_w);
-  const uint32_t wpb = blockDim.x >> 5;
-  const uint32_t n_in_place = di.roi_coding == 0 ? di.pl.n_peaks : 0u;  // else k_dec_roi_coded
-  for (uint32_t k = blockIdx.x * wpb + (threadIdx.x >> 5); k < n_in_place; k += gridDim.x * wpb) {
-    const uint32_t pn = pk[3 * k], r = pk[3 * k + 1], c = pk[3 * k + 2];
-    if (pn >= p.P || r >= p.H || c >= p.W) {
-      if (lane_id() == 0) mark_corrupt(s, f);
-      continue;
-    }
-    float* panel = a.out + (size_t)f * p.frame_px + (size_t)pn * p.H * p.W;
-    if (!RB_CHECK(s, di.pl.off_roi + (uint64_t)(k + 1) * win * 4 <= di.pl.total, ROIBIN_CHECK_STREAM_READ)) continue;
-    warp_restore_roi(roi + (size_t)k * win, di.roi_h, di.roi_w, panel, (int)p.H, (int)p.W, (int)r, (int)c);
   }
 }
 
@@ -947,7 +892,7 @@ __device__ __forceinline__ uint32_t place_strip_outliers(const uint2* v, uint32_
 //   outliers in, then the output rows.  The one pass instead of three took the
 //   kernel from 185 to 108 us on 60 epix10k frames and from 650 to 617 us on 400
 //   CSPAD-like frames (5.96 TB/s of pixels written, 0.88 of the copy rate).
-// k_dec_roi then overwrites the pixels of the ROI windows.
+// k_dec_windows then overwrites the pixels of the ROI windows.
 // The 2-D prefix sum wraps modulo 2^32 in any order, so column-then-row equals
 // the row-then-column definition.
 // kSums (3-D predictor): the panel's 2-D sums go to s.dq instead of pixels;
@@ -1257,11 +1202,6 @@ __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scr
   if (bad) mark_corrupt(s, f);
 }
 
-__global__ void k_dec_finish(Scratch s, int32_t* status, uint32_t n) {
-  const uint32_t f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f < n) status[f] = s.status[f];
-}
-
 // ROI mask: u8 per pixel, 1 on every in-panel pixel of some peak's window.
 __global__ void k_roi_mask_set(DevParams p, const uint16_t* peaks, const uint32_t* npeaks, uint8_t* mask) {
   const uint32_t f = blockIdx.y;
@@ -1359,16 +1299,6 @@ cudaError_t launch_dec_upsample(const DevParams& p, const Scratch& s, const DecA
                     (reinterpret_cast<uintptr_t>(a.out) % 16) == 0;
   dim3 grid(ceil_div((uint32_t)(p.frame_px / 4 / 256), 4) + 1, a.n_frames);
   k_dec_upsample<<<grid, 256, 0, st>>>(p, s, a, vec4 ? 1 : 0);
-  return cudaGetLastError();
-}
-cudaError_t launch_dec_roi(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  // about 4,096 blocks of eight windows a round, at least 8 and at most 64 a frame
-  dim3 grid(std::max<uint32_t>(8, std::min<uint32_t>(64, 4096 / a.n_frames)), a.n_frames);
-  k_dec_roi<<<grid, 256, 0, st>>>(p, s, a);
-  return cudaGetLastError();
-}
-cudaError_t launch_dec_finish(const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  k_dec_finish<<<ceil_div(a.n_frames, 256), 256, 0, st>>>(s, a.frame_status, a.n_frames);
   return cudaGetLastError();
 }
 uint32_t dec_panel_rows(const DevParams& p) {

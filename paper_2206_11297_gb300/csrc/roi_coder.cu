@@ -21,8 +21,9 @@
 //                  counts), their offsets, the choice coded/raw, the section
 //                  head, the frame's header fields and size;
 //   k_roi_write    warp per window: the bits (or the raw floats).
-// k_dec_roi_coded is the inverse: a thread per window decodes its values and
-// writes the in-panel pixels over the decompressed background.
+// k_dec_windows is the inverse, and ends every decompression: it writes the
+// windows' in-panel pixels over the decompressed background, in place ones a warp
+// each, coded ones a thread each.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -347,14 +348,12 @@ cudaError_t launch_roi_code(const DevParams& p, const Scratch& s, const PlainArg
 // section's size, the code lengths (at most 32, a complete code or one class
 // of length 1), the window offsets (the first 0, ascending, within the
 // words), no code or bit past the window's words, and exactly its words used.
-constexpr int kDecRoiThreads = 128;
-__global__ void __launch_bounds__(kDecRoiThreads) k_dec_roi_coded(DevParams p, Scratch s, DecArgs a) {
+__device__ __noinline__ void restore_section(const DevParams& p, const Scratch& s, const DecArgs& a) {
   __shared__ uint32_t count[33], first[33], index0[33], sorted[kRoiClasses];
   __shared__ int ok;
   const uint32_t f = blockIdx.y, tid = threadIdx.x;
-  if (tid == 0) ok = s.status[f] == ROIBIN_OK && s.dec_info[f].roi_coding != 0;
+  if (tid == 0) ok = 1;
   __syncthreads();
-  if (!ok) return;
   const DecInfo& di = s.dec_info[f];
   const uint32_t n = di.pl.n_peaks, coding = di.roi_coding, W = di.roi_words;
   const uint32_t rh = (uint32_t)di.roi_h, rw = (uint32_t)di.roi_w, win = rh * rw;
@@ -481,10 +480,79 @@ __global__ void __launch_bounds__(kDecRoiThreads) k_dec_roi_coded(DevParams p, S
   if (bad) s.status[f] = ROIBIN_ERR_CORRUPT_STREAM;
 }
 
-cudaError_t launch_dec_roi_coded(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  (void)p;
-  const dim3 grid(16, a.n_frames);
-  k_dec_roi_coded<<<grid, kDecRoiThreads, 0, st>>>(p, s, a);
+// One warp writes the in-panel pixels of the roi_h x roi_w window `src`, centred
+// on (r, c), into `panel`.  Ten loads a lane are in flight before the stores, so a
+// 17 x 17 window costs one round trip; (row, column) of the lane's elements are
+// stepped, not divided.
+__device__ __forceinline__ void warp_restore_roi(const float* __restrict__ src, int roi_h, int roi_w, float* panel, int H,
+                                                 int W, int r, int c) {
+  constexpr int U = 10;
+  const int win = roi_h * roi_w, lane = (int)lane_id(), r0 = r - roi_h / 2, c0 = c - roi_w / 2;
+  const int step_r = 32 / roi_w, step_c = 32 - step_r * roi_w;
+  int qr = lane / roi_w, qc = lane - qr * roi_w;
+  for (int e0 = lane; e0 < win + lane; e0 += 32 * U) {
+    float v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = e0 + 32 * u < win ? __ldg(src + e0 + 32 * u) : 0.0f;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int rr = r0 + qr, cc = c0 + qc;
+      if (e0 + 32 * u < win && rr >= 0 && rr < H && cc >= 0 && cc < W) panel[(size_t)rr * W + cc] = v[u];
+      qr += step_r;
+      qc += step_c;
+      if (qc >= roi_w) {
+        qc -= roi_w;
+        ++qr;
+      }
+    }
+  }
+}
+
+// In-place windows, one warp each.  Inside the panel kernel they were one block's
+// work per panel, each warp looking at every peak of the frame in turn: 60 epix10k
+// frames of 3,000 windows, most of them on three panels, took 1,190 us there (108
+// us without windows), and 87 us here.
+__device__ __forceinline__ void restore_in_place(const DevParams& p, const Scratch& s, const DecArgs& a) {
+  const uint32_t f = blockIdx.y;
+  const DecInfo& di = s.dec_info[f];
+  const uint8_t* base = a.in + di.base;
+  const uint16_t* pk = reinterpret_cast<const uint16_t*>(base + di.pl.off_peaks);
+  const float* roi = reinterpret_cast<const float*>(base + di.pl.off_roi);
+  const uint32_t win = (uint32_t)(di.roi_h * di.roi_w), wpb = blockDim.x >> 5;
+  for (uint32_t k = blockIdx.x * wpb + (threadIdx.x >> 5); k < di.pl.n_peaks; k += gridDim.x * wpb) {
+    const uint32_t pn = pk[3 * k], r = pk[3 * k + 1], c = pk[3 * k + 2];
+    if (pn >= p.P || r >= p.H || c >= p.W) {
+      if (lane_id() == 0) s.status[f] = ROIBIN_ERR_CORRUPT_STREAM;
+      continue;
+    }
+    float* panel = a.out + (size_t)f * p.frame_px + (size_t)pn * p.H * p.W;
+    if (!RB_CHECK(s, di.pl.off_roi + (uint64_t)(k + 1) * win * 4 <= di.pl.total, ROIBIN_CHECK_STREAM_READ)) continue;
+    warp_restore_roi(roi + (size_t)k * win, di.roi_h, di.roi_w, panel, (int)p.H, (int)p.W, (int)r, (int)c);
+  }
+}
+
+// The end of every decompression: the ROI windows, then, by the frame's last
+// block, its status to the caller.
+constexpr int kDecWindowThreads = 256;
+__global__ void __launch_bounds__(kDecWindowThreads) k_dec_windows(DevParams p, Scratch s, DecArgs a) {
+  __shared__ int go;  // read once: other blocks of the frame may mark it corrupt
+  const uint32_t f = blockIdx.y;
+  if (threadIdx.x == 0) go = s.status[f] == ROIBIN_OK ? 1 + (s.dec_info[f].roi_coding != 0) : 0;
+  __syncthreads();
+  if (go == 1) restore_in_place(p, s, a);
+  else if (go == 2) restore_section(p, s, a);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(s.thr_count + f, 1u) == gridDim.x - 1) {
+    __threadfence();
+    a.frame_status[f] = __ldcg(s.status + f);
+  }
+}
+
+cudaError_t launch_dec_windows(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
+  // about 4,096 blocks of eight windows a round, at least 8 and at most 64 a frame
+  const dim3 grid(std::max<uint32_t>(8, std::min<uint32_t>(64, 4096 / a.n_frames)), a.n_frames);
+  k_dec_windows<<<grid, kDecWindowThreads, 0, st>>>(p, s, a);
   return cudaGetLastError();
 }
 

@@ -863,15 +863,9 @@ int roibin_compress(roibin_ctx* ctx, const float* d_frames, uint32_t n_frames, c
 
 }  // extern "C"
 namespace {
-// The end of every decompression: the ROI windows of frames whose ROI section
-// comes after the bitstream (any stream may carry one), then the statuses.
+// The end of every decompression: the ROI windows and the statuses.
 int dec_finish(roibin_ctx* ctx, const DecArgs& a, cudaStream_t st) {
-  cudaError_t e;
-  if ((e = timed(ctx, K_DEC_ROI_CODED, st, [&] { return launch_dec_roi_coded(ctx->dp, ctx->s, a, st); })) !=
-      cudaSuccess)
-    return cuda_status(e);
-  ctx->last_launches++;  // the status copy
-  return cuda_status(launch_dec_finish(ctx->s, a, st));
+  return cuda_status(timed(ctx, K_DEC_ROI, st, [&] { return launch_dec_windows(ctx->dp, ctx->s, a, st); }));
 }
 }  // namespace
 extern "C" {
@@ -895,7 +889,6 @@ int roibin_decompress(roibin_ctx* ctx, const uint8_t* d_in, uint64_t in_bytes, c
     ctx->last_launches++;  // the decode step is two kernels: sparse frames, then dense ones
     if ((e = timed(ctx, K_DEC_PANEL, st, [&] { return launch_dec_panel(p, s, a, false, st); })) != cudaSuccess)
       return cuda_status(e);
-    if ((e = timed(ctx, K_DEC_ROI, st, [&] { return launch_dec_roi(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
     return dec_finish(ctx, a, st);
   }
   if (p.dims == 3 && dec_panel_rows(p)) {
@@ -918,12 +911,10 @@ int roibin_decompress(roibin_ctx* ctx, const uint8_t* d_in, uint64_t in_bytes, c
   if (p.dims == 3) {  // across the panels, straight to pixels
     if ((e = timed(ctx, K_DEC_CARRY, st, [&] { return launch_dec_stack_out(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
     if ((e = timed(ctx, K_DEC_PQ, st, [&] { return launch_dec_pq_pixels(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
-    if ((e = timed(ctx, K_DEC_ROI, st, [&] { return launch_dec_roi(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
     return dec_finish(ctx, a, st);
   }
   if ((e = timed(ctx, K_DEC_PQ, st, [&] { return launch_dec_pq(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
   if ((e = timed(ctx, K_DEC_UPSAMPLE, st, [&] { return launch_dec_upsample(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
-  if ((e = timed(ctx, K_DEC_ROI, st, [&] { return launch_dec_roi(p, s, a, st); })) != cudaSuccess) return cuda_status(e);
   return dec_finish(ctx, a, st);
 }
 
