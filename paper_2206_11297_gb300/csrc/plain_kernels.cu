@@ -7,6 +7,8 @@
 //   -> encode (a10 + a11) -> roi (a3)
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "roibin_internal.cuh"
 
 namespace roibin {
@@ -82,8 +84,9 @@ __device__ __forceinline__ void phase_a_v4(const float* __restrict__ panel, cons
       const uint32_t i = i0 + il, j0 = 2 * pr;
       float v0, v1;
       bin_pair(a[u], b[u], two[u], v0, v1);
-      const Quant q0 = prequantize(v0, p);
-      const Quant q1 = prequantize(v1, p);
+      Quant q0{}, q1{};
+      if (!prequant_fast(v0, p, q0.q)) q0 = prequantize(v0, p);
+      if (!prequant_fast(v1, p, q1.q)) q1 = prequantize(v1, p);
       *reinterpret_cast<int2*>(qrow0 + (size_t)il * p.Wb + j0) = make_int2(q0.q, q1.q);
       if (kOwn) {
         pqf[(size_t)il * p.Wb + j0] = q0.outlier;
@@ -103,6 +106,73 @@ __device__ __forceinline__ void phase_a_v4(const float* __restrict__ panel, cons
               const uint32_t slot = atomicAdd(s.thr_count + f, 1u);
               if (slot < p.thr_cap)
                 s.thr_idx[(size_t)f * p.thr_cap + slot] = (pn * p.H + r) * p.W + col;
+            }
+          }
+        }
+      }
+    }
+  }
+}
+
+// phase A for 2x2 bins of rows that no float4 fits (cols % 4 != 0): item = one bin,
+// four bins a thread with all sixteen loads in flight before any is used.  What
+// bounds it is the latency of the loads and their two-float stride.  24 frames of
+// 7 x 255 x 301: k_stream 70 -> 32 us, a bin at a time with a division and a
+// ballot and match per bin before.
+template <bool kOwn>
+__device__ __forceinline__ void phase_a_22(const float* __restrict__ panel, const DevParams& p, uint32_t i0, uint32_t rows,
+                                           int32_t* qrow0, uint8_t* pqf, Scratch& s, uint32_t f, uint32_t pn) {
+  const uint32_t items = rows * p.Wb;
+  constexpr int U = 4;
+  for (uint32_t base = threadIdx.x; base < items; base += kStreamThreads * U) {
+    float x[U][4];
+    uint32_t at[U];  // bit 0: a second column, bit 1: a second row
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t it = base + u * kStreamThreads, il = it / p.Wb, j = it - il * p.Wb;
+      const uint32_t r = 2 * (i0 + il), c = 2 * j;
+      at[u] = (uint32_t)(c + 1 < p.W) | ((uint32_t)(r + 1 < p.H) << 1);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) x[u][k] = 0.0f;
+      if (it < items) {
+        const float* px = panel + (size_t)r * p.W + c;
+        x[u][0] = __ldg(px);
+        if (at[u] & 1u) x[u][1] = __ldg(px + 1);
+        if (at[u] & 2u) x[u][2] = __ldg(px + p.W);
+        if (at[u] == 3u) x[u][3] = __ldg(px + p.W + 1);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t it = base + u * kStreamThreads;
+      if (it >= items) continue;
+      const uint32_t il = it / p.Wb, j = it - il * p.Wb, i = i0 + il;
+      // the in-panel pixels in row-major order; a division by 1, 2 or 4 is the exact product
+      float sum = x[u][0];
+      if (at[u] & 1u) sum = __fadd_rn(sum, x[u][1]);
+      if (at[u] & 2u) sum = __fadd_rn(sum, x[u][2]);
+      if (at[u] == 3u) sum = __fadd_rn(sum, x[u][3]);
+      const float b = __fmul_rn(sum, at[u] == 3u ? 0.25f : at[u] ? 0.5f : 1.0f);
+      int32_t q0;
+      bool outlier = false;
+      if (!prequant_fast(b, p, q0)) {
+        const Quant q = prequantize(b, p);
+        q0 = q.q;
+        outlier = q.outlier;
+        if (kOwn && outlier) s.pq_bits[(size_t)f * p.M + (pn * p.Hb + i) * p.Wb + j] = q.outlier_bits;
+      }
+      qrow0[it] = q0;
+      if (kOwn) {
+        pqf[it] = outlier;
+        // pixels >= amax_thr for the peak finder (rare: screen with the max)
+        const float m = fmaxf(fmaxf(x[u][0], x[u][1]), fmaxf(x[u][2], x[u][3]));
+        if (m >= p.amax) {
+          for (int k = 0; k < 4; ++k) {
+            const bool in = (!(k & 1) || (at[u] & 1u)) && (!(k & 2) || (at[u] & 2u));
+            if (in && x[u][k] >= p.amax) {
+              const uint32_t slot = atomicAdd(s.thr_count + f, 1u);
+              if (slot < p.thr_cap)
+                s.thr_idx[(size_t)f * p.thr_cap + slot] = (pn * p.H + 2 * i + (k >> 1)) * p.W + 2 * j + (k & 1);
             }
           }
         }
@@ -147,7 +217,7 @@ __device__ __forceinline__ void phase_a_generic(const float* __restrict__ panel,
 }
 
 __global__ void __launch_bounds__(kStreamThreads) k_stream(DevParams p, Scratch s, PlainArgs a,
-                                                           int vec4) {
+                                                           int form) {
   extern __shared__ __align__(16) unsigned char dsm[];
   StreamSmem& sm = *reinterpret_cast<StreamSmem*>(dsm);
   const uint32_t RB = a.rows_per_step;
@@ -165,6 +235,15 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream(DevParams p, Scratch 
   const float* panel = a.frames + (size_t)f * p.frame_px + (size_t)pn * p.H * p.W;
   const float* prev_panel = panel - (size_t)p.H * p.W;  // read only when pn > 0
   const bool stack = p.dims == 3 && pn > 0;            // the 3-D predictor's previous panel
+  // form 2: float4s of 2x2 bins; 1: 2x2 bins of any row width; 0: any bin
+  auto phase_a = [&](auto own, const float* src, uint32_t row, uint32_t n, int32_t* q) {
+    constexpr bool kOwn = decltype(own)::value;
+    if (form == 2) phase_a_v4<kOwn>(src, p, row, n, q, pqf, s, f, pn);
+    else if (form == 1) phase_a_22<kOwn>(src, p, row, n, q, pqf, s, f, pn);
+    else phase_a_generic<kOwn>(src, p, row, n, q, pqf, s, f, pn);
+  };
+  const std::true_type own{};
+  const std::false_type halo{};
 
   for (uint32_t k = threadIdx.x; k < p.nsym; k += kStreamThreads) sm.hist[k] = 0;
   // the row above the band; for the 1-D predictor at the top of a panel, the
@@ -174,63 +253,52 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream(DevParams p, Scratch 
   } else {
     const float* src = ib == 0 ? prev_panel : panel;
     const uint32_t row = ib == 0 ? p.Hb - 1 : ib - 1;
-    if (vec4) phase_a_v4<false>(src, p, row, 1, qbuf, pqf, s, f, pn);
-    else phase_a_generic<false>(src, p, row, 1, qbuf, pqf, s, f, pn);
+    phase_a(halo, src, row, 1, qbuf);
   }
   if (stack) {
     if (ib == 0) {
       for (uint32_t j = threadIdx.x; j < p.Wb; j += kStreamThreads) qprev[j] = 0;
-    } else if (vec4) {
-      phase_a_v4<false>(prev_panel, p, ib - 1, 1, qprev, pqf, s, f, pn);
     } else {
-      phase_a_generic<false>(prev_panel, p, ib - 1, 1, qprev, pqf, s, f, pn);
+      phase_a(halo, prev_panel, ib - 1, 1, qprev);
     }
   }
   __syncthreads();
 
   uint16_t* codes = s.codes + (size_t)f * ((size_t)p.n_chunks * kChunk);
+  uint32_t zeros = 0;  // codes of the zero residual this thread saw
   for (uint32_t i0 = ib; i0 < ie; i0 += RB) {
     const uint32_t rows = min(RB, ie - i0);
-    if (vec4) phase_a_v4<true>(panel, p, i0, rows, qbuf + p.Wb, pqf, s, f, pn);
-    else phase_a_generic<true>(panel, p, i0, rows, qbuf + p.Wb, pqf, s, f, pn);
-    if (stack) {
-      if (vec4) phase_a_v4<false>(prev_panel, p, i0, rows, qprev + p.Wb, pqf, s, f, pn);
-      else phase_a_generic<false>(prev_panel, p, i0, rows, qprev + p.Wb, pqf, s, f, pn);
-    }
+    phase_a(own, panel, i0, rows, qbuf + p.Wb);
+    if (stack) phase_a(halo, prev_panel, i0, rows, qprev + p.Wb);
     __syncthreads();
-    // phase B: residuals, codes, histogram, outliers
+    // phase B: residuals, codes, histogram, outliers.  The zero residual is counted
+    // in a register, the rare others in shared memory.
     const uint32_t items = rows * p.Wb;
-    const uint32_t iters = ceil_div(items, kStreamThreads);
-    for (uint32_t t = 0; t < iters; ++t) {
-      const uint32_t it = t * kStreamThreads + threadIdx.x;
-      uint32_t code = 0xFFFFu;  // sentinel: no item
-      if (it < items) {
-        const uint32_t il = it / p.Wb, j = it - il * p.Wb;
-        const int32_t* cur = qbuf + (size_t)(il + 1) * p.Wb;
-        const int32_t* up = qbuf + (size_t)il * p.Wb;
-        const int32_t qc = cur[j], qu = up[j];
-        const int32_t ql = j > 0 ? cur[j - 1] : 0, qd = j > 0 ? up[j - 1] : 0;
-        // integer differences wrap like the oracle's int64 result cast to int32
-        int32_t delta;
-        if (p.dims == 1) {
-          delta = (int32_t)((uint32_t)qc - (uint32_t)(j > 0 ? ql : up[p.Wb - 1]));
-        } else {
-          uint32_t d = (uint32_t)qc - (uint32_t)qu - (uint32_t)ql + (uint32_t)qd;
-          if (stack) {  // minus the previous panel's 2-D difference at the same place
-            const int32_t* pc = qprev + (size_t)(il + 1) * p.Wb;
-            const int32_t* pu = qprev + (size_t)il * p.Wb;
-            d -= (uint32_t)pc[j] - (uint32_t)pu[j] - (uint32_t)(j > 0 ? pc[j - 1] : 0) +
-                 (uint32_t)(j > 0 ? pu[j - 1] : 0);
-          }
-          delta = (int32_t)d;
+    uint16_t* out = codes + (size_t)(pn * p.Hb + i0) * p.Wb;
+    for (uint32_t it = threadIdx.x; it < items; it += kStreamThreads) {
+      const uint32_t il = it / p.Wb, j = it - il * p.Wb;
+      const int32_t* cur = qbuf + p.Wb + it;
+      const int32_t* up = cur - p.Wb;
+      const int32_t qc = cur[0], qu = up[0];
+      const int32_t ql = j > 0 ? cur[-1] : 0, qd = j > 0 ? up[-1] : 0;
+      // integer differences wrap like the oracle's int64 result cast to int32
+      int32_t delta;
+      if (p.dims == 1) {
+        delta = (int32_t)((uint32_t)qc - (uint32_t)(j > 0 ? ql : qbuf[(size_t)il * p.Wb + p.Wb - 1]));
+      } else {
+        uint32_t d = (uint32_t)qc - (uint32_t)qu - (uint32_t)ql + (uint32_t)qd;
+        if (stack) {  // minus the previous panel's 2-D difference at the same place
+          const int32_t* pc = qprev + p.Wb + it;
+          const int32_t* pu = pc - p.Wb;
+          d -= (uint32_t)pc[0] - (uint32_t)pu[0] - (uint32_t)(j > 0 ? pc[-1] : 0) + (uint32_t)(j > 0 ? pu[-1] : 0);
         }
-        code = quant_code(delta, p.R);
-        const uint32_t bin = (pn * p.Hb + i0 + il) * p.Wb + j;
-        const uint32_t flag = pqf[(size_t)il * p.Wb + j] ? 0x8000u : 0u;
-        codes[bin] = (uint16_t)(code | flag);
-        if (code == 0) s.lo_delta[(size_t)f * p.M + bin] = delta;
+        delta = (int32_t)d;
       }
-      hist_add_warp(sm.hist, code, (uint32_t)p.R);
+      const uint32_t code = quant_code(delta, p.R);
+      out[it] = (uint16_t)(code | (pqf[it] ? 0x8000u : 0u));
+      if (code == 0) s.lo_delta[(size_t)f * p.M + (size_t)(pn * p.Hb + i0) * p.Wb + it] = delta;
+      if (delta == 0) ++zeros;
+      else atomicAdd(sm.hist + code, 1u);
     }
     __syncthreads();
     // the last row of this step is the row above the next one
@@ -240,6 +308,10 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream(DevParams p, Scratch 
     }
     __syncthreads();
   }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) zeros += __shfl_xor_sync(0xffffffffu, zeros, d);
+  if (lane_id() == 0 && zeros) atomicAdd(sm.hist + p.R, zeros);
+  __syncthreads();
   for (uint32_t k = threadIdx.x; k < p.nsym; k += kStreamThreads)
     if (sm.hist[k]) atomicAdd(s.hist + (size_t)f * kMaxSymbols + k, sm.hist[k]);
 }
@@ -773,13 +845,13 @@ cudaError_t launch_reset(const DevParams& p, const Scratch& s, uint32_t n, cudaS
 }
 
 cudaError_t launch_stream(const DevParams& p, const Scratch& s, const PlainArgs& a, cudaStream_t st) {
-  const bool vec4 = p.bh == 2 && p.bw == 2 && (p.W % 4) == 0 &&
-                    (reinterpret_cast<uintptr_t>(a.frames) % 16) == 0;
+  const bool two = p.bh == 2 && p.bw == 2;
+  const int form = !two ? 0 : (p.W % 4) == 0 && (reinterpret_cast<uintptr_t>(a.frames) % 16) == 0 ? 2 : 1;
   const size_t smem = stream_smem_bytes(p, a.rows_per_step);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_stream, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   dim3 grid(a.bands_per_panel * p.P, a.n_frames);
-  k_stream<<<grid, kStreamThreads, smem, st>>>(p, s, a, vec4 ? 1 : 0);
+  k_stream<<<grid, kStreamThreads, smem, st>>>(p, s, a, form);
   return cudaGetLastError();
 }
 
