@@ -81,6 +81,7 @@ __device__ __forceinline__ uint32_t* dec_list_starts(const Scratch& s, const Dev
 // lists are strictly ascending and inside the frame, and records where each
 // panel's outliers start in them.
 __global__ void __launch_bounds__(256) k_dec_parse(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   __shared__ uint32_t hdr[24], hhdr[24];
   __shared__ int ok;
   __shared__ uint64_t len_at;  // byte offset of the code lengths in the input
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(256) k_dec_parse(DevParams p, Scratch s, DecAr
 // lorenzo: scatter the Lorenzo-outlier deltas (must land on code-0 bins, in
 // strictly ascending order).
 __global__ void k_dec_lorenzo(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
   const DecInfo& di = s.dec_info[f];
@@ -265,6 +267,7 @@ __global__ void k_dec_lorenzo(DevParams p, Scratch s, DecArgs a) {
 
 // rows: inclusive prefix sum along each binned row (one warp per row).
 __global__ void k_dec_rows(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
   const uint32_t row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -283,6 +286,7 @@ __global__ void k_dec_rows(DevParams p, Scratch s, DecArgs a) {
 // cols: prefix sum down each column of a binned panel, then b^ = fl(q * 2eb)
 // (dequant), or the sums back in place for the 3-D inverse (k_dec_stack_out).
 __global__ void k_dec_cols(DevParams p, Scratch s, DecArgs a, int dequant) {
+  chain_wait();
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -310,6 +314,7 @@ __global__ void k_dec_cols(DevParams p, Scratch s, DecArgs a, int dequant) {
 // frames 226 -> 125 us.
 template <bool kVec>
 __global__ void __launch_bounds__(256) k_dec_stack_out(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, cols = kVec ? p.W / 4 : p.W;
@@ -351,6 +356,7 @@ __global__ void __launch_bounds__(256) k_dec_stack_out(DevParams p, Scratch s, D
 // The prequantisation outliers' pixels, over those of k_dec_stack_out (the lists
 // were checked by the parse step).
 __global__ void k_dec_pq_pixels(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
   const DecInfo& di = s.dec_info[f];
@@ -371,6 +377,7 @@ __global__ void k_dec_pq_pixels(DevParams p, Scratch s, DecArgs a) {
 // walks the rows in tiles of blockDim.x, scanning the tile's row totals.
 constexpr uint32_t kChainThreads = 1024;
 __global__ void __launch_bounds__(kChainThreads) k_dec_chain(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   __shared__ uint32_t carry[kChainThreads];
   __shared__ uint32_t warp_sum[kChainThreads / 32];
   const uint32_t f = blockIdx.x;
@@ -408,6 +415,7 @@ __global__ void __launch_bounds__(kChainThreads) k_dec_chain(DevParams p, Scratc
 
 // pq: prequantisation outliers overwrite b^ with their stored bits.
 __global__ void k_dec_pq(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
   const DecInfo& di = s.dec_info[f];
@@ -426,6 +434,7 @@ __global__ void k_dec_pq(DevParams p, Scratch s, DecArgs a) {
 
 // upsample: every pixel takes its bin's value.
 __global__ void k_dec_upsample(DevParams p, Scratch s, DecArgs a, int vec4) {
+  chain_wait();
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
   const float* bh = s.bhat + (size_t)f * p.M;
@@ -599,6 +608,7 @@ __device__ __forceinline__ bool dec_load_tables(const Scratch& s, uint32_t f, ui
 
 // Sparse frames: G = 2^lg lanes per chunk, words read through L1.
 __global__ void __launch_bounds__(kDecWarps * 32) k_dec_sparse(DevParams p, Scratch s, DecArgs a, uint32_t lg) {
+  chain_wait();
   __shared__ __align__(16) uint32_t tab[kDecTableWords];
   __shared__ int go;
   const uint32_t f = blockIdx.y, G = 1u << lg;
@@ -727,6 +737,7 @@ __device__ __forceinline__ uint32_t decode_long_fast(const uint32_t* sm, uint32_
 // bins; else the frames that are not sparse, their symbols.
 template <bool kDeltas>
 __global__ void __launch_bounds__(kDecWarps * 32, 2) k_dec_dense(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   extern __shared__ __align__(16) uint32_t dec_sm[];
   __shared__ int go;
   const uint32_t f = blockIdx.y, lane = lane_id(), warp = threadIdx.x >> 5;
@@ -917,6 +928,7 @@ __host__ __device__ inline uint32_t panel_smem_bytes(uint32_t Wb, uint32_t sb) {
 template <bool kSums>
 __global__ void __launch_bounds__(kPanelThreads, 8) k_dec_panel(DevParams p, Scratch s, DecArgs a, uint32_t sb,
                                                                 uint32_t rows, uint32_t lg_seg, int vec4) {
+  chain_wait();
   extern __shared__ __align__(16) int32_t sm[];  // carry[Wb], tile[sb][Wb], symbols, mbarrier
   __shared__ int go;
   const uint32_t pn = blockIdx.x, f = blockIdx.y;
@@ -1233,8 +1245,7 @@ __global__ void k_pack(const uint8_t* src, uint64_t stride, const uint64_t* size
 
 // ---------------------------------------------------------------------------
 cudaError_t launch_dec_parse(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  k_dec_parse<<<a.n_frames, 256, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_dec_parse, a.n_frames, 256, 0, st, p, s, a);
 }
 cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArgs& a, bool deltas, cudaStream_t st) {
   // dense blocks: one round of chunks each while that is at most two waves of 304
@@ -1246,7 +1257,7 @@ cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArg
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmem);
   if (e != cudaSuccess) return e;
   if (deltas) {
-    k_dec_dense<true><<<grid, kDecWarps * 32, kDecSmem, st>>>(p, s, a);
+    launch_chained(k_dec_dense<true>, grid, kDecWarps * 32, kDecSmem, st, p, s, a);
     return cudaGetLastError();
   }
   // lanes per chunk of a sparse frame: a whole warp while the lanes of all chunks
@@ -1254,52 +1265,44 @@ cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArg
   // / 1 lanes: 1 frame 9.5 / 14 / 22 / 54 us, 64 frames 16.5 / 16.4 / 25 / 91 us,
   // 400 frames 66 / 58 / 64 / 142 us, 1,000 frames 152 / 127 / 128 / 167 us.
   const uint32_t lg = (uint64_t)p.n_chunks * a.n_frames <= 9728 ? 5 : 4;
-  k_dec_sparse<<<dim3(ceil_div(p.n_chunks << lg, kDecWarps * 32), a.n_frames), kDecWarps * 32, 0, st>>>(p, s, a, lg);
+  launch_chained(k_dec_sparse, dim3(ceil_div(p.n_chunks << lg, kDecWarps * 32), a.n_frames), kDecWarps * 32, 0, st, p, s, a, lg);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_dec_dense<false><<<grid, kDecWarps * 32, kDecSmem, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_dec_dense<false>, grid, kDecWarps * 32, kDecSmem, st, p, s, a);
 }
 cudaError_t launch_dec_lorenzo(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   dim3 grid(64, a.n_frames);
-  k_dec_lorenzo<<<grid, 256, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_dec_lorenzo, grid, 256, 0, st, p, s, a);
 }
 cudaError_t launch_dec_rows(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   dim3 grid(ceil_div(p.P * p.Hb, 8), a.n_frames);
-  k_dec_rows<<<grid, 256, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_dec_rows, grid, 256, 0, st, p, s, a);
 }
 cudaError_t launch_dec_cols(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   dim3 grid(ceil_div(p.P * p.Wb, 128), a.n_frames);
-  k_dec_cols<<<grid, 128, 0, st>>>(p, s, a, p.dims == 2 ? 1 : 0);
-  return cudaGetLastError();
+  return launch_chained(k_dec_cols, grid, 128, 0, st, p, s, a, p.dims == 2 ? 1 : 0);
 }
 cudaError_t launch_dec_carry(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  k_dec_chain<<<a.n_frames, kChainThreads, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_dec_chain, a.n_frames, kChainThreads, 0, st, p, s, a);
 }
 cudaError_t launch_dec_stack_out(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   const bool vec = p.bh == 2 && p.bw == 2 && (p.W % 4) == 0 && (reinterpret_cast<uintptr_t>(a.out) % 16) == 0;
   const dim3 grid(ceil_div(p.Hb * (vec ? p.W / 4 : p.W), 256), a.n_frames);
-  if (vec) k_dec_stack_out<true><<<grid, 256, 0, st>>>(p, s, a);
-  else k_dec_stack_out<false><<<grid, 256, 0, st>>>(p, s, a);
+  if (vec) launch_chained(k_dec_stack_out<true>, grid, 256, 0, st, p, s, a);
+  else launch_chained(k_dec_stack_out<false>, grid, 256, 0, st, p, s, a);
   return cudaGetLastError();
 }
 cudaError_t launch_dec_pq_pixels(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
-  k_dec_pq_pixels<<<dim3(16, a.n_frames), 256, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_dec_pq_pixels, dim3(16, a.n_frames), 256, 0, st, p, s, a);
 }
 cudaError_t launch_dec_pq(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   dim3 grid(16, a.n_frames);
-  k_dec_pq<<<grid, 256, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_dec_pq, grid, 256, 0, st, p, s, a);
 }
 cudaError_t launch_dec_upsample(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   const bool vec4 = p.bh == 2 && p.bw == 2 && (p.W % 4) == 0 && (p.Wb % 2) == 0 &&
                     (reinterpret_cast<uintptr_t>(a.out) % 16) == 0;
   dim3 grid(ceil_div((uint32_t)(p.frame_px / 4 / 256), 4) + 1, a.n_frames);
-  k_dec_upsample<<<grid, 256, 0, st>>>(p, s, a, vec4 ? 1 : 0);
-  return cudaGetLastError();
+  return launch_chained(k_dec_upsample, grid, 256, 0, st, p, s, a, vec4 ? 1 : 0);
 }
 uint32_t dec_panel_rows(const DevParams& p) {
   if (p.Wb > kPanelMaxWb) return 0;
@@ -1331,8 +1334,8 @@ cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs
   uint32_t lg_seg = 5;
   while (lg_seg > 0 && (sb << lg_seg) > (uint32_t)kPanelThreads) --lg_seg;
   dim3 grid(p.P, a.n_frames, ceil_div(p.Hb, rows));
-  if (sums) k_dec_panel<true><<<grid, kPanelThreads, smem, st>>>(p, s, a, sb, rows, lg_seg, vec4 ? 1 : 0);
-  else k_dec_panel<false><<<grid, kPanelThreads, smem, st>>>(p, s, a, sb, rows, lg_seg, vec4 ? 1 : 0);
+  if (sums) launch_chained(k_dec_panel<true>, grid, kPanelThreads, smem, st, p, s, a, sb, rows, lg_seg, vec4 ? 1 : 0);
+  else launch_chained(k_dec_panel<false>, grid, kPanelThreads, smem, st, p, s, a, sb, rows, lg_seg, vec4 ? 1 : 0);
   return cudaGetLastError();
 }
 cudaError_t launch_roi_mask(const DevParams& p, const uint16_t* peaks, const uint32_t* npeaks, uint32_t n,

@@ -24,6 +24,7 @@ const char* kernel_name(int id) {
 // ---------------------------------------------------------------------------
 // reset: per-frame counters and histograms start at zero.
 __global__ void k_reset(DevParams p, Scratch s, uint32_t n) {
+  chain_wait();
   const uint32_t stride = gridDim.x * blockDim.x;
   const uint32_t t0 = blockIdx.x * blockDim.x + threadIdx.x;
   for (uint32_t i = t0; i < n * kMaxSymbols; i += stride) s.hist[i] = 0;
@@ -218,6 +219,7 @@ __device__ __forceinline__ void phase_a_generic(const float* __restrict__ panel,
 
 __global__ void __launch_bounds__(kStreamThreads) k_stream(DevParams p, Scratch s, PlainArgs a,
                                                            int form) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char dsm[];
   StreamSmem& sm = *reinterpret_cast<StreamSmem*>(dsm);
   const uint32_t RB = a.rows_per_step;
@@ -324,6 +326,7 @@ constexpr int kPeakBlocks = 16;
 constexpr int kPeakWarps = 8;
 
 __global__ void __launch_bounds__(kPeakWarps * 32) k_peaks(DevParams p, Scratch s, PlainArgs a) {
+  chain_wait();
   extern __shared__ float nb_all[];
   __shared__ uint32_t q_all[kPeakWarps * 32];  // 32 candidate slots per warp (dense frames)
   const int side = 2 * peak_reach(p) + 1;
@@ -428,6 +431,7 @@ __global__ void __launch_bounds__(kPeakWarps * 32) k_peaks(DevParams p, Scratch 
 // = (panel, row, col) order), CAPACITY past max_peaks.  User peaks: validate
 // and keep the given order.
 __global__ void __launch_bounds__(1024) k_peaks_final(DevParams p, Scratch s, PlainArgs a) {
+  chain_wait();
   extern __shared__ uint32_t keys[];  // [pow2 >= max_peaks]
   __shared__ int bad;
   const uint32_t f = blockIdx.x;
@@ -496,6 +500,7 @@ __global__ void __launch_bounds__(1024) k_peaks_final(DevParams p, Scratch s, Pl
 // them; chunk_ref[f] = f - the chunk's first coded frame, which alone keeps
 // the code lengths in its stream.
 __global__ void __launch_bounds__(1024) k_huffman(DevParams p, Scratch s, uint32_t n_frames) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char dsm[];
   HuffSmem& h = *reinterpret_cast<HuffSmem*>(dsm);
   uint32_t* hsum = reinterpret_cast<uint32_t*>(dsm + align16(sizeof(HuffSmem)));  // [kMaxSymbols]
@@ -548,6 +553,7 @@ __global__ void __launch_bounds__(1024) k_huffman(DevParams p, Scratch s, uint32
 // chunks: bits, Lorenzo outliers and prequantisation outliers per chunk.
 constexpr int kChunkThreads = 128;  // 32 symbols per thread
 __global__ void __launch_bounds__(kChunkThreads) k_chunks(DevParams p, Scratch s) {
+  chain_wait();
   __shared__ uint8_t len[kMaxSymbols];
   __shared__ uint32_t red[3][kChunkThreads / 32];
   const uint32_t k = blockIdx.x, f = blockIdx.y;
@@ -608,6 +614,7 @@ __device__ inline void zero_bytes(uint8_t* base, uint64_t from, uint64_t to) {
 }
 
 __global__ void __launch_bounds__(1024) k_plan(DevParams p, Scratch s, PlainArgs a) {
+  chain_wait();
   __shared__ uint32_t tmp[33];
   __shared__ uint32_t carry[3];
   const uint32_t f = blockIdx.x;
@@ -728,6 +735,7 @@ __global__ void __launch_bounds__(1024) k_plan(DevParams p, Scratch s, PlainArgs
 // encode: one block per chunk writes its words of the bitstream and its
 // Lorenzo and prequantisation outliers, in bin order.
 __global__ void __launch_bounds__(kChunkThreads) k_encode(DevParams p, Scratch s, PlainArgs a) {
+  chain_wait();
   __shared__ uint8_t len[kMaxSymbols];
   __shared__ uint32_t cwd[kMaxSymbols];
   __shared__ uint32_t buf[kChunk];  // worst case: 4096 codes of 32 bits
@@ -800,6 +808,7 @@ __global__ void __launch_bounds__(kChunkThreads) k_encode(DevParams p, Scratch s
 // ---------------------------------------------------------------------------
 // roi: one warp per peak copies its window (fill 0 past the panel edge).
 __global__ void __launch_bounds__(256) k_roi(DevParams p, Scratch s, PlainArgs a) {
+  chain_wait();
   const uint32_t f = blockIdx.y;
   if (s.status[f] != ROIBIN_OK) return;
   const FramePlan& pl = s.plan[f];
@@ -840,8 +849,7 @@ static size_t stream_smem_bytes(const DevParams& p, uint32_t rows_per_step) {
 
 cudaError_t launch_reset(const DevParams& p, const Scratch& s, uint32_t n, cudaStream_t st) {
   const uint32_t blocks = min(1024u, ceil_div(n * kMaxSymbols, 256));
-  k_reset<<<blocks, 256, 0, st>>>(p, s, n);
-  return cudaGetLastError();
+  return launch_chained(k_reset, blocks, 256, 0, st, p, s, n);
 }
 
 cudaError_t launch_stream(const DevParams& p, const Scratch& s, const PlainArgs& a, cudaStream_t st) {
@@ -851,8 +859,7 @@ cudaError_t launch_stream(const DevParams& p, const Scratch& s, const PlainArgs&
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_stream, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   dim3 grid(a.bands_per_panel * p.P, a.n_frames);
-  k_stream<<<grid, kStreamThreads, smem, st>>>(p, s, a, form);
-  return cudaGetLastError();
+  return launch_chained(k_stream, grid, kStreamThreads, smem, st, p, s, a, form);
 }
 
 cudaError_t launch_peaks(const DevParams& p, const Scratch& s, const PlainArgs& a, cudaStream_t st) {
@@ -860,8 +867,7 @@ cudaError_t launch_peaks(const DevParams& p, const Scratch& s, const PlainArgs& 
   const int side = 2 * peak_reach(p) + 1;
   const size_t smem = (size_t)kPeakWarps * side * side * sizeof(float);
   dim3 grid(kPeakBlocks, a.n_frames);
-  k_peaks<<<grid, kPeakWarps * 32, smem, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_peaks, grid, kPeakWarps * 32, smem, st, p, s, a);
 }
 
 cudaError_t launch_peaks_final(const DevParams& p, const Scratch& s, const PlainArgs& a, cudaStream_t st) {
@@ -870,8 +876,7 @@ cudaError_t launch_peaks_final(const DevParams& p, const Scratch& s, const Plain
   const size_t smem = (size_t)n2 * 4;
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_peaks_final, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_peaks_final<<<a.n_frames, 1024, smem, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_peaks_final, a.n_frames, 1024, smem, st, p, s, a);
 }
 
 cudaError_t launch_huffman(const DevParams& p, const Scratch& s, uint32_t n, cudaStream_t st) {
@@ -881,32 +886,27 @@ cudaError_t launch_huffman(const DevParams& p, const Scratch& s, uint32_t n, cud
                          (int)(align16(sizeof(HuffSmem)) + kMaxSymbols * 4));
     attr_set = true;
   }
-  k_huffman<<<ceil_div(n, p.chunk), 1024, align16(sizeof(HuffSmem)) + kMaxSymbols * 4, st>>>(p, s, n);
-  return cudaGetLastError();
+  return launch_chained(k_huffman, ceil_div(n, p.chunk), 1024, align16(sizeof(HuffSmem)) + kMaxSymbols * 4, st, p, s, n);
 }
 
 cudaError_t launch_chunks(const DevParams& p, const Scratch& s, uint32_t n, cudaStream_t st) {
   dim3 grid(p.n_chunks, n);
-  k_chunks<<<grid, kChunkThreads, 0, st>>>(p, s);
-  return cudaGetLastError();
+  return launch_chained(k_chunks, grid, kChunkThreads, 0, st, p, s);
 }
 
 cudaError_t launch_plan(const DevParams& p, const Scratch& s, const PlainArgs& a, cudaStream_t st) {
-  k_plan<<<a.n_frames, 1024, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_plan, a.n_frames, 1024, 0, st, p, s, a);
 }
 
 cudaError_t launch_encode(const DevParams& p, const Scratch& s, const PlainArgs& a, cudaStream_t st) {
   dim3 grid(p.n_chunks, a.n_frames);
-  k_encode<<<grid, kChunkThreads, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_encode, grid, kChunkThreads, 0, st, p, s, a);
 }
 
 cudaError_t launch_roi(const DevParams& p, const Scratch& s, const PlainArgs& a, cudaStream_t st) {
   if (p.max_peaks == 0) return cudaSuccess;
   dim3 grid(ceil_div(p.max_peaks, 8), a.n_frames);
-  k_roi<<<grid, 256, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_roi, grid, 256, 0, st, p, s, a);
 }
 
 cudaError_t launch_last_peaks(const DevParams& p, const Scratch& s, uint16_t* peaks, uint32_t* npeaks,

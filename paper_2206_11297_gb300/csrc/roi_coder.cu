@@ -111,6 +111,7 @@ __device__ __forceinline__ uint32_t roi_residual(const uint32_t* mm, int e, cons
 
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kRoiWarps * 32) k_roi_classes(DevParams p, Scratch s, PlainArgs a) {
+  chain_wait();
   extern __shared__ uint32_t roi_sm[];  // [kRoiWarps][win] staged windows
   __shared__ uint32_t bh[kRoiClasses];
   __shared__ uint32_t wc[kRoiWarps][kRoiClasses];
@@ -148,6 +149,7 @@ __global__ void __launch_bounds__(kRoiWarps * 32) k_roi_classes(DevParams p, Scr
 // ---------------------------------------------------------------------------
 constexpr int kRoiPlanThreads = 256;
 __global__ void __launch_bounds__(kRoiPlanThreads) k_roi_plan(DevParams p, Scratch s, PlainArgs a) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char plan_sm[];
   HuffSmem& hs = *reinterpret_cast<HuffSmem*>(plan_sm);
   __shared__ uint8_t len[kRoiClasses];
@@ -238,6 +240,7 @@ __global__ void __launch_bounds__(kRoiPlanThreads) k_roi_plan(DevParams p, Scrat
 __host__ __device__ inline uint32_t roi_max_words(uint32_t win) { return (win * 63u + 31u) / 32u + 1u; }
 
 __global__ void __launch_bounds__(kRoiWarps * 32) k_roi_write(DevParams p, Scratch s, PlainArgs a) {
+  chain_wait();
   // [warps][win] staged windows, then [warps][roi_max_words(win)] their words; the
   // block has as many warps (up to kRoiWarps) as leave room for both
   extern __shared__ uint32_t roi_sm[];
@@ -334,12 +337,11 @@ cudaError_t launch_roi_code(const DevParams& p, const Scratch& s, const PlainArg
   // elements stepped instead of divided (RoiStep).
   const uint32_t per_frame = std::max<uint32_t>(8, std::min<uint32_t>(128, 4096 / a.n_frames));
   const dim3 grid(std::min<uint32_t>(per_frame, ceil_div(std::max<uint32_t>(p.max_peaks, 1), kRoiWarps)), a.n_frames);
-  k_roi_classes<<<grid, kRoiWarps * 32, smem, st>>>(p, s, a);
+  launch_chained(k_roi_classes, grid, kRoiWarps * 32, smem, st, p, s, a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_roi_plan<<<a.n_frames, kRoiPlanThreads, sizeof(HuffSmem), st>>>(p, s, a);
+  launch_chained(k_roi_plan, a.n_frames, kRoiPlanThreads, sizeof(HuffSmem), st, p, s, a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_roi_write<<<grid, wwarps * 32, smem_w, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_roi_write, grid, wwarps * 32, smem_w, st, p, s, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -535,6 +537,7 @@ __device__ __forceinline__ void restore_in_place(const DevParams& p, const Scrat
 // block, its status to the caller.
 constexpr int kDecWindowThreads = 256;
 __global__ void __launch_bounds__(kDecWindowThreads) k_dec_windows(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   __shared__ int go;  // read once: other blocks of the frame may mark it corrupt
   const uint32_t f = blockIdx.y;
   if (threadIdx.x == 0) go = s.status[f] == ROIBIN_OK ? 1 + (s.dec_info[f].roi_coding != 0) : 0;
@@ -552,8 +555,7 @@ __global__ void __launch_bounds__(kDecWindowThreads) k_dec_windows(DevParams p, 
 cudaError_t launch_dec_windows(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   // about 4,096 blocks of eight windows a round, at least 8 and at most 64 a frame
   const dim3 grid(std::max<uint32_t>(8, std::min<uint32_t>(64, 4096 / a.n_frames)), a.n_frames);
-  k_dec_windows<<<grid, kDecWindowThreads, 0, st>>>(p, s, a);
-  return cudaGetLastError();
+  return launch_chained(k_dec_windows, grid, kDecWindowThreads, 0, st, p, s, a);
 }
 
 }  // namespace roibin
