@@ -1964,6 +1964,7 @@ template <int kG, int RB, bool kBand>
 __global__ void __launch_bounds__(kPT, 4) k_fused(DevParams p, Scratch s, PlainArgs a, FusedShape sh) {
   extern __shared__ __align__(128) unsigned char sm[];
   uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
+  chain_wait();
   const SyncWords sw = sync_words(s, a.n_frames);
   const uint32_t n = a.n_frames;
   const uint64_t total = fused_tickets(sh, n);

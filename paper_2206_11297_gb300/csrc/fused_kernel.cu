@@ -29,6 +29,11 @@ namespace roibin {
 
 // ---------------------------------------------------------------------------
 // host side
+__global__ void k_sync_reset(uint32_t* words, uint32_t n) {
+  chain_wait();
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) words[i] = 0;
+}
+
 // The candidates of an item up to which they are tested a warp each (eight at a
 // time, about 5 us a round); above, they are tested a lane each, band by band
 // (about 12 us a band of rows in shared memory): the two meet near 20 candidates a
@@ -220,8 +225,10 @@ static void band_shape(const DevParams& p, const Scratch& s, uint32_t n, FusedSh
 
 cudaError_t launch_fused(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
                          bool dense, cudaStream_t st) {
-  // stage counters, ready flags and the ticket counter start at zero
-  cudaError_t e = cudaMemsetAsync(s.frame_done, 0, sizeof(uint32_t) * (kSyncWordsPerFrame * (uint64_t)a.n_frames + 1), st);
+  // stage counters, flags and the ticket counter start at zero (by a kernel, so that
+  // the persistent one is set up meanwhile: a memset would end first)
+  const uint32_t words = kSyncWordsPerFrame * a.n_frames + 1;
+  cudaError_t e = launch_chained(k_sync_reset, min(ceil_div(words, 256), 32u), 256, 0, st, s.frame_done, words);
   if (e != cudaSuccess) return e;
   FusedShape s2 = sh;
   band_shape(p, s, a.n_frames, &s2);
@@ -239,8 +246,7 @@ cudaError_t launch_fused(const DevParams& p, const Scratch& s, const PlainArgs& 
   const uint64_t tickets = fused_tickets(s2, a.n_frames);
   if (tickets + sh.n_ctas >= (1ull << 32)) return cudaErrorInvalidValue;
   const uint32_t grid = (uint32_t)(tickets < sh.n_ctas ? tickets : sh.n_ctas);
-  kern<<<grid, kPT, smem, st>>>(p, s, a, s2);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, kPT, smem, st, p, s, a, s2);
 }
 
 }  // namespace roibin

@@ -376,6 +376,7 @@ int compress_device(roibin_ctx* ctx, const float* d_frames, uint32_t n_frames, c
     if (ctx->wait_limit_set) sh.wait_limit = ctx->wait_limit;
     cudaError_t e = timed(ctx, K_FUSED, st,
                           [&] { return launch_fused(ctx->dp, ctx->s, a, sh, ctx->fused_dense_peaks, st); });
+    ctx->last_launches++;  // the sync words' reset before it
     if (e != cudaSuccess) return cuda_status(e);
     return roi_code(ctx, a, st);
   }
