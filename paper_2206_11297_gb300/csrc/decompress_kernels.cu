@@ -477,7 +477,7 @@ __global__ void k_dec_upsample(DevParams p, Scratch s, DecArgs a, int vec4) {
 // 60-frame epix10k batch has 7,920 chunks.  What bounds these is the chain of
 // window, lookup and advance per lane, three times over.  us, a thread per
 // chunk -> now: 60 epix10k frames (2.9 bits a symbol, dense) 1,460 -> 187; one
-// CSPAD-like frame (1.02 bits, sparse) 54 -> 9.5, 400 of them 90 -> 62; 40 of
+// CSPAD-like frame (1.02 bits, sparse) 54 -> 9.5, 400 of them 90 -> 52; 40 of
 // them as residuals for the multi-pass path 943 -> 66.
 //
 // Two shortcuts, as the code allows:
@@ -570,25 +570,26 @@ __device__ __forceinline__ uint32_t decode_range(const uint32_t* tab, const uint
   return n;
 }
 
-// The lanes' starts and counts of one chunk of nw words, decoded by a group of G
-// lanes (lane g of it covers the g-th of G equal ranges of bits).  Every lane of
-// the warp calls it.  `n`: codewords of the lane's range; `listed`: those not in
-// runs; `start`: the bit its first codeword starts at.
-template <class Decode>
-__device__ __forceinline__ void sync_ranges(uint32_t G, uint32_t g, uint32_t first_bit, uint32_t limit, uint32_t& start,
-                                            uint32_t& n, uint32_t& listed, Decode decode) {
-  start = first_bit;
-  uint32_t end = start;
+// The lanes' starts and counts of one chunk of nw words, decoded by a warp (lane l
+// covers bits [l nw, (l + 1) nw)).  `n`: codewords of the lane's range; `listed`: those not in
+// runs; `start`: the bit its first codeword starts at; `end`: the bit after its last.
+// `note(j, i, sym)` sees the j-th listed codeword, the range's i-th; what a lane's
+// last pass noted stands.
+template <class Decode, class Note>
+__device__ __forceinline__ void sync_ranges(uint32_t nw, uint32_t& start, uint32_t& end, uint32_t& n,
+                                            uint32_t& listed, Decode decode, Note note) {
+  const uint32_t lane = lane_id(), limit = (lane + 1) * nw;
+  start = end = lane * nw;
   listed = 0;
-  n = decode(end, limit, 0xFFFFFFFFu, [&](uint32_t, uint32_t) { ++listed; });
+  n = decode(end, limit, 0xFFFFFFFFu, [&](uint32_t i, uint32_t sym) { note(listed++, i, sym); });
   for (uint32_t round = 0; round < 32; ++round) {
-    const uint32_t left = __shfl_up_sync(0xffffffffu, end, 1, G);
-    const bool again = g > 0 && left != start;
+    const uint32_t left = __shfl_up_sync(0xffffffffu, end, 1);
+    const bool again = lane > 0 && left != start;
     if (!__any_sync(0xffffffffu, again)) break;
     if (again) {
       start = end = left;
       listed = 0;
-      n = decode(end, limit, 0xFFFFFFFFu, [&](uint32_t, uint32_t) { ++listed; });
+      n = decode(end, limit, 0xFFFFFFFFu, [&](uint32_t i, uint32_t sym) { note(listed++, i, sym); });
     }
   }
 }
@@ -606,75 +607,85 @@ __device__ __forceinline__ bool dec_load_tables(const Scratch& s, uint32_t f, ui
   return true;
 }
 
-// Sparse frames: G = 2^lg lanes per chunk, words read through L1.
-__global__ void __launch_bounds__(kDecWarps * 32) k_dec_sparse(DevParams p, Scratch s, DecArgs a, uint32_t lg) {
+// Sparse frames: a warp per chunk, words read through L1, a few chunks per warp
+// (each block loads the frame's tables once).  A lane notes the first kDecNotes
+// listed codewords of its range while it settles, so that most lanes (a CSPAD-like
+// frame's list about one in two) write their list without decoding the range again:
+// 1,000 frames 157 -> 125 us, 200 frames 43 -> 35 us.
+constexpr uint32_t kDecNotes = 8;
+__global__ void __launch_bounds__(kDecWarps * 32) k_dec_sparse(DevParams p, Scratch s, DecArgs a) {
   chain_wait();
   __shared__ __align__(16) uint32_t tab[kDecTableWords];
+  __shared__ uint32_t notes[kDecNotes * kDecWarps * 32];
   __shared__ int go;
-  const uint32_t f = blockIdx.y, G = 1u << lg;
+  const uint32_t f = blockIdx.y, lane = lane_id();
   if (!dec_load_tables(s, f, tab, &go)) return;
   const uint16_t* lut = reinterpret_cast<const uint16_t*>(tab + kDecCanonWords);
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, k = t >> lg, g = t & (G - 1);
-  if (((t & ~31u) >> lg) >= p.n_chunks) return;  // the whole warp
   const DecInfo& di = s.dec_info[f];
   const uint8_t* base = a.in + di.base;
   const uint32_t n_words = di.pl.n_words;
   const uint32_t* cidx = reinterpret_cast<const uint32_t*>(base + di.pl.off_cidx);
-  const bool live = k < p.n_chunks;
-  uint32_t w0 = 0, nw = 0, n_sym = 0;
-  bool bad = false;
-  if (live) {
-    w0 = cidx[k];
-    const uint32_t w1 = k + 1 < p.n_chunks ? cidx[k + 1] : n_words;
-    n_sym = min(p.M, k * kChunk + kChunk) - k * kChunk;
-    // a chunk of n symbols takes at most n words
-    bad = w0 > w1 || w1 > n_words || w1 - w0 > kChunk;
-    nw = bad ? 0u : w1 - w0;
-  }
-  const uint32_t* words = reinterpret_cast<const uint32_t*>(base + di.pl.off_bits) + w0;
   const uint32_t zsym = tab[102];  // the length-1 code is code 0: first in the (length, symbol) order
-  auto decode = [&](uint32_t& at, uint32_t limit, uint32_t room, auto other) {
-    return decode_range(tab, lut, at, limit, room, [&](uint32_t i) { return i < nw ? __ldg(words + i) : 0u; }, other);
-  };
-  const uint32_t share = nw << (5 - lg), limit = (g + 1) * share;
-  uint32_t start, n, listed;
-  sync_ranges(G, g, g * share, limit, start, n, listed, decode);
-  uint32_t first = n, at_list = listed;  // exclusive scans in the group
-  for (uint32_t d = 1; d < G; d <<= 1) {
-    const uint32_t x = __shfl_up_sync(0xffffffffu, first, d, G), y = __shfl_up_sync(0xffffffffu, at_list, d, G);
-    if (g >= d) {
-      first += x;
-      at_list += y;
-    }
-  }
-  if (g == G - 1 && first < n_sym) bad = true;  // the chunk's bits end too early
-  first -= n;
-  at_list -= listed;
-  uint32_t zeros = 0, wrote = 0;
-  if (live && !bad && first < n_sym && n > 0) {
-    uint32_t* list = dec_list(s, p, f, k);
-    const uint32_t room = min(n, n_sym - first);
-    uint32_t bit = start;
-    decode(bit, limit, room, [&](uint32_t i, uint32_t sym) {
-      if (sym > 0xFFFFu || at_list + wrote >= kDecSparseMax) bad = true;
-      else list[at_list + wrote] = ((first + i) << 16) | sym;
-      ++wrote;
-      zeros += sym == 0;
+  for (uint32_t k = blockIdx.x * kDecWarps + (threadIdx.x >> 5); k < p.n_chunks; k += gridDim.x * kDecWarps) {
+    const uint32_t w0 = cidx[k], w1 = k + 1 < p.n_chunks ? cidx[k + 1] : n_words;
+    const uint32_t n_sym = min(p.M, k * kChunk + kChunk) - k * kChunk;
+    // a chunk of n symbols takes at most n words
+    bool bad = w0 > w1 || w1 > n_words || w1 - w0 > kChunk;
+    const uint32_t nw = bad ? 0u : w1 - w0;
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(base + di.pl.off_bits) + w0;
+    auto decode = [&](uint32_t& at, uint32_t limit, uint32_t room, auto other) {
+      return decode_range(tab, lut, at, limit, room, [&](uint32_t i) { return i < nw ? __ldg(words + i) : 0u; }, other);
+    };
+    uint32_t start, end, n, listed;
+    uint32_t* noted = notes + threadIdx.x;  // position in the range << 16 | symbol; a range is at most 4,127 bits
+    sync_ranges(nw, start, end, n, listed, decode, [&](uint32_t j, uint32_t i, uint32_t sym) {
+      if (j < kDecNotes) noted[j * (kDecWarps * 32)] = i << 16 | (sym & 0xFFFFu);
     });
-    if (zsym == 0) zeros += room - wrote;
-    // the chunk's last symbol: its words must end with it
-    if (first + room == n_sym && (bit + 31) / 32 != nw) bad = true;
-  }
-  uint32_t any_bad = bad;
-  for (uint32_t d = 1; d < G; d <<= 1) {
-    zeros += __shfl_xor_sync(0xffffffffu, zeros, d);
-    wrote += __shfl_xor_sync(0xffffffffu, wrote, d);
-    any_bad |= __shfl_xor_sync(0xffffffffu, any_bad, d);
-  }
-  if (live && g == 0) {
-    dec_list_count(s, p, f)[k] = any_bad ? 0u : wrote;
-    if (any_bad) mark_corrupt(s, f);
-    if (zeros) atomicAdd(s.dec_zero + f, zeros);
+    uint32_t first = warp_incl_scan(n), at_list = warp_incl_scan(listed);
+    if (lane == 31 && first < n_sym) bad = true;  // the chunk's bits end too early
+    first -= n;
+    at_list -= listed;
+    uint32_t zeros = 0, wrote = 0;
+    if (!bad && first < n_sym && n > 0) {
+      uint32_t* list = dec_list(s, p, f, k);
+      const uint32_t room = min(n, n_sym - first);
+      // the noted codewords stand for the range when they are all of its listed ones, each a
+      // code, and inside the chunk: what the range holds past the chunk's end is then runs of
+      // the length-1 code, a bit each
+      bool all = listed <= kDecNotes;
+      for (uint32_t j = 0; all && j < listed; ++j) {
+        const uint32_t v = noted[j * (kDecWarps * 32)];
+        all = (v >> 16) < room && (v & 0xFFFFu) != 0xFFFFu;
+      }
+      uint32_t bit = start;
+      if (all) {
+        for (; wrote < listed; ++wrote) {
+          const uint32_t v = noted[wrote * (kDecWarps * 32)];
+          if (at_list + wrote >= kDecSparseMax) bad = true;
+          else list[at_list + wrote] = v + (first << 16);
+          zeros += (v & 0xFFFFu) == 0;
+        }
+        bit = end - (n - room);
+      } else {
+        decode(bit, (lane + 1) * nw, room, [&](uint32_t i, uint32_t sym) {
+          if (sym > 0xFFFFu || at_list + wrote >= kDecSparseMax) bad = true;
+          else list[at_list + wrote] = ((first + i) << 16) | sym;
+          ++wrote;
+          zeros += sym == 0;
+        });
+      }
+      if (zsym == 0) zeros += room - wrote;
+      // the chunk's last symbol: its words must end with it
+      if (first + room == n_sym && (bit + 31) / 32 != nw) bad = true;
+    }
+    const bool any_bad = __any_sync(0xffffffffu, bad);
+    zeros = __reduce_add_sync(0xffffffffu, zeros);
+    wrote = __reduce_add_sync(0xffffffffu, wrote);
+    if (lane == 0) {
+      dec_list_count(s, p, f)[k] = any_bad ? 0u : wrote;
+      if (any_bad) mark_corrupt(s, f);
+      if (zeros) atomicAdd(s.dec_zero + f, zeros);
+    }
   }
 }
 
@@ -806,9 +817,9 @@ __global__ void __launch_bounds__(kDecWarps * 32, 2) k_dec_dense(DevParams p, Sc
       at = pos;
       return n;
     };
-    const uint32_t limit = (lane + 1) * nw;  // lane l covers bits [l nw, (l + 1) nw)
-    uint32_t start, n, listed;
-    sync_ranges(32, lane, lane * nw, limit, start, n, listed, count_range);
+    const uint32_t limit = (lane + 1) * nw;
+    uint32_t start, end, n, listed;
+    sync_ranges(nw, start, end, n, listed, count_range, [](uint32_t, uint32_t, uint32_t) {});
     const uint32_t first = warp_incl_scan(n) - n;
     // the storing pass: this lane's codewords are symbols first .. first + n - 1
     uint32_t zeros = 0;
@@ -1260,12 +1271,13 @@ cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArg
     launch_chained(k_dec_dense<true>, grid, kDecWarps * 32, kDecSmem, st, p, s, a);
     return cudaGetLastError();
   }
-  // lanes per chunk of a sparse frame: a whole warp while the lanes of all chunks
-  // fit the GPU at once (311,296 threads), else 16.  CSPAD-like frames, 32 / 16 / 8
-  // / 1 lanes: 1 frame 9.5 / 14 / 22 / 54 us, 64 frames 16.5 / 16.4 / 25 / 91 us,
-  // 400 frames 66 / 58 / 64 / 142 us, 1,000 frames 152 / 127 / 128 / 167 us.
-  const uint32_t lg = (uint64_t)p.n_chunks * a.n_frames <= 9728 ? 5 : 4;
-  launch_chained(k_dec_sparse, dim3(ceil_div(p.n_chunks << lg, kDecWarps * 32), a.n_frames), kDecWarps * 32, 0, st, p, s, a, lg);
+  // sparse blocks: as many chunks per warp as bring them to two waves of eight blocks
+  // per SM, since each block loads the frame's tables (13 KB).  CSPAD-like frames, caches
+  // flushed, 1 / 2 / 3 / 9 chunks per warp: 16 frames 16 / 22 / 25 / 48 us, 200 frames
+  // 39 / 35 / 39 / 64 us, 400 frames 67 / 58 / 57 / 67 us, 1,000 frames 165 / 134 / 126 / 124 us
+  const uint32_t blocks = ceil_div(p.n_chunks, kDecWarps);
+  const uint32_t per = std::max<uint32_t>(1, (uint32_t)(((uint64_t)blocks * a.n_frames + 2431) / 2432));
+  launch_chained(k_dec_sparse, dim3(ceil_div(blocks, per), a.n_frames), kDecWarps * 32, 0, st, p, s, a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return launch_chained(k_dec_dense<false>, grid, kDecWarps * 32, kDecSmem, st, p, s, a);
 }

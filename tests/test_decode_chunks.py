@@ -17,6 +17,9 @@ def residuals(kind, m, rng):
         return np.zeros(m, np.int64)
     if kind == "runs":  # a length-1 code with a few others: the sparse lists
         return np.where(rng.random(m) < 0.02, rng.integers(-3, 4, m), 0)
+    if kind == "bursts":  # around and past the eight listed symbols a lane keeps of its range
+        dense = (np.arange(m) // 96) % 4 == 0
+        return np.where(rng.random(m) < np.where(dense, 0.12, 0.005), rng.integers(-3, 4, m), 0)
     if kind == "crowded":  # a length-1 code, more than 1,024 other symbols per chunk
         return np.where(rng.random(m) < 0.45, rng.integers(-2, 3, m), 0)
     if kind == "flat":  # ten bits a symbol: more words than the stage holds
@@ -34,7 +37,7 @@ def residuals(kind, m, rng):
     raise ValueError(kind)
 
 
-@pytest.mark.parametrize("kind", ["one", "runs", "crowded", "flat", "fib", "outliers"])
+@pytest.mark.parametrize("kind", ["one", "runs", "bursts", "crowded", "flat", "fib", "outliers"])
 @pytest.mark.parametrize("panels,width", [(1, 1), (1, 33), (3, 1365), (1, 4096), (2, 2049), (5, 4093)])
 def test_chunk_decoder(kind, panels, width):
     rng = np.random.default_rng([len(kind), panels, width])
