@@ -140,9 +140,9 @@ typedef struct {
  *     2: each panel on its own, the 2-D predictor (default);
  *     3: the panels as a volume, the 3-D predictor (seven neighbours in the
  *        previous panel, row and column);
- *   neighbours outside the array count as 0.  Only 2 runs on the fused path
- *   and on the PANEL decompression path; 1 and 3 take the plain path and the
- *   multi-pass decompression path.
+ *   neighbours outside the array count as 0.  1 takes the plain path, 2 and 3
+ *   the plain or the fused one; only 2 runs on the PANEL decompression path
+ *   (the multi-pass one takes all three).
  *   nhr_min_peaks (§1, §4, non-hit rejection): frames whose peak list (found
  *   or given) has fewer entries are not compressed; their status is
  *   ROIBIN_REJECTED and their size 0.  0 (default) keeps every frame.  A frame
@@ -275,12 +275,11 @@ int roibin_ctx_autotune(roibin_ctx* ctx, const float* d_frames, uint32_t n_frame
                         float* best_ms);
 
 /* Variant of the fused kernel for frames with many peak candidates (hot
- * pixels).  Its warp tests first try an exact rejection screen (interval
- * bounds on the ring statistics; a candidate that could pass still gets the
- * full evaluation), and a work item whose candidates overflow its list
- * evaluates them one per lane instead of one per warp.  It pays on such frames
- * and costs a little on frames with few candidates; both variants write the
- * same bytes.  Off by default; the autotuner tries both on its best fused
+ * pixels).  Either variant tests a work item's candidates one per warp while
+ * they are few and one per lane, from bands of rows in shared memory, above
+ * that.  This one gives its CTAs all the shared memory their number per SM
+ * leaves them, for taller bands, and does not list more candidates than fit
+ * shared memory.  It pays on such frames; both variants write the same bytes.  Off by default; the autotuner tries both on its best fused
  * shape.  ROIBIN_ERR_INVALID_ARG when the context has no fused path. */
 int roibin_ctx_set_fused_dense_peaks(roibin_ctx* ctx, int on);
 /* 1 if the fused kernel's dense-peaks variant is selected, else 0. */

@@ -1271,8 +1271,8 @@ cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArg
     launch_chained(k_dec_dense<true>, grid, kDecWarps * 32, kDecSmem, st, p, s, a);
     return cudaGetLastError();
   }
-  // sparse blocks: as many chunks per warp as bring them to two waves of eight blocks
-  // per SM, since each block loads the frame's tables (13 KB).  CSPAD-like frames, caches
+  // sparse blocks: as many chunks per warp as bring them to 2,432 (six are resident per
+  // SM, 912 in all), since each block loads the frame's tables (13 KB).  CSPAD-like frames, caches
   // flushed, 1 / 2 / 3 / 9 chunks per warp: 16 frames 16 / 22 / 25 / 48 us, 200 frames
   // 39 / 35 / 39 / 64 us, 400 frames 67 / 58 / 57 / 67 us, 1,000 frames 165 / 134 / 126 / 124 us
   const uint32_t blocks = ceil_div(p.n_chunks, kDecWarps);

@@ -963,7 +963,7 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
 
 // ---------------------------------------------------------------------------
 // After its panels, a frame moves through three more stages:
-//   (1) the CTA that completes the frame's last panel gathers the peak list
+//   (1) the CTA that completes the frame's last item sorts the peak list
 //       and builds the codebook;
 //   (2) chunk-size items count the bits and outliers of groups of chunks;
 //       the last one scans, lays the frame out and writes its head;

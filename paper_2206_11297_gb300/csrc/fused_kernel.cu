@@ -13,15 +13,15 @@
 //     registers (row above) and shuffles (bin to the left) and writes one byte
 //     per bin (byte = residual + 128 for residuals in [-127, 126], 0 = Lorenzo
 //     outlier, 255 = escape whose code sits in a side array);
-//   - keeps the item's histogram, prequantisation-outlier bits and the 2x4
-//     blocks holding a pixel >= amax_thr in shared memory and flushes them to
-//     per-item and per-panel slots with plain stores;
-//   - screens the listed blocks, tests and evaluates the surviving candidates
-//     and stores its sorted peak list.
+//   - keeps the item's histogram, prequantisation outliers and the 2x4 blocks
+//     holding a pixel >= amax_thr in shared memory, adds the histogram to the
+//     frame's and writes the outliers' bits to a slot per panel and band;
+//   - prunes the listed blocks' candidates, tests and evaluates the others and adds
+//     its peaks to the frame's list (the codebook stage sorts it).
+// In small batches an item is a band of rows of its panels (band_shape).
 // The rest of a frame's work (codebook, chunk sizes, layout, bit-packing)
-// runs as later work items of the same kernel (see the stages below), so the
-// latency-bound coding of earlier frames overlaps the HBM-bound streaming of
-// later ones.  After use, a frame's code bytes are dropped from L2 without a
+// runs as later work items of the same kernel (see the stages below), after the
+// whole batch has streamed; a codebook is built by the CTA that completes its frame.  After use, a frame's code bytes are dropped from L2 without a
 // write-back.
 #include "fused_device.cuh"
 
