@@ -208,9 +208,12 @@ __device__ __forceinline__ FinView fin_view(unsigned char* sm, const FusedShape&
 }
 
 // Per-frame words, zeroed before each launch:
-//   panel_done, size_done   streaming (then stack) / size items finished;
+//   panel_done, size_done   streaming / size items finished;
 //   stage                   bit 0: the codebook is published, bit 1: the plan is,
-//                           bit 2: the frame has streamed (3-D predictor);
+//                           with the 3-D predictor bit 2: the frame has streamed,
+//                           and from bit 3 on its stack items finished, plus one
+//                           for its streaming (not counted with the streaming items:
+//                           a stack item that gives up may finish before them);
 //   fin                     the plan and the write items finished (the one that
 //                           finishes last settles the frame's status); bit 31 is
 //                           set by any item that gave up waiting (sticky: no later
@@ -220,7 +223,7 @@ __device__ __forceinline__ FinView fin_view(unsigned char* sm, const FusedShape&
 struct SyncWords {
   uint32_t *panel_done, *size_done, *stage, *fin, *chunk_done, *peak_n, *pq_n, *ticket;
 };
-constexpr uint32_t kStageCodebook = 1u, kStagePlan = 2u, kStageStreamed = 4u, kGaveUp = 1u << 31;
+constexpr uint32_t kStageCodebook = 1u, kStagePlan = 2u, kStageStreamed = 4u, kStageStack = 8u, kGaveUp = 1u << 31;
 __device__ __forceinline__ SyncWords sync_words(const Scratch& s, uint32_t n) {
   SyncWords w;
   w.panel_done = s.frame_done;
@@ -1288,22 +1291,28 @@ __device__ void stack_slice(const DevParams& p, const Scratch& s, const FusedSha
     if (total[k]) atomicAdd(s.hist_f + (size_t)f * kMaxSymbols + k, total[k]);
 }
 
-// A stack item: its slice once the frame has streamed; the one that finishes last
-// builds the frame's codebook.
+// Counts a finished stack item of frame f, or its streaming as a whole.  The CTA that
+// counts last (true in every thread) builds the codebook, however many of the stack
+// items gave up: that stage clears the frame's histogram for the next launch.
+__device__ __forceinline__ bool stack_last(const FusedShape& sh, unsigned char* sm, uint32_t f, const SyncWords& sw) {
+  uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) ctl[CTL_LAST] = atomicAdd(sw.stage + f, kStageStack) / kStageStack == sh.stack ? 1u : 0u;
+  __syncthreads();
+  if (!ctl[CTL_LAST]) return false;
+  __threadfence();
+  return true;
+}
+
+// A stack item: its slice once the frame has streamed.
 __device__ void stack_item(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
                            unsigned char* sm, uint32_t f, uint32_t slice, const SyncWords& sw) {
   uint32_t* ctl = reinterpret_cast<uint32_t*>(sm + sh.off_ctl);
   const bool ready = wait_flag(sw.stage + f, kStageStreamed, ctl + CTL_WAIT, sh.wait_limit);
   if (ready) stack_slice(p, s, sh, sm, f, slice);
   else if (threadIdx.x == 0) atomicOr(sw.fin + f, kGaveUp);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) ctl[CTL_LAST] = atomicAdd(sw.panel_done + f, 1u) == sh.U + sh.stack - 1 ? 1u : 0u;
-  __syncthreads();
-  if (ctl[CTL_LAST]) {
-    __threadfence();
-    frame_codebook(p, s, a, sh, sm, f, sw);
-  }
+  if (stack_last(sh, sm, f, sw)) frame_codebook(p, s, a, sh, sm, f, sw);
 }
 
 // Per-byte tables of a frame's codebook (byte = stored code byte):
@@ -1895,8 +1904,11 @@ __device__ __forceinline__ void streamed(const DevParams& p, const Scratch& s, c
   __syncthreads();
   if (!ctl[CTL_LAST]) return;
   __threadfence();
-  if (sh.stack == 0) frame_codebook(p, s, a, sh, sm, f, sw);
-  else if (threadIdx.x == 0) flag_release(sw.stage + f, kStageStreamed);
+  if (sh.stack) {
+    if (threadIdx.x == 0) flag_release(sw.stage + f, kStageStreamed);
+    if (!stack_last(sh, sm, f, sw)) return;
+  }
+  frame_codebook(p, s, a, sh, sm, f, sw);
 }
 // The item of a ticket after the streaming ones (c counted from the first of them).
 __device__ __forceinline__ void later_item(const DevParams& p, const Scratch& s, const PlainArgs& a, const FusedShape& sh,
