@@ -64,7 +64,7 @@ bool fused_jobs_plan(FusedJobs* m, const FusedShape* tuned, int num_sms, uint32_
       need = bytes > need ? bytes : need;
     }
     if (!ok) continue;
-    if (cudaFuncSetAttribute(k_fused_jobs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need) != cudaSuccess) {
+    if (allow_smem(k_fused_jobs) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -106,7 +106,7 @@ bool fused_jobs_plan(FusedJobs* m, const FusedShape* tuned, int num_sms, uint32_
 }
 
 cudaError_t launch_fused_jobs(const FusedJobs& m, uint32_t smem, uint32_t grid, cudaStream_t st) {
-  const cudaError_t e = cudaFuncSetAttribute(k_fused_jobs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(k_fused_jobs);
   if (e != cudaSuccess) return e;
   k_fused_jobs<<<grid, kPT, smem, st>>>(m);
   return cudaGetLastError();

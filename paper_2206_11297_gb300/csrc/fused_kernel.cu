@@ -119,7 +119,7 @@ static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, ui
   // the item's rows are coded.  A band's candidates are tested in parallel, one
   // per thread, so a taller band keeps more threads busy.
   const uint32_t share = 233472u / ctas_per_sm - 1024u;
-  sh.smem_dense = sh.smem > share ? sh.smem : (share < 227u * 1024u ? share : 227u * 1024u);
+  sh.smem_dense = sh.smem > share ? sh.smem : (share < kBlockSmem ? share : kBlockSmem);
   const uint32_t least = 2 * (uint32_t)peak_reach(p) + 2;
   auto rows_in = [&](uint32_t smem) {
     const uint32_t rows = (smem - sh.off_ring) / (p.W * 4);
@@ -129,7 +129,7 @@ static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, ui
   sh.band_rows_dense = rows_in(sh.smem_dense);
   set_list_max(p, &sh);
   *out = sh;
-  return sh.smem <= 227 * 1024;
+  return sh.smem <= kBlockSmem;
 }
 
 // The kernel instantiation for a shape: column groups, rows per step, row bands.
@@ -156,7 +156,7 @@ bool fused_shape_for(const DevParams& p, uint32_t ctas_per_sm, uint32_t rows_per
   }
   if (!ok) return false;
   const FusedKernel kern = fused_kernel(sh);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem) != cudaSuccess) {
+  if (allow_smem(kern) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -235,7 +235,7 @@ cudaError_t launch_fused(const DevParams& p, const Scratch& s, const PlainArgs& 
   const uint32_t smem = dense ? sh.smem_dense : sh.smem;
   s2.dense = dense ? 1u : 0u;
   const FusedKernel kern = fused_kernel(s2);
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   // Every frame streams before any is sized: streaming is bound by the bytes each
   // CTA keeps in flight, and a CTA on a coding item has none (interleaving the

@@ -883,8 +883,10 @@ cudaError_t launch_stream(const DevParams& p, const Scratch& s, const PlainArgs&
   const bool two = p.bh == 2 && p.bw == 2;
   const int form = !two ? 0 : (p.W % 4) == 0 && (reinterpret_cast<uintptr_t>(a.frames) % 16) == 0 ? 2 : 1;
   const size_t smem = stream_smem_bytes(p, a.rows_per_step);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_stream, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = allow_smem(k_stream);
+    if (e != cudaSuccess) return e;
+  }
   dim3 grid(a.bands_per_panel * p.P, a.n_frames);
   return launch_chained(k_stream, grid, kStreamThreads, smem, st, p, s, a, form);
 }
@@ -901,19 +903,14 @@ cudaError_t launch_peaks_final(const DevParams& p, const Scratch& s, const Plain
   uint32_t n2 = 1;
   while (n2 < p.max_peaks) n2 <<= 1;
   const size_t smem = (size_t)n2 * 4;
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_peaks_final, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static_assert(kMaxPeaksLimit * 4 <= 48 * 1024, "the keys fit the default shared memory");
   return launch_chained(k_peaks_final, a.n_frames, 1024, smem, st, p, s, a);
 }
 
 cudaError_t launch_huffman(const DevParams& p, const Scratch& s, uint32_t n, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_huffman, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(align16(sizeof(HuffSmem)) + kMaxSymbols * 4));
-    attr_set = true;
-  }
-  return launch_chained(k_huffman, ceil_div(n, p.chunk), 1024, align16(sizeof(HuffSmem)) + kMaxSymbols * 4, st, p, s, n);
+  constexpr uint32_t kSmem = (sizeof(HuffSmem) + 15) / 16 * 16 + kMaxSymbols * 4;
+  static_assert(kSmem <= 40 * 1024, "the scratch fits the default shared memory");
+  return launch_chained(k_huffman, ceil_div(n, p.chunk), 1024, kSmem, st, p, s, n);
 }
 
 cudaError_t launch_chunks(const DevParams& p, const Scratch& s, uint32_t n, cudaStream_t st) {

@@ -323,11 +323,11 @@ cudaError_t launch_roi_code(const DevParams& p, const Scratch& s, const PlainArg
   const size_t per_warp = ((size_t)win + roi_max_words(win)) * 4;
   const uint32_t wwarps = (uint32_t)std::min<size_t>(kRoiWarps, (220u * 1024u) / per_warp);
   const size_t smem_w = wwarps * per_warp;
-  // the shared memory each kernel needs, set per call (sizes follow the window)
-  cudaError_t e = cudaFuncSetAttribute(k_roi_classes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_roi_write, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_roi_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HuffSmem));
+  // their own shared memory: counts of a block's warps, a codebook
+  constexpr uint32_t kOwnClasses = (kRoiWarps + 1) * kRoiClasses * 4, kOwnWrite = 2 * kRoiClasses * 4;
+  static_assert(sizeof(HuffSmem) <= 40 * 1024, "the plan's scratch fits the default shared memory");
+  cudaError_t e = allow_smem(k_roi_classes, (kOwnClasses + 1023) & ~1023u);
+  if (e == cudaSuccess) e = allow_smem(k_roi_write, (kOwnWrite + 1023) & ~1023u);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(s.roi_hist, 0, sizeof(uint32_t) * kRoiClasses * a.n_frames, st);
   if (e != cudaSuccess) return e;

@@ -180,6 +180,16 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, uint32_t threads, si
   return cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 
+// Lets launches of a kernel with `fixed` bytes of its own take all the dynamic shared
+// memory a block may have.  The limit belongs to the kernel, not to a launch: set to
+// each launch's size, another host thread's call could lower it before the launch it
+// was set for, which the runtime then refused.
+constexpr uint32_t kBlockSmem = 227 * 1024;
+template <class... P>
+cudaError_t allow_smem(void (*kernel)(P...), uint32_t fixed = 0) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kBlockSmem - fixed));
+}
+
 // ---- small helpers -------------------------------------------------------
 __host__ __device__ inline uint64_t align16(uint64_t x) { return (x + 15u) & ~uint64_t(15u); }
 __host__ __device__ inline uint32_t ceil_div(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
