@@ -1264,22 +1264,19 @@ cudaError_t launch_dec_decode(const DevParams& p, const Scratch& s, const DecArg
   // tables once, and the blocks of sparse frames end at once)
   const uint32_t rounds = std::max<uint32_t>(1, (uint32_t)((uint64_t)ceil_div(p.n_chunks, kDecWarps) * a.n_frames / 608));
   const dim3 grid(ceil_div(ceil_div(p.n_chunks, kDecWarps), rounds), a.n_frames);
-  const void* kern = deltas ? (const void*)k_dec_dense<true> : (const void*)k_dec_dense<false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmem);
+  const auto dense = deltas ? k_dec_dense<true> : k_dec_dense<false>;
+  cudaError_t e = allow_smem(dense, 1024);
   if (e != cudaSuccess) return e;
-  if (deltas) {
-    launch_chained(k_dec_dense<true>, grid, kDecWarps * 32, kDecSmem, st, p, s, a);
-    return cudaGetLastError();
-  }
+  if (deltas) return launch_chained(dense, grid, kDecWarps * 32, kDecSmem, st, p, s, a);
   // sparse blocks: as many chunks per warp as bring them to 2,432 (six are resident per
   // SM, 912 in all), since each block loads the frame's tables (13 KB).  CSPAD-like frames, caches
   // flushed, 1 / 2 / 3 / 9 chunks per warp: 16 frames 16 / 22 / 25 / 48 us, 200 frames
   // 39 / 35 / 39 / 64 us, 400 frames 67 / 58 / 57 / 67 us, 1,000 frames 165 / 134 / 126 / 124 us
   const uint32_t blocks = ceil_div(p.n_chunks, kDecWarps);
   const uint32_t per = std::max<uint32_t>(1, (uint32_t)(((uint64_t)blocks * a.n_frames + 2431) / 2432));
-  launch_chained(k_dec_sparse, dim3(ceil_div(blocks, per), a.n_frames), kDecWarps * 32, 0, st, p, s, a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return launch_chained(k_dec_dense<false>, grid, kDecWarps * 32, kDecSmem, st, p, s, a);
+  e = launch_chained(k_dec_sparse, dim3(ceil_div(blocks, per), a.n_frames), kDecWarps * 32, 0, st, p, s, a);
+  if (e != cudaSuccess) return e;
+  return launch_chained(dense, grid, kDecWarps * 32, kDecSmem, st, p, s, a);
 }
 cudaError_t launch_dec_lorenzo(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   dim3 grid(64, a.n_frames);
@@ -1299,9 +1296,7 @@ cudaError_t launch_dec_carry(const DevParams& p, const Scratch& s, const DecArgs
 cudaError_t launch_dec_stack_out(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   const bool vec = p.bh == 2 && p.bw == 2 && (p.W % 4) == 0 && (reinterpret_cast<uintptr_t>(a.out) % 16) == 0;
   const dim3 grid(ceil_div(p.Hb * (vec ? p.W / 4 : p.W), 256), a.n_frames);
-  if (vec) launch_chained(k_dec_stack_out<true>, grid, 256, 0, st, p, s, a);
-  else launch_chained(k_dec_stack_out<false>, grid, 256, 0, st, p, s, a);
-  return cudaGetLastError();
+  return launch_chained(vec ? k_dec_stack_out<true> : k_dec_stack_out<false>, grid, 256, 0, st, p, s, a);
 }
 cudaError_t launch_dec_pq_pixels(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
   return launch_chained(k_dec_pq_pixels, dim3(16, a.n_frames), 256, 0, st, p, s, a);
@@ -1346,9 +1341,8 @@ cudaError_t launch_dec_panel(const DevParams& p, const Scratch& s, const DecArgs
   uint32_t lg_seg = 5;
   while (lg_seg > 0 && (sb << lg_seg) > (uint32_t)kPanelThreads) --lg_seg;
   dim3 grid(p.P, a.n_frames, ceil_div(p.Hb, rows));
-  if (sums) launch_chained(k_dec_panel<true>, grid, kPanelThreads, smem, st, p, s, a, sb, rows, lg_seg, vec4 ? 1 : 0);
-  else launch_chained(k_dec_panel<false>, grid, kPanelThreads, smem, st, p, s, a, sb, rows, lg_seg, vec4 ? 1 : 0);
-  return cudaGetLastError();
+  return launch_chained(sums ? k_dec_panel<true> : k_dec_panel<false>, grid, kPanelThreads, smem, st, p, s, a, sb, rows,
+                        lg_seg, vec4 ? 1 : 0);
 }
 cudaError_t launch_roi_mask(const DevParams& p, const uint16_t* peaks, const uint32_t* npeaks, uint32_t n,
                             uint8_t* mask, cudaStream_t st) {

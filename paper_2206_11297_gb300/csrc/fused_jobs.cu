@@ -64,10 +64,7 @@ bool fused_jobs_plan(FusedJobs* m, const FusedShape* tuned, int num_sms, uint32_
       need = bytes > need ? bytes : need;
     }
     if (!ok) continue;
-    if (allow_smem(k_fused_jobs) != cudaSuccess) {
-      cudaGetLastError();
-      continue;
-    }
+    if (allow_smem(k_fused_jobs) != cudaSuccess) continue;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused_jobs, kPT, need) != cudaSuccess ||
         per_sm < (int)ctas) {

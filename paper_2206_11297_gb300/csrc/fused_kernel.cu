@@ -156,10 +156,7 @@ bool fused_shape_for(const DevParams& p, uint32_t ctas_per_sm, uint32_t rows_per
   }
   if (!ok) return false;
   const FusedKernel kern = fused_kernel(sh);
-  if (allow_smem(kern) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
+  if (allow_smem(kern) != cudaSuccess) return false;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPT, sh.smem) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();

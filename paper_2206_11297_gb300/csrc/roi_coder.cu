@@ -329,7 +329,7 @@ cudaError_t launch_roi_code(const DevParams& p, const Scratch& s, const PlainArg
   cudaError_t e = allow_smem(k_roi_classes, (kOwnClasses + 1023) & ~1023u);
   if (e == cudaSuccess) e = allow_smem(k_roi_write, (kOwnWrite + 1023) & ~1023u);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(s.roi_hist, 0, sizeof(uint32_t) * kRoiClasses * a.n_frames, st);
+  e = reported(cudaMemsetAsync(s.roi_hist, 0, sizeof(uint32_t) * kRoiClasses * a.n_frames, st));
   if (e != cudaSuccess) return e;
   // windows are independent: about 4,096 blocks in all (several waves of the 152 SMs),
   // at least 8 and at most 128 a frame.  The three kernels on 30 epix10k frames of
@@ -337,10 +337,8 @@ cudaError_t launch_roi_code(const DevParams& p, const Scratch& s, const PlainArg
   // elements stepped instead of divided (RoiStep).
   const uint32_t per_frame = std::max<uint32_t>(8, std::min<uint32_t>(128, 4096 / a.n_frames));
   const dim3 grid(std::min<uint32_t>(per_frame, ceil_div(std::max<uint32_t>(p.max_peaks, 1), kRoiWarps)), a.n_frames);
-  launch_chained(k_roi_classes, grid, kRoiWarps * 32, smem, st, p, s, a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  launch_chained(k_roi_plan, a.n_frames, kRoiPlanThreads, sizeof(HuffSmem), st, p, s, a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_chained(k_roi_classes, grid, kRoiWarps * 32, smem, st, p, s, a)) != cudaSuccess) return e;
+  if ((e = launch_chained(k_roi_plan, a.n_frames, kRoiPlanThreads, sizeof(HuffSmem), st, p, s, a)) != cudaSuccess) return e;
   return launch_chained(k_roi_write, grid, wwarps * 32, smem_w, st, p, s, a);
 }
 

@@ -165,6 +165,13 @@ __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// The status of a runtime call, for the caller to report: a refusal also stays behind as
+// the runtime's last error, which the next check in the process (this library and
+// PyTorch share the runtime) would take for its own.
+inline cudaError_t reported(cudaError_t e) {
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, uint32_t threads, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchAttribute attr{};
@@ -177,7 +184,7 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, uint32_t threads, si
   c.stream = st;
   c.attrs = &attr;
   c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, kernel, P(args)...);
+  return reported(cudaLaunchKernelEx(&c, kernel, P(args)...));
 }
 
 // Lets launches of a kernel with `fixed` bytes of its own take all the dynamic shared
@@ -187,7 +194,8 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, uint32_t threads, si
 constexpr uint32_t kBlockSmem = 227 * 1024;
 template <class... P>
 cudaError_t allow_smem(void (*kernel)(P...), uint32_t fixed = 0) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kBlockSmem - fixed));
+  return reported(
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kBlockSmem - fixed)));
 }
 
 // ---- small helpers -------------------------------------------------------
