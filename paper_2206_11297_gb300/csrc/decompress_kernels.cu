@@ -4,7 +4,7 @@
 //   parse (header, layout, decoding tables) -> decode (chunk-parallel
 //   canonical Huffman) -> lorenzo outliers -> row prefix sums -> column prefix
 //   sums + dequantisation -> prequantisation outliers -> up-sampling -> ROI
-//   windows and status (k_dec_windows, roi_coder.cu)
+//   windows and status (k_dec_roi_coded and k_dec_windows, roi_coder.cu)
 //
 // Every index taken from the stream is bounds-checked; a failed check marks
 // the frame ROIBIN_ERR_CORRUPT_STREAM and skips the access.
@@ -914,7 +914,7 @@ __device__ __forceinline__ uint32_t place_strip_outliers(const uint2* v, uint32_
 //   outliers in, then the output rows.  The one pass instead of three took the
 //   kernel from 185 to 108 us on 60 epix10k frames and from 650 to 617 us on 400
 //   CSPAD-like frames (5.96 TB/s of pixels written, 0.88 of the copy rate).
-// k_dec_windows then overwrites the pixels of the ROI windows.
+// k_dec_roi_coded or k_dec_windows then overwrites the pixels of the ROI windows.
 // The 2-D prefix sum wraps modulo 2^32 in any order, so column-then-row equals
 // the row-then-column definition.
 // kSums (3-D predictor): the panel's 2-D sums go to s.dq instead of pixels;

@@ -18,7 +18,7 @@ const char* kernel_name(int id) {
   static const char* names[K_COUNT] = {
       "reset", "stream", "peaks", "peaks_final", "huffman", "chunks", "plan", "encode", "roi",
       "fused", "dec_parse", "dec_decode", "dec_lorenzo", "dec_rows", "dec_cols", "dec_pq",
-      "dec_upsample", "dec_roi", "dec_panel", "roi_mask", "pack", "dec_carry", "roi_code"};
+      "dec_upsample", "dec_roi", "dec_panel", "roi_mask", "pack", "dec_carry", "roi_code", "dec_roi_coded"};
   return (id >= 0 && id < K_COUNT) ? names[id] : "?";
 }
 

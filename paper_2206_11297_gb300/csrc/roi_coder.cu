@@ -21,9 +21,9 @@
 //                  counts), their offsets, the choice coded/raw, the section
 //                  head, the frame's header fields and size;
 //   k_roi_write    warp per window: the bits (or the raw floats).
-// k_dec_windows is the inverse, and ends every decompression: it writes the
-// windows' in-panel pixels over the decompressed background, in place ones a warp
-// each, coded ones a thread each.
+// The inverse writes the windows' in-panel pixels over the decompressed background:
+// k_dec_roi_coded those of a section after the bitstream, a thread each; k_dec_windows,
+// which ends every decompression, those in place, a warp each.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -348,12 +348,21 @@ cudaError_t launch_roi_code(const DevParams& p, const Scratch& s, const PlainArg
 // section's size, the code lengths (at most 32, a complete code or one class
 // of length 1), the window offsets (the first 0, ascending, within the
 // words), no code or bit past the window's words, and exactly its words used.
-__device__ __noinline__ void restore_section(const DevParams& p, const Scratch& s, const DecArgs& a) {
+// Bound by each window's chain of codewords (a thread each).  A kernel of its own: as a
+// function of k_dec_windows it was slower than the chain alone, and its blocks of 256
+// windows left few frames' windows on one multiprocessor each.  us there -> here: 33
+// frames of 200 windows 330 -> 234, 64 frames of 200 windows of noise 376 -> 227, 1,000
+// frames of 60 788 -> 367, 40 hot-pixel frames of 3,000 557 -> 441 (at the 96 registers that
+// the compiler takes by itself 228, 220, 552 and 689).
+constexpr int kDecRoiThreads = 128;
+__global__ void __launch_bounds__(kDecRoiThreads, 8) k_dec_roi_coded(DevParams p, Scratch s, DecArgs a) {
+  chain_wait();
   __shared__ uint32_t count[33], first[33], index0[33], sorted[kRoiClasses];
   __shared__ int ok;
-  const uint32_t f = blockIdx.y, tid = threadIdx.x;
-  if (tid == 0) ok = 1;
+  const uint32_t f = blockIdx.x, tid = threadIdx.x;
+  if (tid == 0) ok = s.status[f] == ROIBIN_OK && s.dec_info[f].roi_coding != 0;
   __syncthreads();
+  if (!ok) return;
   const DecInfo& di = s.dec_info[f];
   const uint32_t n = di.pl.n_peaks, coding = di.roi_coding, W = di.roi_words;
   const uint32_t rh = (uint32_t)di.roi_h, rw = (uint32_t)di.roi_w, win = rh * rw;
@@ -400,7 +409,7 @@ __device__ __noinline__ void restore_section(const DevParams& p, const Scratch& 
   const uint32_t* off = reinterpret_cast<const uint32_t*>(sec + kRoiHead);
   const uint32_t* words = reinterpret_cast<const uint32_t*>(sec + kRoiHead + align16((uint64_t)n * 4));
   bool bad = false;
-  for (uint32_t k = blockIdx.x * blockDim.x + tid; k < n; k += gridDim.x * blockDim.x) {
+  for (uint32_t k = blockIdx.y * blockDim.x + tid; k < n; k += gridDim.y * blockDim.x) {
     const uint32_t kp = pk[3 * k], r = pk[3 * k + 1], c = pk[3 * k + 2];
     if (kp >= p.P || r >= p.H || c >= p.W) {
       bad = true;
@@ -480,6 +489,14 @@ __device__ __noinline__ void restore_section(const DevParams& p, const Scratch& 
   if (bad) s.status[f] = ROIBIN_ERR_CORRUPT_STREAM;
 }
 
+cudaError_t launch_dec_roi_coded(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st) {
+  // about 1,024 blocks of 128 windows a round, at most 64 a frame, the first of every
+  // frame before the second of any: most batches have no such section, and blocks without
+  // a window only hold up those with one
+  const uint32_t per_frame = std::min<uint32_t>(64, 1024 / a.n_frames + 1);
+  return launch_chained(k_dec_roi_coded, dim3(a.n_frames, per_frame), kDecRoiThreads, 0, st, p, s, a);
+}
+
 // One warp writes the in-panel pixels of the roi_h x roi_w window `src`, centred
 // on (r, c), into `panel`.  Ten loads a lane are in flight before the stores, so a
 // 17 x 17 window costs one round trip; (row, column) of the lane's elements are
@@ -531,17 +548,16 @@ __device__ __forceinline__ void restore_in_place(const DevParams& p, const Scrat
   }
 }
 
-// The end of every decompression: the ROI windows, then, by the frame's last
+// The end of every decompression: the ROI windows in place, then, by the frame's last
 // block, its status to the caller.
 constexpr int kDecWindowThreads = 256;
 __global__ void __launch_bounds__(kDecWindowThreads) k_dec_windows(DevParams p, Scratch s, DecArgs a) {
   chain_wait();
   __shared__ int go;  // read once: other blocks of the frame may mark it corrupt
   const uint32_t f = blockIdx.y;
-  if (threadIdx.x == 0) go = s.status[f] == ROIBIN_OK ? 1 + (s.dec_info[f].roi_coding != 0) : 0;
+  if (threadIdx.x == 0) go = s.status[f] == ROIBIN_OK && s.dec_info[f].roi_coding == 0;
   __syncthreads();
-  if (go == 1) restore_in_place(p, s, a);
-  else if (go == 2) restore_section(p, s, a);
+  if (go) restore_in_place(p, s, a);
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0 && atomicAdd(s.thr_count + f, 1u) == gridDim.x - 1) {

@@ -864,8 +864,11 @@ int roibin_compress(roibin_ctx* ctx, const float* d_frames, uint32_t n_frames, c
 
 }  // extern "C"
 namespace {
-// The end of every decompression: the ROI windows and the statuses.
+// The end of every decompression: the ROI windows of frames whose ROI section
+// comes after the bitstream (any stream may carry one), those in place and the statuses.
 int dec_finish(roibin_ctx* ctx, const DecArgs& a, cudaStream_t st) {
+  const cudaError_t e = timed(ctx, K_DEC_ROI_CODED, st, [&] { return launch_dec_roi_coded(ctx->dp, ctx->s, a, st); });
+  if (e != cudaSuccess) return cuda_status(e);
   return cuda_status(timed(ctx, K_DEC_ROI, st, [&] { return launch_dec_windows(ctx->dp, ctx->s, a, st); }));
 }
 }  // namespace

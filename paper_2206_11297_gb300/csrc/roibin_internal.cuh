@@ -1042,6 +1042,7 @@ enum KernelId {
   K_PACK,
   K_DEC_CARRY,
   K_ROI_CODE,
+  K_DEC_ROI_CODED,
   K_COUNT
 };
 const char* kernel_name(int id);
@@ -1079,8 +1080,9 @@ cudaError_t launch_dec_cols(const DevParams& p, const Scratch& s, const DecArgs&
 cudaError_t launch_dec_carry(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_dec_pq(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 cudaError_t launch_dec_upsample(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
-// the ROI windows, in place or in the section after the bitstream, and the per-frame
-// statuses to the caller (ends every decompression)
+// restores the ROI windows of frames with a coded (or moved raw) ROI section
+cudaError_t launch_dec_roi_coded(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
+// the ROI windows in place, and the per-frame statuses to the caller (ends every decompression)
 cudaError_t launch_dec_windows(const DevParams& p, const Scratch& s, const DecArgs& a, cudaStream_t st);
 // the panel path: decode through the prefix table into symbols, then one block
 // per (frame, panel) rebuilds the panel strip by strip
