@@ -356,11 +356,12 @@ __global__ void __launch_bounds__(kPeakWarps * 32) k_peaks(DevParams p, Scratch 
     return;
   }
   if (count <= p.thr_cap) {
-    // more than a pixel per warp: a block's share goes through the local-maximum rule a
-    // thread each first (neighbours in the list in different warps), and the warps test
-    // what is left, about one pixel per peak.  A warp per listed pixel spent its 13 x 13
-    // neighbourhood on pixels beside a peak's maximum: 1,000 CSPAD-like frames
-    // 693 -> 486 us.  With a pixel per warp at most, the one test is the shorter way.
+    // more than a pixel per warp: a block's share is compared with the pixels around it, a
+    // thread each (neighbours in the list in different warps), and the warps test what is
+    // left, about one pixel per peak.  A warp per listed pixel spent its 13 x 13
+    // neighbourhood on pixels beside a peak's maximum: 1,000 CSPAD-like frames of 60
+    // peaks 577 -> 300 us.  The whole window a thread each, a chain of loads, took 507 us,
+    // and slowed frames of lone hot pixels: one of 2,300 of them 74 -> 87 us (76 so).
     const uint32_t share = ceil_div(count, gridDim.x), e1 = min(count, (blockIdx.x + 1) * share);
     for (uint32_t e0 = blockIdx.x * share; e0 < e1; e0 += kPeakWarps * 32) {
       if (threadIdx.x == 0) n_left = 0;
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(kPeakWarps * 32) k_peaks(DevParams p, Scratch 
         const int r = (int)(rem / p.W), c = (int)(rem - (uint32_t)r * p.W);
         const float* pan = frame + (size_t)pn * plane;
         auto px = [&](int dr, int dc) { return __ldg(pan + (size_t)(r + dr) * p.W + (c + dc)); };
-        if (is_local_max_at(px, (int)p.H, (int)p.W, r, c, p)) q_all[atomicAdd(&n_left, 1u)] = i;
+        if (!beaten_beside(px, (int)p.H, (int)p.W, r, c)) q_all[atomicAdd(&n_left, 1u)] = i;
       }
       __syncthreads();
       for (uint32_t k = threadIdx.x >> 5; k < n_left; k += kPeakWarps) test(q_all[k]);

@@ -422,6 +422,26 @@ __device__ inline bool is_local_max_at(Px px, int H, int W, int r, int c, const 
   return true;
 }
 
+// The local-maximum rule on the eight pixels around (r, c) alone: true when one of them
+// rules it out, as it does most pixels beside a peak's maximum, in any window.  The
+// loads are independent, where is_local_max_at waits for each before the next.
+template <class Px>
+__device__ __forceinline__ bool beaten_beside(Px px, int H, int W, int r, int c) {
+  const float v = px(0, 0);
+  bool beaten = false;
+#pragma unroll
+  for (int dr = -1; dr <= 1; ++dr) {
+#pragma unroll
+    for (int dc = -1; dc <= 1; ++dc) {
+      if (dr == 0 && dc == 0) continue;
+      const bool in = r + dr >= 0 && r + dr < H && c + dc >= 0 && c + dc < W;
+      const float u = in ? px(dr, dc) : v;
+      beaten |= in && !(dr < 0 || (dr == 0 && dc < 0) ? v > u : v >= u);
+    }
+  }
+  return beaten;
+}
+
 // The paper's test (rank 3, ring 5 .. 7) for one thread on pixels in shared
 // memory, `at` the candidate's, rows W apart, every pixel within 6 of it inside
 // the panel: the same operations in the same order as is_local_max_at +
