@@ -384,7 +384,10 @@ __device__ __forceinline__ void item_peaks(const DevParams& p, const Scratch& s,
     const uint32_t r = rem / p.W, c = rem - r * p.W;
     auto ld = [](const float* q) { return __ldg(q); };
     const float* pan = item_px + (size_t)pj * plane;
-    if (warp_peak_test(pan, p.H, p.W, r, c, p, nb, ld) && lane == 0) add_peak(p, a, peak_n, f, pn0 * plane + lp);
+    // frames of many candidates (the dense variant) reject most of them by the screen
+    const bool hit = dense ? warp_peak_test<true>(pan, p.H, p.W, r, c, p, nb, ld)
+                           : warp_peak_test<false>(pan, p.H, p.W, r, c, p, nb, ld);
+    if (hit && lane == 0) add_peak(p, a, peak_n, f, pn0 * plane + lp);
   };
   // a listed pixel is tested; a listed 2x4 block is screened first (a pixel
   // beaten inside its own block, which lies inside its window, by the
