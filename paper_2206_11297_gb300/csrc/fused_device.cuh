@@ -417,13 +417,16 @@ __device__ __forceinline__ void item_peaks(const DevParams& p, const Scratch& s,
       test(key + (l >> 2) * p.W + (l & 3u));
     }
   };
-  // more candidates than this: lane per candidate, band by band, where a band
-  // fits; else every pixel of the item again
-  if (cnt <= (dense ? min(kThrLocalCap, sh.list_max) : sh.list_max)) {
+  // more candidates than sh.list_max (those of the shared list that pruning leaves, and
+  // the spilled ones): lane per candidate, band by band, where a band fits; more than the
+  // lists hold: the same, or every pixel of the item again
+  const uint32_t band_rows = dense ? sh.band_rows_dense : sh.band_rows;
+  const uint32_t cnt_local = min(cnt, kThrLocalCap), spilled = cnt - cnt_local;
+  bool listed_only = cnt <= kThrLocalCap + (dense ? 0u : kThrSpill) && (band_rows == 0 || spilled <= sh.list_max);
+  if (listed_only) {
     // a listed candidate beaten by another candidate of the shared list
     // inside its window (larger, or equal and earlier in row-major order)
     // fails the local-maximum rule; the others are tested in full
-    const uint32_t cnt_local = min(cnt, kThrLocalCap);
     if (tid == 0) v.ctl[CTL_NCAND] = 0;
     // each listed pixel's (panel, row, col), decoded once, in the per-warp
     // neighbourhood buffers (unused until the tests): the pairwise pass below
@@ -484,11 +487,14 @@ __device__ __forceinline__ void item_peaks(const DevParams& p, const Scratch& s,
     }
     __syncthreads();
     const uint32_t n_cand = v.ctl[CTL_NCAND];
-    for (uint32_t e = warp; e < n_cand; e += kPW) test_listed(v.cand[e]);
-    // the spilled candidates (written before the barriers above)
-    for (uint32_t e = warp; e < cnt - cnt_local; e += kPW) test_listed(spill_at(e));
-  } else {
-    const uint32_t band_rows = dense ? sh.band_rows_dense : sh.band_rows;
+    listed_only = band_rows == 0 || n_cand + spilled <= sh.list_max;
+    if (listed_only) {
+      for (uint32_t e = warp; e < n_cand; e += kPW) test_listed(v.cand[e]);
+      // the spilled candidates (written before the barriers above)
+      for (uint32_t e = warp; e < spilled; e += kPW) test_listed(spill_at(e));
+    }
+  }
+  if (!listed_only) {
     if (band_rows) {
       dense_band_peaks(p, a, sh, peak_n, f, pn0, kp, row0, row1, band_rows);
     } else if (dense) {
