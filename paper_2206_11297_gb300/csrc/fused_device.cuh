@@ -327,6 +327,11 @@ __device__ __noinline__ void dense_band_peaks(const DevParams& p, const PlainArg
             if (rank < q0 || rank >= q0 + kBandList) continue;
             const uint32_t bit = __ffs(m) - 1, x = 4 * (base + (bit >> 2) * kPT + tid) + (bit & 3u);
             const uint32_t r = r0 + x / W, c = x % W;
+            // crowded: bright areas, most of whose pixels a neighbour beats
+            const float* px_at = band + (size_t)(r - rb0) * W + c;
+            if (total > kBandList &&
+                beaten_beside([&](int dr, int dc) { return px_at[dr * (int)W + dc]; }, (int)H, (int)W, (int)r, (int)c))
+              continue;
             const bool inner = paper && r >= 6 && r + 6 < H && c >= 6 && c + 6 < W;
             const uint32_t at = atomicAdd(ctl + CTL_CARRY0 + (inner ? 0 : 1), 1u);
             list[inner ? at : kBandList - 1 - at] = (r << 16) | c;
