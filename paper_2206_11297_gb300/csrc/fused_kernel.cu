@@ -23,6 +23,8 @@
 // runs as later work items of the same kernel (see the stages below), after the
 // whole batch has streamed; a codebook is built by the CTA that completes its frame.  After use, a frame's code bytes are dropped from L2 without a
 // write-back.
+#include <algorithm>
+
 #include "fused_device.cuh"
 
 namespace roibin {
@@ -119,7 +121,13 @@ static bool make_shape(const DevParams& p, uint32_t ctas_per_sm, uint32_t rb, ui
   // the item's rows are coded.  A band's candidates are tested in parallel, one
   // per thread, so a taller band keeps more threads busy.
   const uint32_t share = 233472u / ctas_per_sm - 1024u;
-  sh.smem_dense = sh.smem > share ? sh.smem : (share < kBlockSmem ? share : kBlockSmem);
+  // A large neighbourhood leaves such a band few rows of its own: it also takes what the
+  // warp tests' buffers and a frame's list of peaks need, at the cost of a CTA (31 x 31 and
+  // 8,192 peaks at 388 columns: 11 rows instead of 2; 100 frames with 1% of hot pixels
+  // 45.6 -> 13.0 ms).
+  const uint64_t tests = sh.off_ring + (uint64_t)kPW * sh.side * sh.side * 4 + (uint64_t)n2 * 4 + kThrLocalCap * 4;
+  const uint32_t room = (uint32_t)std::min<uint64_t>(kBlockSmem, std::max<uint64_t>(share, tests));
+  sh.smem_dense = sh.smem > room ? sh.smem : room;
   const uint32_t least = 2 * (uint32_t)peak_reach(p) + 2;
   auto rows_in = [&](uint32_t smem) {
     const uint32_t rows = (smem - sh.off_ring) / (p.W * 4);
