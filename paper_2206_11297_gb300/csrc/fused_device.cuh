@@ -422,17 +422,37 @@ __device__ __forceinline__ void item_peaks(const DevParams& p, const Scratch& s,
       test(key + (l >> 2) * p.W + (l & 3u));
     }
   };
-  // more candidates than sh.list_max (those of the shared list that pruning leaves, and
-  // the spilled ones): lane per candidate, band by band, where a band fits; more than the
-  // lists hold: the same, or every pixel of the item again
+  // more candidates than sh.list_max: lane per candidate, band by band, where a band
+  // fits; more than the lists hold: the same, or every pixel of the item again
   const uint32_t band_rows = dense ? sh.band_rows_dense : sh.band_rows;
   const uint32_t cnt_local = min(cnt, kThrLocalCap), spilled = cnt - cnt_local;
   bool listed_only = cnt <= kThrLocalCap + (dense ? 0u : kThrSpill) && (band_rows == 0 || spilled <= sh.list_max);
-  if (listed_only) {
+  const bool pairs = band_rows == 0 || cnt <= sh.list_max;
+  if (listed_only && tid == 0) v.ctl[CTL_NCAND] = 0;
+  if (listed_only && !pairs) {
+    // spots or hot pixels?  Most of what a spot lists is beaten by a pixel beside it, and
+    // hot pixels are not: what is left of the shared list, a thread each, decides.  (All
+    // pairs of 200 listed pixels, as below, took 30 us of an item.)
+    __syncthreads();
+    static_assert(kThrLocalCap == kPT, "a thread per entry of the shared list");
+    if (tid < cnt_local) {
+      const uint32_t key = v.thr[tid];
+      bool keep = true;
+      if (!(key & kBlockKey)) {
+        const uint32_t pj = key / plane, rem = key - pj * plane;
+        const int r = (int)(rem / p.W), c = (int)(rem - (uint32_t)r * p.W);
+        const float* at = item_px + key;
+        keep = v.thrv[tid] >= p.amax &&
+               !beaten_beside([&](int dr, int dc) { return __ldg(at + dr * (int)p.W + dc); }, (int)p.H, (int)p.W, r, c);
+      }
+      if (keep) v.cand[atomicAdd(v.ctl + CTL_NCAND, 1u)] = key;
+    }
+    __syncthreads();
+    listed_only = v.ctl[CTL_NCAND] + spilled <= sh.list_max;
+  } else if (listed_only) {
     // a listed candidate beaten by another candidate of the shared list
     // inside its window (larger, or equal and earlier in row-major order)
     // fails the local-maximum rule; the others are tested in full
-    if (tid == 0) v.ctl[CTL_NCAND] = 0;
     // each listed pixel's (panel, row, col), decoded once, in the per-warp
     // neighbourhood buffers (unused until the tests): the pairwise pass below
     // then compares without dividing
@@ -491,15 +511,13 @@ __device__ __forceinline__ void item_peaks(const DevParams& p, const Scratch& s,
       if (keep && lane == 0) v.cand[atomicAdd(v.ctl + CTL_NCAND, 1u)] = key;
     }
     __syncthreads();
-    const uint32_t n_cand = v.ctl[CTL_NCAND];
-    listed_only = band_rows == 0 || n_cand + spilled <= sh.list_max;
-    if (listed_only) {
-      for (uint32_t e = warp; e < n_cand; e += kPW) test_listed(v.cand[e]);
-      // the spilled candidates (written before the barriers above)
-      for (uint32_t e = warp; e < spilled; e += kPW) test_listed(spill_at(e));
-    }
   }
-  if (!listed_only) {
+  if (listed_only) {
+    const uint32_t n_cand = v.ctl[CTL_NCAND];
+    for (uint32_t e = warp; e < n_cand; e += kPW) test_listed(v.cand[e]);
+    // the spilled candidates (written before the barriers above)
+    for (uint32_t e = warp; e < spilled; e += kPW) test_listed(spill_at(e));
+  } else {
     if (band_rows) {
       dense_band_peaks(p, a, sh, peak_n, f, pn0, kp, row0, row1, band_rows);
     } else if (dense) {

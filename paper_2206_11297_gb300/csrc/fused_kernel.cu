@@ -36,10 +36,12 @@ __global__ void k_sync_reset(uint32_t* words, uint32_t n) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) words[i] = 0;
 }
 
-// The candidates of an item up to which they are tested a warp each (eight at a
-// time, about 5 us a round); above, they are tested a lane each, band by band
-// (about 12 us a band of rows in shared memory): the two meet near 20 candidates a
-// band.
+// The candidates of an item up to which they are tested a warp each (eight at a time,
+// about 5 us a round); above, they are tested a lane each, band by band (a few us a band
+// of rows in shared memory).  100 CSPAD-like frames (32 bands an item) with 0.2, 0.3 and
+// 0.4% of hot pixels, 7 / 10 / 14 / 20 candidates a band: 1,253 / 1,646 / 1,640 / 1,646 us,
+// 1,380 / 1,375 / 2,216 / 2,216 us, 1,385 / 1,477 / 1,487 / 2,712 us; with 0.15%, 7 cost
+// 1,434 us and the others 1,350 us.
 static void set_list_max(const DevParams& p, FusedShape* sh) {
   if (!sh->band_rows) {
     sh->list_max = kThrLocalCap + kThrSpill;
@@ -47,7 +49,7 @@ static void set_list_max(const DevParams& p, FusedShape* sh) {
   }
   const uint32_t own = sh->band_rows - 2 * (uint32_t)peak_reach(p);  // rows a band adds
   const uint32_t bands = sh->k * ceil_div(min(p.H, 2 * sh->band_bins), own);
-  sh->list_max = min(20u * bands, kThrLocalCap + kThrSpill);
+  sh->list_max = min(10u * bands, kThrLocalCap + kThrSpill);
 }
 
 // Shared memory a CTA of this shape needs (0 if the shape is impossible).
