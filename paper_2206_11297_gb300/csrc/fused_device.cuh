@@ -886,8 +886,8 @@ __device__ void process_item(const DevParams& p, const Scratch& s, const PlainAr
               if (b0 != (uint32_t)((d0 + 128) & 0xFF) || b1 != (uint32_t)((d1 + 128) & 0xFF))
                 st_keep_u16_if(codes + ii * p.Wb, (uint16_t)(b0 | (b1 << 8)), keep_pol, true);
             }
-            hist_add_warp(v.hist, c0 != (uint32_t)p.R ? c0 : 0xFFFFu, 0xFFFFFFFFu);
-            hist_add_warp(v.hist, c1 != (uint32_t)p.R ? c1 : 0xFFFFu, 0xFFFFFFFFu);
+            hist_add_warp(v.hist, c0 != (uint32_t)p.R ? c0 : 0xFFFFu);
+            hist_add_warp(v.hist, c1 != (uint32_t)p.R ? c1 : 0xFFFFu);
           }
         }
         cols[g].codes += RB * p.Wb;

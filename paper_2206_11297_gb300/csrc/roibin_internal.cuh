@@ -306,16 +306,13 @@ __device__ __forceinline__ void bin_pair(const float4& a, const float4& b, bool 
   b1 = __fmul_rn(s1, rc);
 }
 
-// Histogram update by a whole warp (every lane calls; code 0xFFFF = no item).
-// Lanes holding the frame's most common code (`common`, the zero residual)
-// are counted with one ballot; the others are aggregated by value.
-__device__ __forceinline__ void hist_add_warp(uint32_t* hist, uint32_t code, uint32_t common) {
-  const uint32_t mc = __ballot_sync(0xffffffffu, code == common);
-  if (mc && lane_id() == (uint32_t)(__ffs(mc) - 1)) atomicAdd(hist + common, (uint32_t)__popc(mc));
-  const bool rest = code != common && code != 0xFFFFu;
-  const uint32_t mr = __ballot_sync(0xffffffffu, rest);
-  if (rest) {
-    const uint32_t peers = __match_any_sync(mr, code);
+// Histogram update by a whole warp (every lane calls; code 0xFFFF = no item), the lanes
+// aggregated by value.
+__device__ __forceinline__ void hist_add_warp(uint32_t* hist, uint32_t code) {
+  const bool item = code != 0xFFFFu;
+  const uint32_t mi = __ballot_sync(0xffffffffu, item);
+  if (item) {
+    const uint32_t peers = __match_any_sync(mi, code);
     if ((peers & lanemask_lt()) == 0) atomicAdd(hist + code, (uint32_t)__popc(peers));
   }
 }
