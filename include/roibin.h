@@ -278,9 +278,13 @@ int roibin_ctx_autotune(roibin_ctx* ctx, const float* d_frames, uint32_t n_frame
  * pixels).  Either variant tests a work item's candidates one per warp while
  * they are few and one per lane, from bands of rows in shared memory, above
  * that.  This one gives its CTAs all the shared memory their number per SM
- * leaves them, for taller bands, and does not list more candidates than fit
- * shared memory.  It pays on such frames; both variants write the same bytes.  Off by default; the autotuner tries both on its best fused
- * shape.  ROIBIN_ERR_INVALID_ARG when the context has no fused path. */
+ * leaves them, for taller bands, does not list more candidates than fit
+ * shared memory, and tries an exact rejection screen on the listed ones
+ * (interval bounds on the ring statistics; a candidate that could pass still
+ * gets the full evaluation).  It pays on such frames and costs a little on
+ * others; both variants write the same bytes.  Off by default; the autotuner
+ * tries both on its best fused shape.  ROIBIN_ERR_INVALID_ARG when the context
+ * has no fused path. */
 int roibin_ctx_set_fused_dense_peaks(roibin_ctx* ctx, int on);
 /* 1 if the fused kernel's dense-peaks variant is selected, else 0. */
 int roibin_ctx_fused_dense_peaks(const roibin_ctx* ctx);

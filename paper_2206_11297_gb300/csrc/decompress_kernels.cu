@@ -477,8 +477,8 @@ __global__ void k_dec_upsample(DevParams p, Scratch s, DecArgs a, int vec4) {
 // 60-frame epix10k batch has 7,920 chunks.  What bounds these is the chain of
 // window, lookup and advance per lane, three times over.  us, a thread per
 // chunk -> now: 60 epix10k frames (2.9 bits a symbol, dense) 1,460 -> 187; one
-// CSPAD-like frame (1.02 bits, sparse) 54 -> 9.5, 400 of them 90 -> 52; 40 of
-// them as residuals for the multi-pass path 943 -> 66.
+// CSPAD-like frame (1.02 bits, sparse) 54 -> 9.5, 400 of them 90 -> 44 (within calls; 57
+// with caches flushed); 40 of them as residuals for the multi-pass path 943 -> 66.
 //
 // Two shortcuts, as the code allows:
 //   - When a code of length 1 exists it is the all-zero code, so a run of z zero
@@ -594,8 +594,9 @@ __device__ __forceinline__ void sync_ranges(uint32_t nw, uint32_t& start, uint32
   }
 }
 
-// Loads the frame's decoding tables; false when the frame is not sparse (or not OK).  Other blocks of the frame may mark it corrupt meanwhile, so the
-// decision is read once and shared.
+// Loads the frame's decoding tables; false when the frame is not sparse (or not OK).
+// Other blocks of the frame may mark it corrupt meanwhile, so the decision is read once
+// and shared.
 __device__ __forceinline__ bool dec_load_tables(const Scratch& s, uint32_t f, uint32_t* tab, int* go) {
   if (threadIdx.x == 0) *go = s.status[f] == ROIBIN_OK && s.dec_info[f].sparse != 0;
   __syncthreads();

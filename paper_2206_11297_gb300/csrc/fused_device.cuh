@@ -254,7 +254,9 @@ __device__ __forceinline__ void add_peak(const DevParams& p, const PlainArgs& a,
 // a lane each), the others from the back (warp_peak_test_small, a warp each; a
 // lane's test with its checks per pixel took 13 thousand cycles, and one such
 // candidate held up its whole band).  Other windows and rings run the general
-// test.  Accepted pixels go to the frame's list (add_peak).
+// test.  Where more than a list of them come at once, bright areas, those that a pixel
+// beside them beats are left out (100 frames with a bright ring 4,355 -> 2,548 us).
+// Accepted pixels go to the frame's list (add_peak).
 // The test is bound by its chain of ordered sums and by shared-memory reads of
 // scattered pixels: an SM holds about 12 warps of candidates (what fits its shared
 // memory with the halos), each issuing one instruction in 8 cycles.  100 epix10k
@@ -1920,8 +1922,9 @@ __device__ void write_item_work(const DevParams& p, const Scratch& s, const Plai
 
 // ---------------------------------------------------------------------------
 // The tickets of a launch over n frames: n U streaming items (frame by frame), the
-// stack items of the 3-D predictor, then lag frames' size items, then rounds of a frame's size items and the write
-// items of the frame lag before it, then the last lag frames' write items.
+// stack items of the 3-D predictor, then lag frames' size items, then rounds of a frame's
+// size items and the write items of the frame lag before it, then the last lag frames'
+// write items.
 __host__ __device__ inline uint64_t fused_tickets(const FusedShape& sh, uint32_t n) {
   return (uint64_t)n * (sh.U + sh.stack + 2 * sh.groups);
 }

@@ -21,8 +21,8 @@
 // In small batches an item is a band of rows of its panels (band_shape).
 // The rest of a frame's work (codebook, chunk sizes, layout, bit-packing)
 // runs as later work items of the same kernel (see the stages below), after the
-// whole batch has streamed; a codebook is built by the CTA that completes its frame.  After use, a frame's code bytes are dropped from L2 without a
-// write-back.
+// whole batch has streamed; a codebook is built by the CTA that completes its frame.
+// After use, a frame's code bytes are dropped from L2 without a write-back.
 #include <algorithm>
 
 #include "fused_device.cuh"
@@ -151,7 +151,7 @@ static FusedKernel fused_kernel(const FusedShape& sh) {
 
 bool fused_shape_for(const DevParams& p, uint32_t ctas_per_sm, uint32_t rows_per_step, uint32_t stages,
                      FusedShape* out) {
-  // the 2-D predictor, or the 3-D one (the 2-D residuals stacked by the codebook stage)
+  // the 2-D predictor, or the 3-D one (the 2-D residuals stacked by items of their own)
   if (p.dims < 2 || p.bh != 2 || p.bw != 2 || (p.W % 4) != 0 || p.W / 4 > kMaxG * kGroupCols) return false;
   if (ctas_per_sm < 1 || ctas_per_sm > 8 || stages < 1 || stages > 8) return false;
   if (rows_per_step != 0 && (rows_per_step < 2 || rows_per_step > 3)) return false;

@@ -222,8 +222,9 @@ uint64_t carve_scratch(const DevParams& d, uint32_t n, uint8_t* base, Scratch* s
   const uint64_t mask_words = ceil_div(d.Hb * d.Wb, 32) + 1;
   t.codes8 = c.take<uint8_t>((uint64_t)n * d.n_chunks * kChunk);
   // the frames' code counts, and room for the outlier slots of a launch that cuts
-  // panels into row bands (more slots than panels).  These four sizes are what a
-  // context has always held, so that a budget admits the contexts it did.
+  // panels into row bands (more slots than panels).  Launches need less: these
+  // sections keep the size of the per-item lists they replaced, so that a budget,
+  // and the static call's fixed scratch, admits and refuses what it did.
   t.hist_f = c.take<uint32_t>((uint64_t)n * kMaxSymbols);
   t.pq_mask_words = (uint64_t)n * d.P * mask_words + (uint64_t)n * (d.P - 1) * kMaxSymbols +
                     (uint64_t)n * d.P * std::max<uint32_t>(d.max_peaks, 1) + 2ull * n * d.P;
